@@ -349,6 +349,7 @@ struct ckfwi_model {
     int pool_tag = -1;              // storage mode whose layout the pool holds
     DevMem slotbase;                // codec: device word offsets of slots
     DevMem scratch;                 // codec scratch
+    int scratch_fields = 0;         // fields it serves at once: 2 (a takeshot's pair), or 1 when memory is short
     DevMem flags;                   // int error flags
     DevMem phi, partials;
     DevMem statw;                   // codec: words per compression
@@ -737,6 +738,7 @@ struct Ctx {
     std::vector<FwdArgs> ftab;      // one row per lane and step, in launch order
     std::vector<AdjArgs> atab;
     size_t fi = 0, ai = 0;          // next row
+    const CodecLane* ctab_d = nullptr;   // the lanes' codec sides
     const FwdArgs* ftab_d = nullptr;
     const AdjArgs* atab_d = nullptr;
     const int* fstart_d = nullptr;
@@ -1467,6 +1469,42 @@ CodecView field_view(const FieldGeom& f)
     return v;
 }
 
+// Fields a codec call names by index: the zero state, then the working fields
+int codec_field(const Role& r) { return r.kind == R_WORK ? 1 + r.idx : 0; }
+
+CodecLane codec_lane(ckfwi_model* m)
+{
+    CodecLane a{};
+    a.v = field_view(m->fg);
+    a.f[0] = org(m->zero, m->fg);
+    for (int i = 0; i < 3; ++i) a.f[1 + i] = org(m->work[i], m->fg);
+    a.pool = m->pool.as<uint32_t>();
+    a.cap_words = m->cap_words;
+    a.base = m->slotbase.as<long long>();
+    a.scratch = m->scratch.p;
+    a.err = m->flags.as<int>() + 1;
+    a.stat = m->statw.as<unsigned long long>();
+    return a;
+}
+
+// A codec call on every lane of the context; fields and words still to name
+CodecCall codec_call(const Ctx& cx, const RunCfg& rc, int nf)
+{
+    CodecCall c{};
+    c.one = codec_lane(cx.m);
+    c.tab = cx.batch ? cx.ctab_d : nullptr;
+    c.lanes = cx.nl();
+    c.nf = nf;
+    c.dims = cx.m->fg.dims;
+    for (int l = 0; l < c.lanes; ++l) {
+        const FieldGeom& f = cx.lane(l)->fg;
+        c.blocks = std::max(c.blocks, codec_blocks(f.dims, f.nz, f.ny, f.nx));
+    }
+    c.tol_f = rc.tol_f;
+    c.rate = rc.rate;
+    return c;
+}
+
 // a working field that holds neither the current nor the previous state
 Role pick_free(const State& s)
 {
@@ -1542,8 +1580,6 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
     const int ut_slot = rc.mode == CKFWI_STORE_BF16 ? U_BF16 : (rc.mode == CKFWI_STORE_FP16 ? U_FP16 : U_FP32);
     // codec: slotbase[0..M] are the slots' start words, [M+1..2M] the
     // start words of their second field
-    auto sbase = [&](ckfwi_model* m, int slot) { return m->slotbase.as<long long>() + slot; };
-    auto smid = [&](ckfwi_model* m, int slot) { return m->slotbase.as<long long>() + (rc.M + 1) + slot; };
     if (rc.codec && cx.issue) {
         for (int l = 0; l < NL; ++l) {
             ckfwi_model* m = cx.lane(l);
@@ -1618,30 +1654,27 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
         } else if (A.op == ACT_TAKESHOT) {
             if (rc.codec) {
                 if (cx.issue) {
-                    // a field into the pool at *from, its end written to *to
-                    auto comp = [&](ckfwi_model* m, const float* x, const long long* from, long long* to,
-                                    unsigned long long* sw) -> cudaError_t {
-                        if (rc.rate)
-                            return codec_rate_compress_dev(x, field_view(m->fg), rc.rate, m->pool.as<uint32_t>(), from,
-                                                           m->cap_words, to, m->flags.as<int>() + 1, sw, cx.st);
-                        return codec_compress_dev(x, field_view(m->fg), rc.tol_f, m->pool.as<uint32_t>(), from,
-                                                  m->cap_words, to, m->scratch.p, m->flags.as<int>() + 1, sw, cx.st);
-                    };
-                    int tok = cx.begin(PC_COMP);
-                    for (int l = 0; l < NL; ++l) {
-                        ckfwi_model* m = cx.lane(l);
-                        unsigned long long* sw = m->statw.as<unsigned long long>();
-                        CK_TRY(comp(m, cx.fptr(l, st.cur), sbase(m, A.b), smid(m, A.b), sw + ncomp));
+                    // u^s and u^{s-1} of every lane; one field at a time where a
+                    // lane's scratch serves only one
+                    int nf = 2;
+                    for (int l = 0; l < NL && !rc.rate; ++l) nf = std::min(nf, cx.lane(l)->scratch_fields);
+                    const int fld[2] = {codec_field(st.cur), codec_field(st.prev)};
+                    const int word[3] = {A.b, rc.M + 1 + A.b, A.b + 1};
+                    for (int k = 0; k < 2; k += nf) {
+                        CodecCall c = codec_call(cx, rc, nf);
+                        for (int i = 0; i < nf; ++i) {
+                            c.src[i] = fld[k + i];
+                            c.from[i] = word[k + i];
+                        }
+                        c.to = word[k + nf];
+                        c.stat0 = ncomp + k;
+                        const int tok = cx.begin(PC_COMP);
+                        cx.count[PC_COMP] += nf - 1;   // counted by field
+                        if (rc.rate) CK_TRY(codec_rate_compress_dev(c, cx.st));
+                        else CK_TRY(codec_compress_dev(c, cx.st));
+                        cx.end(tok);
+                        cx.launches += 2;   // two launches in either mode
                     }
-                    cx.end(tok);
-                    tok = cx.begin(PC_COMP);
-                    for (int l = 0; l < NL; ++l) {
-                        ckfwi_model* m = cx.lane(l);
-                        unsigned long long* sw = m->statw.as<unsigned long long>();
-                        CK_TRY(comp(m, cx.fptr(l, st.prev), smid(m, A.b), sbase(m, A.b + 1), sw + ncomp + 1));
-                    }
-                    cx.end(tok);
-                    cx.launches += 4LL * NL;   // two launches per field in either mode
                 }
                 ncomp += 2;
             }
@@ -1720,30 +1753,18 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 st = State{slot_r(A.b, 0), slot_r(A.b, 1), U_FP32, U_FP32};   // the slot is the state
             } else if (rc.codec) {
                 if (cx.issue) {
-                    auto dec = [&](ckfwi_model* m, const long long* from, float* x) -> cudaError_t {
-                        if (rc.rate)
-                            return codec_rate_decompress_dev(m->pool.as<uint32_t>(), from, m->cap_words,
-                                                             field_view(m->fg), rc.rate, x, m->flags.as<int>() + 1,
-                                                             cx.st);
-                        return codec_decompress_dev(m->pool.as<uint32_t>(), from, m->cap_words, field_view(m->fg), x,
-                                                    m->flags.as<int>() + 1, cx.st);
-                    };
-                    int tok = cx.begin(PC_DECOMP);
-                    for (int l = 0; l < NL; ++l) {
-                        ckfwi_model* m = cx.lane(l);
-                        CK_TRY(dec(m, sbase(m, A.b), cx.fptr(l, work_r(0))));
-                        ++cx.launches;
-                    }
+                    // a reverse step needs u^s only
+                    CodecCall c = codec_call(cx, rc, next_turn ? 1 : 2);
+                    c.src[0] = codec_field(work_r(0));
+                    c.src[1] = codec_field(work_r(1));
+                    c.from[0] = A.b;
+                    c.from[1] = rc.M + 1 + A.b;
+                    const int tok = cx.begin(PC_DECOMP);
+                    cx.count[PC_DECOMP] += c.nf - 1;   // counted by field
+                    if (rc.rate) CK_TRY(codec_rate_decompress_dev(c, cx.st));
+                    else CK_TRY(codec_decompress_dev(c, cx.st));
                     cx.end(tok);
-                    if (!next_turn) {   // a reverse step needs u^s only
-                        tok = cx.begin(PC_DECOMP);
-                        for (int l = 0; l < NL; ++l) {
-                            ckfwi_model* m = cx.lane(l);
-                            CK_TRY(dec(m, smid(m, A.b), cx.fptr(l, work_r(1))));
-                            ++cx.launches;
-                        }
-                        cx.end(tok);
-                    }
+                    ++cx.launches;
                 }
                 st = State{work_r(0), work_r(1), U_FP32, U_FP32};
             } else if (next_turn) {
@@ -1811,7 +1832,7 @@ double storage_bytes(const FieldGeom& f, const RunCfg& rc, const ckfwi_grad_opts
     if (!rc.codec) return nslot * field_bytes(f, 2);
     if (rc.rate) return nslot * 4.0 * (double)codec_rate_words(f.dims, f.nz, f.ny, f.nx, rc.rate);
     const double pool = o->pool_bytes ? (double)o->pool_bytes : nslot * f.npts * 4.0;
-    return pool + (double)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx);
+    return pool + (double)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx, 2);
 }
 
 int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
@@ -1890,7 +1911,17 @@ int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
         CK_TRY(m->slotbase.alloc(sizeof(long long) * (2 * (size_t)rc.M + 4)));
         // a fresh scratch is zeroed (its counter and group sums start at zero;
         // every compression of this model's fields leaves them zero)
-        if (!rc.rate) CK_TRY(m->scratch.alloc((size_t)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx), true));
+        if (!rc.rate) {
+            // both fields of a takeshot at once, one after the other when memory is short
+            m->scratch_fields = 2;
+            cudaError_t e = m->scratch.alloc((size_t)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx, 2), true);
+            if (e == cudaErrorMemoryAllocation) {
+                cudaGetLastError();
+                m->scratch_fields = 1;
+                e = m->scratch.alloc((size_t)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx, 1), true);
+            }
+            CK_TRY(e);
+        }
         CK_TRY(m->statw.alloc(sizeof(unsigned long long) * (size_t)(4 * rc.N + 8)));
     }
     return CKFWI_OK;
@@ -2418,7 +2449,10 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
         const size_t fb = ((sizeof(FwdArgs) * cx.ftab.size() + 255) / 256) * 256;
         const size_t ab = ((sizeof(AdjArgs) * cx.atab.size() + 255) / 256) * 256;
         const size_t sb = sizeof(int) * 2 * (NL + 1);
-        int rs = cuda_status_or_ok(tabs.alloc(fb + ab + sb, false));
+        std::vector<CodecLane> ctab;
+        for (int l = 0; rc.codec && l < NL; ++l) ctab.push_back(codec_lane(lanes[l]));
+        const size_t so = (sb + 255) / 256 * 256;
+        int rs = cuda_status_or_ok(tabs.alloc(fb + ab + so + sizeof(CodecLane) * ctab.size(), false));
         if (rs == CKFWI_OK && !cx.ftab.empty())
             rs = cuda_status_or_ok(cudaMemcpy(tabs.p, cx.ftab.data(), sizeof(FwdArgs) * cx.ftab.size(),
                                               cudaMemcpyHostToDevice));
@@ -2430,10 +2464,14 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
         if (rs == CKFWI_OK)
             rs = cuda_status_or_ok(
                 cudaMemcpy(tabs.as<char>() + fb + ab, starts.data(), sb, cudaMemcpyHostToDevice));
+        if (rs == CKFWI_OK && !ctab.empty())
+            rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so, ctab.data(),
+                                              sizeof(CodecLane) * ctab.size(), cudaMemcpyHostToDevice));
         if (rs != CKFWI_OK) {
             if (graph) m0->bgraphs.erase(key);
             return rs;
         }
+        cx.ctab_d = reinterpret_cast<const CodecLane*>(tabs.as<char>() + fb + ab + so);
         cx.ftab_d = tabs.as<FwdArgs>();
         cx.atab_d = reinterpret_cast<const AdjArgs*>(tabs.as<char>() + fb);
         cx.fstart_d = reinterpret_cast<const int*>(tabs.as<char>() + fb + ab);
@@ -2950,6 +2988,28 @@ namespace {
 std::mutex g_codec_mu;
 DevMem* g_codec_scratch[64] = {};
 DevMem* g_codec_scal[64] = {};
+
+// A call on one dense field: its stream in `pool` from the word in sc[0] on,
+// the end of a compressed stream to sc[1], error bits at sc[4]
+CodecCall dense_call(float* x, int dims, int nz, int ny, int nx, uint32_t* pool, long long cap, long long* sc)
+{
+    CodecCall c{};
+    CodecLane& a = c.one;
+    a.v.dims = dims; a.v.nz = nz; a.v.ny = ny; a.v.nx = nx;
+    a.v.py = nx;
+    a.v.pz = (long long)ny * nx;
+    a.v.aligned = (nx % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
+    a.f[0] = x;
+    a.pool = pool;
+    a.cap_words = cap;
+    a.base = sc;
+    a.err = reinterpret_cast<int*>(sc + 4);
+    c.lanes = c.nf = 1;
+    c.dims = dims;
+    c.to = 1;
+    c.blocks = codec_blocks(dims, nz, ny, nx);
+    return c;
+}
 }  // namespace
 
 extern "C" int ckfwi_codec_compress(const float* x, int dims, int nz, int ny, int nx, double tol, uint32_t* out,
@@ -2967,21 +3027,18 @@ extern "C" int ckfwi_codec_compress(const float* x, int dims, int nz, int ny, in
     if (!g_codec_scal[dev]) g_codec_scal[dev] = new DevMem();
     DevMem& scr = *g_codec_scratch[dev];
     DevMem& scal = *g_codec_scal[dev];
-    const size_t need = (size_t)codec_scratch_bytes(dims, nz, ny, nx);
+    const size_t need = (size_t)codec_scratch_bytes(dims, nz, ny, nx, 1);
     if (scr.bytes < need) CK_TRY(scr.alloc(need, false));
     CK_TRY(scal.alloc(64, true));
     CK_TRY(cudaMemsetAsync(scal.p, 0, 64, st));
     // the scratch serves fields of any size here: its counter and group sums
     // are cleared for this one's layout
     CK_TRY(cudaMemsetAsync(scr.p, 0, (size_t)codec_scratch_zero_bytes(dims, nz, ny, nx), st));
-    CodecView v{};
-    v.dims = dims; v.nz = nz; v.ny = ny; v.nx = nx;
-    v.py = nx;
-    v.pz = (long long)ny * nx;
-    v.aligned = (nx % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
     long long* sc = scal.as<long long>();
-    int* err = reinterpret_cast<int*>(sc + 4);
-    CK_TRY(codec_compress_dev(x, v, tol_float(tol), out, sc, cap, sc + 1, scr.p, err, nullptr, st));
+    CodecCall c = dense_call(const_cast<float*>(x), dims, nz, ny, nx, out, cap, sc);
+    c.one.scratch = scr.p;
+    c.tol_f = tol_float(tol);
+    CK_TRY(codec_compress_dev(c, st));
     long long h[5];
     CK_TRY(cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st));
     CK_TRY(cudaStreamSynchronize(st));
@@ -3015,14 +3072,10 @@ extern "C" int ckfwi_codec_compress_rate(const float* x, int dims, int nz, int n
     DevMem& scal = *g_codec_scal[dev];
     CK_TRY(scal.alloc(64, true));
     CK_TRY(cudaMemsetAsync(scal.p, 0, 64, st));
-    CodecView v{};
-    v.dims = dims; v.nz = nz; v.ny = ny; v.nx = nx;
-    v.py = nx;
-    v.pz = (long long)ny * nx;
-    v.aligned = false;
     long long* sc = scal.as<long long>();
-    int* err = reinterpret_cast<int*>(sc + 4);
-    CK_TRY(codec_rate_compress_dev(x, v, rate, out, sc, cap, sc + 1, err, nullptr, st));
+    CodecCall c = dense_call(const_cast<float*>(x), dims, nz, ny, nx, out, cap, sc);
+    c.rate = rate;
+    CK_TRY(codec_rate_compress_dev(c, st));
     long long h[5];
     CK_TRY(cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st));
     CK_TRY(cudaStreamSynchronize(st));
@@ -3047,13 +3100,9 @@ extern "C" int ckfwi_codec_decompress(const uint32_t* in, long long nwords, int 
     DevMem& scal = *g_codec_scal[dev];
     CK_TRY(scal.alloc(64, true));
     CK_TRY(cudaMemsetAsync(scal.p, 0, 64, st));
-    CodecView v{};
-    v.dims = dims; v.nz = nz; v.ny = ny; v.nx = nx;
-    v.py = nx;
-    v.pz = (long long)ny * nx;
-    v.aligned = (nx % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
     long long* sc = scal.as<long long>();
-    int* err = reinterpret_cast<int*>(sc + 4);
+    CodecCall c = dense_call(x, dims, nz, ny, nx, const_cast<uint32_t*>(in), nwords, sc);
+    int* err = c.one.err;
     // the header's version word says which mode wrote the stream
     uint32_t hv[9] = {};
     if (nwords < 16) return CKFWI_CORRUPT;
@@ -3061,9 +3110,10 @@ extern "C" int ckfwi_codec_decompress(const uint32_t* in, long long nwords, int 
     CK_TRY(cudaStreamSynchronize(st));
     if ((hv[1] >> 8) == 2u) {
         if (hv[8] < 1u || hv[8] > 32u) return CKFWI_CORRUPT;   // the rate word of a fixed-rate stream
-        CK_TRY(codec_rate_decompress_dev(in, sc, nwords, v, (int)hv[8], x, err, st));
+        c.rate = (int)hv[8];
+        CK_TRY(codec_rate_decompress_dev(c, st));
     } else {
-        CK_TRY(codec_decompress_dev(in, sc, nwords, v, x, err, st));
+        CK_TRY(codec_decompress_dev(c, st));
     }
     int e = 0;
     CK_TRY(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -40,9 +40,16 @@
 //     writes them back over the slot, with the chunk's word count, which it
 //     also adds to the sums of its group of 32 and of 1024 chunks;
 //  2. compact: a small CTA per 4 chunks copies them from staging to the
-//     payload at offsets formed from at most (chunks / 1024) + 62 group sums
-//     and chunk counts (linear total work); CTA 0 writes the header, the
-//     last CTA resets the group sums.
+//     payload, and their blocks' sizes to the table, at offsets formed from
+//     at most (chunks / 1024) + 62 group sums and chunk counts (linear total
+//     work); CTA 0 writes the header, the last CTA resets the group sums.
+// Both launches take every field of a call: one or two fields of each of
+// several lanes (blockIdx.y).  A lane's second stream starts where its first
+// ends, which the compaction forms from the first field's group sums, so the
+// encoder knows no pool position and a takeshot of any number of shots is two
+// launches.  (One launch pair per field left most of the GPU idle on 2D
+// fields: 464 x 1104, eight shots, 16 pairs of 12.4 + 5.4 us a takeshot;
+// now one pair of 40 + 20 us.)
 // The pool position of a stream is read from and written to device memory,
 // so a schedule of compressions and decompressions runs without host
 // synchronisation; running out of pool raises an error bit and the stream
@@ -392,10 +399,7 @@ __device__ __forceinline__ int encode_block(const float* __restrict__ x, const C
 // its groups of 32 and of 1024 chunks (the compaction's offsets).
 constexpr int ENC_MIN_CTAS = 10;
 template <int DIMS>
-__global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const float* __restrict__ x, CodecView v,
-                                                          Geo G, float tol_f, uint32_t* __restrict__ scratch,
-                                                          uint32_t* __restrict__ out, const long long* base_word,
-                                                          long long cap_words, int* err)
+__global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const __grid_constant__ CodecCall call)
 {
     constexpr int V = Cfg<DIMS>::V;
     constexpr int CWD = V > 32 ? V : 32;       // plane words need 32 rows even in 2D
@@ -403,25 +407,20 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const fl
     constexpr int MW = Cfg<DIMS>::AREA;
     __shared__ uint32_t colw[CWD * ENC_THREADS];
     __shared__ uint32_t xtra[ENC_THREADS / 32][4];
+    int fld;
+    const CodecLane& A = item_of(call, fld);
+    const Geo G = geo_of(A.v);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const long long b = (long long)blockIdx.x * ENC_THREADS + threadIdx.x;
-    const long long base = *base_word;
-    if (base + G.table_words > cap_words) {
-        if (b == 0) atomicOr(err, 2);
-        return;
-    }
-    const ScratchLayout L = scratch_layout(G);
-    uint16_t* sizes = reinterpret_cast<uint16_t*>(out + base + HDR + G.nchunks);
-    if (b == 0 && (G.nblocks & 1)) sizes[G.nblocks] = 0;
     const long long c = b / CHUNK;
-    uint32_t* stage = scratch + L.stage + c * L.cw;          // dereferenced only for c < nchunks
+    if (c >= G.nchunks) return;                // whole warp
+    const ScratchLayout L = scratch_layout(G);
+    uint32_t* scratch = static_cast<uint32_t*>(A.scratch) + fld * L.words;
+    uint32_t* stage = scratch + L.stage + c * L.cw;
     uint32_t* gs = stage + (b % CHUNK) * MW;
     int nbits = 0;
-    if (b < G.nblocks) {
-        nbits = encode_block<DIMS>(x, v, G, tol_f, b, colw + threadIdx.x, gs, err);
-        sizes[b] = (uint16_t)nbits;
-    }
-    if (c >= G.nchunks) return;                // whole warp
+    if (b < G.nblocks) nbits = encode_block<DIMS>(A.f[call.src[fld]], A.v, G, call.tol_f, b, colw + threadIdx.x, gs, A.err);
+    reinterpret_cast<uint16_t*>(scratch + L.sizes)[b] = (uint16_t)nbits;    // 0 past the last block
     __syncwarp();
     int incl = nbits;
 #pragma unroll
@@ -472,33 +471,33 @@ constexpr int CMP_THREADS = 128;
 constexpr int CPB = 4;
 
 template <int DIMS>
-__global__ void __launch_bounds__(CMP_THREADS) compact_kernel(uint32_t* __restrict__ out, const long long* base_word,
-                                                              long long cap_words, long long* next_word, Geo G,
-                                                              float tol_f, uint32_t* __restrict__ scratch,
-                                                              int* err, unsigned long long* stat_words)
+__global__ void __launch_bounds__(CMP_THREADS) compact_kernel(const __grid_constant__ CodecCall call)
 {
     constexpr int NW = CMP_THREADS / 32;
-    __shared__ long long red[2][NW];
+    __shared__ long long red[3][NW];
     __shared__ uint32_t offs[CPB + 1];
     __shared__ int s_last;
+    int fld;
+    const CodecLane& A = item_of(call, fld);
+    const Geo G = geo_of(A.v);
+    const long long c0 = (long long)blockIdx.x * CPB;
+    if (c0 >= G.nchunks) return;                       // whole CTA
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const long long base = *base_word;
-    if (base + G.table_words > cap_words) {            // the encoder raised the error
-        if (blockIdx.x == 0 && threadIdx.x == 0) *next_word = base;
-        return;
-    }
+    const long long cap_words = A.cap_words;
     const ScratchLayout L = scratch_layout(G);
     const long long ng1 = (G.nchunks + 31) / 32, ng2 = (G.nchunks + 1023) / 1024;
+    uint32_t* scratch0 = static_cast<uint32_t*>(A.scratch);      // the lane's first field
+    uint32_t* scratch = scratch0 + fld * L.words;
     const uint32_t* counts = scratch + L.counts;
-    uint32_t* g1 = scratch + L.g1;
-    uint32_t* g2 = scratch + L.g2;
-    const long long c0 = (long long)blockIdx.x * CPB;
+    const uint32_t* g1 = scratch + L.g1;
+    const uint32_t* g2 = scratch + L.g2;
     const long long q2 = c0 >> 10, q1 = c0 >> 5;
-    long long before = 0, total = 0;
+    long long before = 0, total = 0, first = 0;        // first: the first field's total, in a second field's CTAs
     for (long long i = threadIdx.x; i < ng2; i += CMP_THREADS) {
         const uint32_t w = g2[i];
         total += w;
         if (i < q2) before += w;
+        if (fld) first += scratch0[L.g2 + i];
     }
     for (long long g = (q2 << 5) + threadIdx.x; g < q1; g += CMP_THREADS) before += g1[g];
     for (long long k = (q1 << 5) + threadIdx.x; k < c0; k += CMP_THREADS) before += counts[k];
@@ -514,33 +513,50 @@ __global__ void __launch_bounds__(CMP_THREADS) compact_kernel(uint32_t* __restri
     for (int o = 16; o > 0; o >>= 1) {
         before += __shfl_xor_sync(0xffffffffu, before, o);
         total += __shfl_xor_sync(0xffffffffu, total, o);
+        first += __shfl_xor_sync(0xffffffffu, first, o);
     }
     if (lane == 0) {
         red[0][wid] = before;
         red[1][wid] = total;
+        red[2][wid] = first;
     }
     __syncthreads();
     long long prefix = 0;
-    total = 0;
+    total = first = 0;
 #pragma unroll
     for (int k = 0; k < NW; ++k) {
         prefix += red[0][k];
         total += red[1][k];
+        first += red[2][k];
     }
-    // every thread of this CTA has read the sums; the last CTA resets them
+    // every thread of this CTA has read the sums; the last CTA of the lane's
+    // fields resets them (the counter is the first field's)
     if (threadIdx.x == 0) {
+        const unsigned ctas = (unsigned)((G.nchunks + CPB - 1) / CPB) * call.nf;
         __threadfence();
-        s_last = atomicAdd(scratch, 1u) == gridDim.x - 1;
+        s_last = atomicAdd(scratch0, 1u) == ctas - 1;
     }
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (long long i = threadIdx.x; i < ng1; i += CMP_THREADS) g1[i] = 0u;
-        for (long long i = threadIdx.x; i < ng2; i += CMP_THREADS) g2[i] = 0u;
-        if (threadIdx.x == 0) scratch[0] = 0u;
+        for (int k = 0; k < call.nf; ++k) {
+            uint32_t* sk = scratch0 + k * L.words;
+            for (long long i = threadIdx.x; i < ng1; i += CMP_THREADS) sk[L.g1 + i] = 0u;
+            for (long long i = threadIdx.x; i < ng2; i += CMP_THREADS) sk[L.g2 + i] = 0u;
+        }
+        if (threadIdx.x == 0) scratch0[0] = 0u;
     }
+    long long base = A.base[call.from[0]];
+    if (fld && base + G.table_words + first <= cap_words) base += G.table_words + first;
     const long long end = base + G.table_words + total;
-    uint32_t* hdr = out + base;
+    const bool fits = end <= cap_words;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (!fits) atomicOr(A.err, 2);
+        A.base[fld + 1 < call.nf ? call.from[1] : call.to] = fits ? end : base;
+        if (A.stat) atomicAdd(A.stat + call.stat0 + fld, (unsigned long long)(G.table_words + total));
+    }
+    if (!fits) return;                                 // overflow: nothing is written
+    uint32_t* hdr = A.pool + base;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hdr[0] = MAGIC;
         hdr[1] = (uint32_t)G.dims | (VERSION << 8);
@@ -550,27 +566,24 @@ __global__ void __launch_bounds__(CMP_THREADS) compact_kernel(uint32_t* __restri
         hdr[5] = (uint32_t)G.nblocks;
         hdr[6] = (uint32_t)G.nchunks;
         hdr[7] = (uint32_t)total;
-        hdr[8] = __float_as_uint(tol_f);
-        hdr[9] = (*err & 1) ? 1u : 0u;
+        hdr[8] = __float_as_uint(call.tol_f);
+        hdr[9] = (*A.err & 1) ? 1u : 0u;
         for (int i = 10; i < HDR; ++i) hdr[i] = 0u;
-        if (end > cap_words) {
-            atomicOr(err, 2);
-            *next_word = base;
-        } else {
-            *next_word = end;
-        }
-        if (stat_words) atomicAdd(stat_words, (unsigned long long)(G.table_words + total));
     }
-    if (end > cap_words) return;                       // overflow: nothing is written
     if (threadIdx.x < CPB && c0 + threadIdx.x < G.nchunks) {
         const int k = threadIdx.x;
-        if (offs[k + 1] - offs[k] > (uint32_t)L.cw) atomicOr(err, 4);   // not a count the encoder can write
+        if (offs[k + 1] - offs[k] > (uint32_t)L.cw) atomicOr(A.err, 4);   // not a count the encoder can write
         hdr[HDR + c0 + k] = (uint32_t)(prefix + offs[k]);
+    }
+    // the sizes of the CTA's blocks, two to a word (the word of an odd last block is half zero)
+    {
+        const long long w = c0 * (CHUNK / 2) + threadIdx.x;
+        if (threadIdx.x < CPB * CHUNK / 2 && w < (G.nblocks + 1) / 2) hdr[HDR + G.nchunks + w] = scratch[L.sizes + w];
     }
     // the CTA's chunks are contiguous in the payload: every thread copies
     // words of them (all loads independent, so their latencies overlap)
     const uint32_t gw = offs[CPB];
-    uint32_t* payload = out + base + G.table_words + prefix;
+    uint32_t* payload = hdr + G.table_words + prefix;
     const uint32_t* stage = scratch + L.stage + c0 * L.cw;
     for (uint32_t w = threadIdx.x; w < gw; w += CMP_THREADS) {
         int lo = 0;
@@ -595,19 +608,25 @@ __device__ __forceinline__ unsigned long long peek64(const uint32_t* __restrict_
 }
 
 template <int DIMS>
-__global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const uint32_t* __restrict__ in, const long long* base_word,
-                                                          long long cap_words, Geo G, CodecView v,
-                                                          float* __restrict__ x, int* err)
+__global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_constant__ CodecCall call)
 {
     constexpr int V = Cfg<DIMS>::V;
     constexpr int CWD = V > 32 ? V : 32;
     __shared__ uint32_t colw[CWD * DEC_THREADS];
     uint32_t* col = colw + threadIdx.x;
+    int fld;
+    const CodecLane& A = item_of(call, fld);
+    const CodecView& v = A.v;
+    const Geo G = geo_of(v);
+    const uint32_t* __restrict__ in = A.pool;
+    float* __restrict__ x = A.f[call.src[fld]];
+    int* err = A.err;
+    const long long cap_words = A.cap_words;
     const long long b = (long long)blockIdx.x * DEC_THREADS + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const long long c = b / CHUNK;
     if (c >= G.nchunks) return;                    // whole warp
-    const long long base = *base_word;
+    const long long base = A.base[call.from[fld]];
     if (base < 0 || base + G.table_words > cap_words) {
         if (lane == 0) atomicOr(err, 4);
         return;
@@ -752,9 +771,9 @@ long long codec_bound_words(int dims, int nz, int ny, int nx)
     return G.table_words + G.nchunks * per_chunk;
 }
 
-long long codec_scratch_bytes(int dims, int nz, int ny, int nx)
+long long codec_scratch_bytes(int dims, int nz, int ny, int nx, int fields)
 {
-    return scratch_layout(make_geo(dims, nz, ny, nx)).words * 4;
+    return scratch_layout(make_geo(dims, nz, ny, nx)).words * 4 * fields;
 }
 
 long long codec_scratch_zero_bytes(int dims, int nz, int ny, int nx)
@@ -762,35 +781,30 @@ long long codec_scratch_zero_bytes(int dims, int nz, int ny, int nx)
     return scratch_zero_words(make_geo(dims, nz, ny, nx)) * 4;
 }
 
-cudaError_t codec_compress_dev(const float* x, const CodecView& v, float tol_f, uint32_t* out,
-                               const long long* base_word, long long cap_words, long long* next_word,
-                               void* scratch, int* err, unsigned long long* stat_words, cudaStream_t s)
+long long codec_blocks(int dims, int nz, int ny, int nx) { return make_geo(dims, nz, ny, nx).nblocks; }
+
+cudaError_t codec_compress_dev(const CodecCall& c, cudaStream_t s)
 {
-    const Geo G = make_geo(v.dims, v.nz, v.ny, v.nx);
-    uint32_t* sc = static_cast<uint32_t*>(scratch);
-    const unsigned eb = (unsigned)((G.nblocks + ENC_THREADS - 1) / ENC_THREADS);
-    const unsigned cb = (unsigned)((G.nchunks + CPB - 1) / CPB);
-    if (v.dims == 3) {
-        enc_kernel<3><<<eb, ENC_THREADS, 0, s>>>(x, v, G, tol_f, sc, out, base_word, cap_words, err);
-        compact_kernel<3><<<cb, CMP_THREADS, 0, s>>>(out, base_word, cap_words, next_word, G, tol_f, sc, err,
-                                                         stat_words);
+    const unsigned items = (unsigned)(c.lanes * c.nf);
+    const long long chunks = (c.blocks + CHUNK - 1) / CHUNK;
+    const dim3 eg((unsigned)((c.blocks + ENC_THREADS - 1) / ENC_THREADS), items);
+    const dim3 cg((unsigned)((chunks + CPB - 1) / CPB), items);
+    if (c.dims == 3) {
+        enc_kernel<3><<<eg, ENC_THREADS, 0, s>>>(c);
+        compact_kernel<3><<<cg, CMP_THREADS, 0, s>>>(c);
     } else {
-        enc_kernel<2><<<eb, ENC_THREADS, 0, s>>>(x, v, G, tol_f, sc, out, base_word, cap_words, err);
-        compact_kernel<2><<<cb, CMP_THREADS, 0, s>>>(out, base_word, cap_words, next_word, G, tol_f, sc, err,
-                                                         stat_words);
+        enc_kernel<2><<<eg, ENC_THREADS, 0, s>>>(c);
+        compact_kernel<2><<<cg, CMP_THREADS, 0, s>>>(c);
     }
     return cudaGetLastError();
 }
 
-cudaError_t codec_decompress_dev(const uint32_t* in, const long long* base_word, long long cap_words,
-                                 const CodecView& v, float* x, int* err, cudaStream_t s)
+cudaError_t codec_decompress_dev(const CodecCall& c, cudaStream_t s)
 {
-    const Geo G = make_geo(v.dims, v.nz, v.ny, v.nx);
-    const unsigned db = (unsigned)((G.nchunks * CHUNK + DEC_THREADS - 1) / DEC_THREADS);
-    if (v.dims == 3)
-        dec_kernel<3><<<db, DEC_THREADS, 0, s>>>(in, base_word, cap_words, G, v, x, err);
-    else
-        dec_kernel<2><<<db, DEC_THREADS, 0, s>>>(in, base_word, cap_words, G, v, x, err);
+    const long long chunks = (c.blocks + CHUNK - 1) / CHUNK;
+    const dim3 dg((unsigned)((chunks * CHUNK + DEC_THREADS - 1) / DEC_THREADS), (unsigned)(c.lanes * c.nf));
+    if (c.dims == 3) dec_kernel<3><<<dg, DEC_THREADS, 0, s>>>(c);
+    else dec_kernel<2><<<dg, DEC_THREADS, 0, s>>>(c);
     return cudaGetLastError();
 }
 

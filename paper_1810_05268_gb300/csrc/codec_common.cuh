@@ -39,14 +39,16 @@ __host__ __device__ inline Geo make_geo(int dims, int nz, int ny, int nx)
     return G;
 }
 
-// Scratch of one fixed-accuracy compression, in 32-bit words: a counter of
-// finished compaction CTAs, the payload words of every group of 1024 chunks
-// and of every group of 32 chunks (accumulated by the encoder, read and
-// reset to zero by the compaction), each chunk's word count, and each
-// chunk's staging slot of CW = 32 AREA words (first the blocks' own streams,
+__host__ __device__ inline Geo geo_of(const CodecView& v) { return make_geo(v.dims, v.nz, v.ny, v.nx); }
+
+// Scratch of one field's fixed-accuracy compression, in 32-bit words: a
+// counter of finished compaction CTAs, the payload words of every group of
+// 1024 chunks and of every group of 32 chunks (accumulated by the encoder,
+// read and reset to zero by the compaction), each chunk's word count, the
+// blocks' bit sizes (16 bits each, whole chunks), and each chunk's staging slot of CW = 32 AREA words (first the blocks' own streams,
 // AREA words apart, then the chunk's bits assembled contiguously).
 struct ScratchLayout {
-    long long g2, g1, counts, stage, words;
+    long long g2, g1, counts, sizes, stage, words;
     int cw;
 };
 constexpr ScratchLayout scratch_layout_for(int dims, long long nchunks)
@@ -57,8 +59,9 @@ constexpr ScratchLayout scratch_layout_for(int dims, long long nchunks)
     L.g2 = 32;
     L.g1 = L.g2 + ng2;
     L.counts = (L.g1 + ng1 + 31) / 32 * 32;
-    L.stage = (L.counts + nchunks + 63) / 64 * 64;
-    L.words = L.stage + nchunks * L.cw;
+    L.sizes = (L.counts + nchunks + 31) / 32 * 32;
+    L.stage = (L.sizes + nchunks * (CHUNK / 2) + 63) / 64 * 64;
+    L.words = L.stage + nchunks * L.cw;                     // a multiple of 64
     return L;
 }
 __host__ __device__ inline ScratchLayout scratch_layout(const Geo& G) { return scratch_layout_for(G.dims, G.nchunks); }
@@ -174,6 +177,14 @@ __device__ __forceinline__ uint32_t nega(int32_t c) { return ((uint32_t)c + 0xAA
 __device__ __forceinline__ int32_t unnega(uint32_t n) { return (int32_t)((n ^ 0xAAAAAAAAu) - 0xAAAAAAAAu); }
 
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
+
+// item blockIdx.y of a call: lane and field
+__device__ __forceinline__ const CodecLane& item_of(const CodecCall& c, int& k)
+{
+    const int l = c.nf == 2 ? blockIdx.y >> 1 : blockIdx.y;
+    k = c.nf == 2 ? blockIdx.y & 1 : 0;
+    return c.tab ? c.tab[l] : c.one;
+}
 
 // block coordinates and clamped sample positions
 struct BlockPos { int bz, by, bx; };

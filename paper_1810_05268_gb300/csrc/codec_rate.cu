@@ -74,21 +74,32 @@ struct RateW {
     }
 };
 
-__global__ void rate_header_kernel(uint32_t* __restrict__ out, const long long* base_word, long long cap_words,
-                                   long long* next_word, Geo G, int rate, int* err, unsigned long long* stat_words)
+// First word of field `fld`'s stream: a lane's second stream follows its
+// first (every stream has the same length), which starts at the word in
+// base[from[0]]; a stream that does not fit the pool takes no room.
+__device__ __forceinline__ long long rate_base(const CodecCall& c, const CodecLane& A, int fld, long long total)
 {
-    const long long W = rate_block_words(G.dims, rate);
-    const long long total = HDR + G.nblocks * W;
-    const long long base = *base_word;
-    if (base + total > cap_words) {
-        if (threadIdx.x == 0) {
-            atomicOr(err, 2);
-            *next_word = base;
-        }
-        return;
+    const long long b = A.base[c.from[0]];
+    return fld && b + total <= A.cap_words ? b + total : b;
+}
+
+// The 16 header words, the pool's next word and the statistics of every
+// field of a call, before its blocks are coded (a block with a non-finite
+// value marks the header).
+__global__ void rate_header_kernel(const __grid_constant__ CodecCall c)
+{
+    int fld;
+    const CodecLane& A = item_of(c, fld);
+    const Geo G = geo_of(A.v);
+    const long long total = HDR + G.nblocks * rate_block_words(G.dims, c.rate);
+    const long long base = rate_base(c, A, fld, total);
+    const bool fits = base + total <= A.cap_words;
+    if (threadIdx.x == 0) {
+        if (!fits) atomicOr(A.err, 2);
+        A.base[fld + 1 < c.nf ? c.from[1] : c.to] = fits ? base + total : base;
+        if (fits && A.stat) A.stat[c.stat0 + fld] = (unsigned long long)total;
     }
-    uint32_t* o = out + base;
-    if (threadIdx.x < HDR) {
+    if (fits && threadIdx.x < HDR) {
         uint32_t h = 0;
         switch (threadIdx.x) {
         case 0: h = MAGIC; break;
@@ -97,36 +108,34 @@ __global__ void rate_header_kernel(uint32_t* __restrict__ out, const long long* 
         case 3: h = (uint32_t)G.ny; break;
         case 4: h = (uint32_t)G.nx; break;
         case 5: h = (uint32_t)G.nblocks; break;
-        case 7: h = (uint32_t)(G.nblocks * W); break;
-        case 8: h = (uint32_t)rate; break;
+        case 7: h = (uint32_t)(total - HDR); break;
+        case 8: h = (uint32_t)c.rate; break;
         default: h = 0;
         }
-        o[threadIdx.x] = h;
-    }
-    if (threadIdx.x == 0) {
-        *next_word = base + total;
-        if (stat_words) *stat_words = (unsigned long long)total;
+        A.pool[base + threadIdx.x] = h;
     }
 }
 
 template <int DIMS>
-__global__ void __launch_bounds__(RT) rate_enc_kernel(const float* __restrict__ x, CodecView v, Geo G, int rate,
-                                                      uint32_t* __restrict__ out, const long long* base_word,
-                                                      long long cap_words, int* err)
+__global__ void __launch_bounds__(RT) rate_enc_kernel(const __grid_constant__ CodecCall call)
 {
     constexpr int V = Cfg<DIMS>::V;
     constexpr Perm P = make_perm(DIMS);
     __shared__ unsigned long long spl[32][RT];      // plane masks of each thread's block
+    int fld;
+    const CodecLane& A = item_of(call, fld);
+    const Geo G = geo_of(A.v);
     const int tid = threadIdx.x;
     const long long b = (long long)blockIdx.x * RT + tid;
     if (b >= G.nblocks) return;
-    const int W = (int)rate_block_words(DIMS, rate);
-    const long long base = *base_word;
-    if (base + HDR + G.nblocks * W > cap_words) return;     // the header kernel raised the error
-    uint32_t* o = out + base + HDR + b * W;
+    const int W = (int)rate_block_words(DIMS, call.rate);
+    const long long total = HDR + G.nblocks * W;
+    const long long base = rate_base(call, A, fld, total);
+    if (base + total > A.cap_words) return;                 // the header kernel raised the error
+    uint32_t* o = A.pool + base + HDR + b * W;
 
     float f[V];
-    gather<DIMS>(x, v, block_pos(G, b), f);
+    gather<DIMS>(A.f[call.src[fld]], A.v, block_pos(G, b), f);
     bool bad = false;
     int emax = -1000;
 #pragma unroll
@@ -138,8 +147,8 @@ __global__ void __launch_bounds__(RT) rate_enc_kernel(const float* __restrict__ 
     }
     if (bad || emax < RATE_EMIN) {           // zero-coded block (no non-zero value: emax = -1000)
         if (bad) {
-            atomicOr(err, 1);
-            atomicOr(out + base + 9, 1u);
+            atomicOr(A.err, 1);
+            atomicOr(A.pool + base + 9, 1u);
         }
         for (int k = 0; k < W; ++k) o[k] = 0u;
         return;
@@ -217,18 +226,25 @@ struct RateR {
 };
 
 template <int DIMS>
-__global__ void __launch_bounds__(RT) rate_dec_kernel(const uint32_t* __restrict__ in, const long long* base_word,
-                                                      long long cap_words, Geo G, int rate, CodecView v,
-                                                      float* __restrict__ x, int* err)
+__global__ void __launch_bounds__(RT) rate_dec_kernel(const __grid_constant__ CodecCall call)
 {
     constexpr int V = Cfg<DIMS>::V;
     constexpr Perm P = make_perm(DIMS);
     __shared__ unsigned long long spl[32][RT];
+    int fld;
+    const CodecLane& A = item_of(call, fld);
+    const CodecView& v = A.v;
+    const Geo G = geo_of(v);
+    const uint32_t* __restrict__ in = A.pool;
+    float* __restrict__ x = A.f[call.src[fld]];
+    int* err = A.err;
+    const long long cap_words = A.cap_words;
+    const int rate = call.rate;
     const int tid = threadIdx.x;
     const long long b = (long long)blockIdx.x * RT + tid;
     if (b >= G.nblocks) return;
     const int W = (int)rate_block_words(DIMS, rate);
-    const long long base = *base_word;
+    const long long base = A.base[call.from[fld]];
     if (base < 0 || base + HDR + G.nblocks * W > cap_words) {
         atomicOr(err, 4);
         return;
@@ -323,27 +339,23 @@ long long codec_rate_words(int dims, int nz, int ny, int nx, int rate)
     return HDR + G.nblocks * rate_block_words(dims, rate);
 }
 
-cudaError_t codec_rate_compress_dev(const float* x, const CodecView& v, int rate, uint32_t* out,
-                                    const long long* base_word, long long cap_words, long long* next_word, int* err,
-                                    unsigned long long* stat_words, cudaStream_t s)
+cudaError_t codec_rate_compress_dev(const CodecCall& c, cudaStream_t s)
 {
-    if (rate < 1 || rate > 32) return cudaErrorInvalidValue;
-    const Geo G = make_geo(v.dims, v.nz, v.ny, v.nx);
-    const unsigned nb = (unsigned)((G.nblocks + RT - 1) / RT);
-    rate_header_kernel<<<1, 32, 0, s>>>(out, base_word, cap_words, next_word, G, rate, err, stat_words);
-    if (v.dims == 3) rate_enc_kernel<3><<<nb, RT, 0, s>>>(x, v, G, rate, out, base_word, cap_words, err);
-    else rate_enc_kernel<2><<<nb, RT, 0, s>>>(x, v, G, rate, out, base_word, cap_words, err);
+    if (c.rate < 1 || c.rate > 32) return cudaErrorInvalidValue;
+    const unsigned items = (unsigned)(c.lanes * c.nf);
+    const dim3 grd((unsigned)((c.blocks + RT - 1) / RT), items);
+    rate_header_kernel<<<dim3(1, items), 32, 0, s>>>(c);
+    if (c.dims == 3) rate_enc_kernel<3><<<grd, RT, 0, s>>>(c);
+    else rate_enc_kernel<2><<<grd, RT, 0, s>>>(c);
     return cudaGetLastError();
 }
 
-cudaError_t codec_rate_decompress_dev(const uint32_t* in, const long long* base_word, long long cap_words,
-                                      const CodecView& v, int rate, float* x, int* err, cudaStream_t s)
+cudaError_t codec_rate_decompress_dev(const CodecCall& c, cudaStream_t s)
 {
-    if (rate < 1 || rate > 32) return cudaErrorInvalidValue;
-    const Geo G = make_geo(v.dims, v.nz, v.ny, v.nx);
-    const unsigned nb = (unsigned)((G.nblocks + RT - 1) / RT);
-    if (v.dims == 3) rate_dec_kernel<3><<<nb, RT, 0, s>>>(in, base_word, cap_words, G, rate, v, x, err);
-    else rate_dec_kernel<2><<<nb, RT, 0, s>>>(in, base_word, cap_words, G, rate, v, x, err);
+    if (c.rate < 1 || c.rate > 32) return cudaErrorInvalidValue;
+    const dim3 grd((unsigned)((c.blocks + RT - 1) / RT), (unsigned)(c.lanes * c.nf));
+    if (c.dims == 3) rate_dec_kernel<3><<<grd, RT, 0, s>>>(c);
+    else rate_dec_kernel<2><<<grd, RT, 0, s>>>(c);
     return cudaGetLastError();
 }
 

@@ -255,26 +255,47 @@ struct CodecView {       // a float field to (de)compress, origin based
     bool aligned;        // rows 16-byte aligned with a multiple-of-4 pitch
 };
 long long codec_bound_words(int dims, int nz, int ny, int nx);
-long long codec_scratch_bytes(int dims, int nz, int ny, int nx);
-// leading bytes of that scratch that must be zero before a compression
+// scratch of the fixed-accuracy compression of `fields` fields at once
+long long codec_scratch_bytes(int dims, int nz, int ny, int nx, int fields);
+// leading bytes of one field's scratch that must be zero before a compression
 // (a compression leaves them zero again)
 long long codec_scratch_zero_bytes(int dims, int nz, int ny, int nx);
-// Compress into `out` at word offset read from *base_word (device), checking
-// against cap_words; writes *next_word = base + stream length (device) and
-// raises err bits: 1 NONFINITE, 2 OVERFLOW.
-cudaError_t codec_compress_dev(const float* x, const CodecView& v, float tol_f,
-                               uint32_t* out, const long long* base_word, long long cap_words,
-                               long long* next_word, void* scratch, int* err,
-                               unsigned long long* stat_words, cudaStream_t s);
-cudaError_t codec_decompress_dev(const uint32_t* in, const long long* base_word,
-                                 long long cap_words, const CodecView& v, float* x, int* err,
-                                 cudaStream_t s);
+
+// One lane's side of a codec call: the fields it may name, the stream pool
+// and the table of word offsets into it (device).
+constexpr int CODEC_FIELDS = 6;
+struct CodecLane {
+    CodecView v;
+    float* f[CODEC_FIELDS];
+    uint32_t* pool;
+    long long cap_words;
+    long long* base;
+    void* scratch;                 // fixed accuracy: one scratch per field of a call, back to back
+    int* err;                      // bits: 1 NONFINITE, 2 OVERFLOW, 4 CORRUPT
+    unsigned long long* stat;      // words of each stream, or null
+};
+// One launch group for all lanes: field k (of nf, 1 or 2) of every lane is
+// f[src[k]].  Compression: the streams follow one another in the pool, field
+// 0's from the word in base[from[0]]; field 0's end goes to base[from[1]]
+// (nf = 2), the last field's to base[to].  Decompression: field k's stream
+// starts at the word in base[from[k]].  One lane is passed by value, several
+// by a device table.
+struct CodecCall {
+    CodecLane one;
+    const CodecLane* tab;          // null: `one` alone
+    int lanes, nf, dims;
+    int src[2], from[2], to;
+    long long stat0;               // the fields' first entry of stat
+    long long blocks;              // 4^d blocks of the largest lane
+    float tol_f;                   // fixed accuracy: the bound
+    int rate;                      // fixed rate: bits per value
+};
+long long codec_blocks(int dims, int nz, int ny, int nx);
+cudaError_t codec_compress_dev(const CodecCall& c, cudaStream_t s);
+cudaError_t codec_decompress_dev(const CodecCall& c, cudaStream_t s);
 // codec_rate.cu: the fixed-rate mode (same pool conventions; rate 1..32)
 long long codec_rate_words(int dims, int nz, int ny, int nx, int rate);
-cudaError_t codec_rate_compress_dev(const float* x, const CodecView& v, int rate, uint32_t* out,
-                                    const long long* base_word, long long cap_words, long long* next_word,
-                                    int* err, unsigned long long* stat_words, cudaStream_t s);
-cudaError_t codec_rate_decompress_dev(const uint32_t* in, const long long* base_word, long long cap_words,
-                                      const CodecView& v, int rate, float* x, int* err, cudaStream_t s);
+cudaError_t codec_rate_compress_dev(const CodecCall& c, cudaStream_t s);
+cudaError_t codec_rate_decompress_dev(const CodecCall& c, cudaStream_t s);
 
 }  // namespace ckfwi

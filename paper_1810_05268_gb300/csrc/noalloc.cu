@@ -85,7 +85,7 @@ extern "C" int ckfwi_codec_compress_noalloc(const float* x, int dims, int nz, in
     const int rs = resolve(dev, &scratch, &sc);
     if (rs != CKFWI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (codec_scratch_bytes(dims, nz, ny, nx) > (long long)sizeof(uint32_t) * NOALLOC_SCRATCH_WORDS)
+    if (codec_scratch_bytes(dims, nz, ny, nx, 1) > (long long)sizeof(uint32_t) * NOALLOC_SCRATCH_WORDS)
         return CKFWI_EINVAL;
     // the stream's start word, end word and error bits start at zero, and
     // so do the scratch's counter and group sums for this field's layout
@@ -93,16 +93,26 @@ extern "C" int ckfwi_codec_compress_noalloc(const float* x, int dims, int nz, in
     if (cudaMemsetAsync(sc, 0, sizeof(long long) * 8, st) != cudaSuccess) return CKFWI_ECUDA;
     if (cudaMemsetAsync(scratch, 0, (size_t)codec_scratch_zero_bytes(dims, nz, ny, nx), st) != cudaSuccess)
         return CKFWI_ECUDA;
-    CodecView v{};
-    v.dims = dims; v.nz = nz; v.ny = ny; v.nx = nx;
-    v.py = nx;
-    v.pz = (long long)ny * nx;
-    v.aligned = (nx % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
+    CodecCall cc{};
+    CodecLane& A = cc.one;
+    A.v.dims = dims; A.v.nz = nz; A.v.ny = ny; A.v.nx = nx;
+    A.v.py = nx;
+    A.v.pz = (long long)ny * nx;
+    A.v.aligned = (nx % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
     float tf = (float)tol;
     if ((double)tf > tol) tf = std::nextafter(tf, 0.0f);
-    int* err = reinterpret_cast<int*>(sc + 4);
-    if (codec_compress_dev(x, v, tf, out, sc, cap, sc + 1, scratch, err, nullptr, st) != cudaSuccess)
-        return CKFWI_ECUDA;
+    A.f[0] = const_cast<float*>(x);           // read only by a compression
+    A.pool = out;
+    A.cap_words = cap;
+    A.base = sc;
+    A.scratch = scratch;
+    A.err = reinterpret_cast<int*>(sc + 4);
+    cc.lanes = cc.nf = 1;
+    cc.dims = dims;
+    cc.to = 1;
+    cc.blocks = nb;
+    cc.tol_f = tf;
+    if (codec_compress_dev(cc, st) != cudaSuccess) return CKFWI_ECUDA;
     long long h[5];
     if (cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess) return CKFWI_ECUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return CKFWI_ECUDA;
