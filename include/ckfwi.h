@@ -175,16 +175,18 @@ typedef struct ckfwi_stats {
                                 codec tolerance (Sec. 2.2) can be read as
                                 tol / max|u|.  Batches: the largest over all
                                 shots. */
-    /* with opts->profile: device time [ms] and launches per kernel class */
+    /* with opts->profile: device time [ms] per kernel class, and how many time
+     * steps (of all lanes together), compressed and decompressed fields it
+     * covers */
     double fwd_ms, adj_ms, comp_ms, decomp_ms, other_ms;
     long long fwd_launches, adj_launches, comp_calls, decomp_calls;
     /* stencil kernel generation the autotuner chose for the forward and the
      * reverse step: 1 register-queue, 2 TMA-fed, 3 vector-blocked, 4 fed by
      * asynchronous copies, 5 / 6 the OT4 kernels (register-queue / vector-
      * blocked), 7 lean asynchronous copies, 8 fed by tensor copies (its
-     * reverse step split in two launches); and the tile (x points, y rows,
-     * x points per thread, z planes per CTA or, for generation 2, CTAs per
-     * SM) */
+     * reverse step split in two launches), 9 many steps a launch (2D); and
+     * the tile (x points, y rows, x points per thread, z planes per CTA or,
+     * for generation 2, CTAs per SM, for generation 9, z rows) */
     int fwd_ver, fwd_bx, fwd_by, fwd_vec, fwd_zlen;
     int adj_ver, adj_bx, adj_by, adj_vec, adj_zlen;
     int fwd_pf, adj_pf;      /* generations 4 and 8: planes of prefetch (4: 0 = the

@@ -266,7 +266,7 @@ struct DevInj {
 struct ShotDev {
     int nrec = 0;
     int nst = 0;
-    DevMem ridx, rwt, wavelet;
+    DevMem ridx, rwt, rzx, wavelet;
     DevInj src, adj;
     DevMem dsim, dobs, resid;
     std::vector<unsigned char> key;    // host description the maps were built from
@@ -339,7 +339,15 @@ struct ckfwi_model {
                                     // last two reverse steps (alternating by step parity)
     bool have_model = false;
     DevMem eta, w, cvel, zero, uN;
-    DevMem work[3], lam[3], gacc;
+    DevMem work[4], lam[4], gacc;   // the fourth: 2D, where a launch of several steps writes two levels
+    DevMem ures[CODEC_NF];          // 2D codec: restored states of one launch of reverse steps
+    // 2D: the exchange buffer and step counts of launches of many steps, by
+    // tile and direction (a buffer is only ever used with one tile: an old
+    // value of another layout could look like an awaited one)
+    struct Exchange {
+        DevMem buf, epoch;
+    };
+    std::map<std::tuple<int, int, int>, Exchange> xch;
     DevMem traj;                    // store-all trajectory
     DevMem pool;                    // checkpoint pool
     HostMem hpool;                  // checkpoint slots in host memory (second level)
@@ -566,6 +574,15 @@ int set_shot(ckfwi_model* m, const ckfwi_shot* s)
         }
     }
     ST_TRY(d.adj.set(build_inj(es)));
+    if (g.dims == 2) {
+        std::vector<int2> rzx(s->nrec);
+        for (int r = 0; r < s->nrec; ++r) {
+            const long long o = ridx[(size_t)r * nst];
+            rzx[r] = make_int2((int)(o / f.pxy), (int)(o % f.pxy));
+        }
+        CK_TRY(d.rzx.alloc(rzx.size() * sizeof(int2), false));
+        CK_TRY(cudaMemcpy(d.rzx.p, rzx.data(), rzx.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    }
     CK_TRY(d.ridx.alloc(ridx.size() * sizeof(long long), false));
     CK_TRY(d.rwt.alloc(rw.size() * sizeof(float), false));
     CK_TRY(cudaMemcpy(d.ridx.p, ridx.data(), ridx.size() * sizeof(long long), cudaMemcpyHostToDevice));
@@ -603,7 +620,7 @@ struct Prof {
 // The buffers a schedule step reads and writes.  Every lane (shot) of a
 // batch runs the same schedule, so a step names roles, and each lane
 // resolves them to its own buffers.
-enum RoleKind { R_NONE, R_ZERO, R_WORK, R_LAM, R_UN, R_TRAJ, R_SLOT, R_HSTAGE, R_HREST };
+enum RoleKind { R_NONE, R_ZERO, R_WORK, R_LAM, R_UN, R_TRAJ, R_SLOT, R_HSTAGE, R_HREST, R_URES };
 struct Role {
     int kind = R_NONE;
     int idx = 0;      // work / lam index, trajectory level, or slot (>= 1)
@@ -619,6 +636,7 @@ Role lam_r(int i) { return Role{R_LAM, i, 0}; }
 Role traj_r(int n) { return Role{R_TRAJ, n, 0}; }
 Role slot_r(int s, int w) { return Role{R_SLOT, s, w}; }
 Role hstage_r(int k, int w) { return Role{R_HSTAGE, k, w}; }
+Role ures_r(int i) { return Role{R_URES, i, 0}; }
 Role hrest_r(int r, int w) { return Role{R_HREST, r, w}; }
 
 void* rptr(ckfwi_model* m, int mode, const Role& r)
@@ -630,6 +648,7 @@ void* rptr(ckfwi_model* m, int mode, const Role& r)
     case R_LAM: return org(m->lam[r.idx], f);
     case R_UN: return org(m->uN, f);
     case R_TRAJ: return m->traj.as<float>() + (size_t)r.idx * f.alloc + f.origin;
+    case R_URES: return org(m->ures[r.idx], f);
     case R_HSTAGE: return org(m->hstage[r.idx][r.which], f);
     case R_HREST: return org(m->hrest[r.idx][r.which], f);
     case R_SLOT: {
@@ -664,8 +683,9 @@ bool role_extent(const ckfwi_model* m, int mode, const Role& r, const char** bas
     const DevMem* d = nullptr;
     switch (r.kind) {
     case R_ZERO: d = &m->zero; break;
-    case R_WORK: if (r.idx < 0 || r.idx >= 3) return false; d = &m->work[r.idx]; break;
-    case R_LAM: if (r.idx < 0 || r.idx >= 3) return false; d = &m->lam[r.idx]; break;
+    case R_WORK: if (r.idx < 0 || r.idx >= 4) return false; d = &m->work[r.idx]; break;
+    case R_LAM: if (r.idx < 0 || r.idx >= 4) return false; d = &m->lam[r.idx]; break;
+    case R_URES: if (r.idx < 0 || r.idx >= CODEC_NF) return false; d = &m->ures[r.idx]; break;
     case R_UN: d = &m->uN; break;
     case R_TRAJ: if (r.idx < 0) return false; d = &m->traj; break;
     case R_HSTAGE: if (r.idx < 0 || r.idx >= 3 || r.which < 0 || r.which > 1) return false;
@@ -737,15 +757,23 @@ struct Ctx {
     bool issue = true;              // false: only collect the batch argument tables
     std::vector<FwdArgs> ftab;      // one row per lane and step, in launch order
     std::vector<AdjArgs> atab;
-    size_t fi = 0, ai = 0;          // next row
+    std::vector<Step2Args> stab;    // rows of the launches of several 2D steps
+    size_t fi = 0, ai = 0, si = 0;  // next row
+    const Step2Args* stab_d = nullptr;
     const CodecLane* ctab_d = nullptr;   // the lanes' codec sides
     const FwdArgs* ftab_d = nullptr;
     const AdjArgs* atab_d = nullptr;
     const int* fstart_d = nullptr;
     const int* astart_d = nullptr;
     long long fblocks = 0, ablocks = 0;
+    // launches of many 2D steps take the lanes in groups whose tiles fit the
+    // GPU together: group g is lanes grp[r][g] .. grp[r][g + 1] - 1 (r: reverse)
+    std::vector<int> grp[2];
     Tile bf{}, ba{};                // batch tile shapes; z-run length per lane in zf / za
     std::vector<int> zf, za;
+    // the tile of the forward / reverse steps; launches of several 2D steps take ver 9
+    const Tile& tile(bool reverse) const { return batch ? (reverse ? ba : bf) : (reverse ? m->ta : m->tf); }
+    bool several(bool reverse) const { return tile(reverse).ver == 9; }
     int nl() const { return lanes.empty() ? 1 : (int)lanes.size(); }
     ckfwi_model* lane(int l) const { return lanes.empty() ? m : lanes[l]; }
     void* ptr(int l, const Role& r) const { return rptr(lane(l), mode, r); }
@@ -918,10 +946,23 @@ int adjq_maps(ckfwi_model* m, const AdjArgs& a, CUtensorMap* mp)
     return CKFWI_OK;
 }
 
+typedef std::vector<std::pair<int, Role>> Emits;    // (level after the launch's first, destination)
+int fwd_steps2(Ctx& cx, const Role& u, const Role& up, int n, int T, bool record, const Emits& e32, const Emits& e16,
+               int ck);
+int adj_steps2(Ctx& cx, const Role& l1, const Role& l2, const Role& o0, const Role& o1, const Role* us, const int* uts,
+               int j, int T);
+
 int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, bool record, int ck,
              const Role& ck_u, const Role& ck_up)
 {
     const int NL = cx.nl();
+    if (cx.several(false)) {
+        // u^{n+1}, and the checkpoint's fields: u^{n+1} (16-bit) and u^n
+        Emits e32{{1, out}}, e16;
+        if (ck == CK_FP32) e32.emplace_back(0, ck_up);
+        if (ck == CK_BF16 || ck == CK_FP16) e16 = {{1, ck_u}, {0, ck_up}};
+        return fwd_steps2(cx, u, up, n, 1, record, e32, e16, ck);
+    }
     for (int l = 0; l < NL; ++l) {
         ckfwi_model* m = cx.lane(l);
         FwdArgs a = fwd_args(m);
@@ -1016,11 +1057,247 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
     return CKFWI_OK;
 }
 
+// ------------------------------------------- several 2D steps in one launch
+
+long long tiles_of(const FieldGeom& f, const Tile& t)
+{
+    return (long long)((f.nx + t.bx - 1) / t.bx) * ((f.nz + t.zlen - 1) / t.zlen);
+}
+
+// Lanes in groups of at most `cap` tiles each, in order; empty when a lane alone has more
+std::vector<int> step2_groups(const std::vector<ckfwi_model*>& lanes, const Tile& t, long long cap)
+{
+    std::vector<int> g{0};
+    long long have = 0;
+    for (size_t l = 0; l < lanes.size(); ++l) {
+        const long long n = tiles_of(lanes[l]->fg, t);
+        if (n > cap) return {};
+        if (have + n > cap) {
+            g.push_back((int)l);
+            have = 0;
+        }
+        have += n;
+    }
+    g.push_back((int)lanes.size());
+    return g;
+}
+
+// The tile of launches of many 2D steps: of those whose tiles (of every lane,
+// or of groups of lanes, one SM a tile) fit the GPU, the one with the least
+// estimated time of a step.  A step costs its edge points (computed first),
+// the larger of the neighbours' edges' way here (about 1500 cycles) and the
+// other points (about 1.5 cycles a vector of four at order 8); a group of
+// lanes costs a step of its own.  False when no tile fits: the grid is too
+// large for the SMs' shared memory, and the kernels of one step a launch are
+// the better ones there anyway (the step is then bound by its points, not by
+// its launch).
+bool step2_tile(const std::vector<ckfwi_model*>& lanes, bool reverse, Tile* out)
+{
+    ckfwi_model* m = lanes[0];
+    if (m->fg.dims != 2 || m->ot != 2) return false;
+    for (ckfwi_model* L : lanes)
+        if (!L->work[3].p) return false;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    int nxm = 0, nzm = 0;
+    for (ckfwi_model* L : lanes) {
+        nxm = std::max(nxm, L->fg.nx);
+        nzm = std::max(nzm, L->fg.nz);
+    }
+    const double per = 1.5 * (2 + m->K) / 6.0;   // cycles a vector
+    double best = 1e30;
+    // the smallest tile of every number of columns and rows of the widest grid
+    for (int cols = 1; cols <= nsm; ++cols)
+        for (int rows = 1; rows * cols <= nsm; ++rows) {
+            Tile t;
+            t.ver = 9;
+            t.bx = std::max(m->K <= 4 ? 8 : 16, (nxm + 4 * cols - 1) / (4 * cols) * 4);
+            t.by = 1;
+            t.zlen = std::max(std::max(4, 2 * m->K), (nzm + rows - 1) / rows);
+            t.vec = 4;
+            if (!step2_supported(2, m->K, t, reverse)) continue;
+            const std::vector<int> g = step2_groups(lanes, t, nsm);
+            if (g.empty()) continue;
+            const double vecs = (double)t.zlen * (t.bx / 4), edge = 2.0 * (m->K * (t.bx / 4) + 2.0 * t.zlen);
+            const double rest = std::max(0.0, vecs - edge) + (reverse ? vecs : 0.0);
+            const double step = 400.0 + per * std::min(edge, vecs) + std::max(1500.0, per * rest);
+            const double cost = (double)(g.size() - 1) * step;
+            if (cost < best) {
+                best = cost;
+                *out = t;
+            }
+        }
+    return best < 1e30;
+}
+
+// the lane's exchange buffer for a tile, zeroed when new
+int step2_exchange(ckfwi_model* m, const Tile& t, bool reverse, Step2Args* a)
+{
+    auto& x = m->xch[std::make_tuple(t.bx, t.zlen, reverse ? 1 : 0)];
+    const long long n = tiles_of(m->fg, t);
+    CK_TRY(x.buf.alloc(step2_exchange_bytes(m->K, t, n)));
+    CK_TRY(x.epoch.alloc(sizeof(unsigned) * (size_t)n));
+    a->xbuf = x.buf.as<uint4>();
+    a->epoch = x.epoch.as<unsigned>();
+    return CKFWI_OK;
+}
+
+int step2_args(ckfwi_model* m, const Tile& t, bool reverse, int T, Step2Args* out)
+{
+    Step2Args& a = *out;
+    a = Step2Args{};
+    a.g = m->fg;
+    a.T = T;
+    a.bx = t.bx;
+    a.bz = t.zlen;
+    a.w = org(m->w, m->fg);
+    a.eta = m->eta.as<float>();
+    a.hdt = m->hdt;
+    std::memcpy(a.c, m->c, sizeof(a.c));
+    a.src = m->shot.src.view;
+    a.err = m->flags.as<int>();
+    a.wait_limit = m->wait_limit;
+    return step2_exchange(m, t, reverse, out);
+}
+
+// one more destination of a level
+int step2_dst(Step2Args* a, int level, void* p, int type)
+{
+    for (int k = 0; k < 3; ++k)
+        if (!a->dst[level][k]) {
+            a->dst[level][k] = p;
+            a->levels[level >> 5] |= 1u << (level & 31);
+            a->dtype[level][k] = (unsigned char)type;
+            return CKFWI_OK;
+        }
+    return CKFWI_EINVAL;
+}
+
+// one lane's launch, or (batch) its row of the launch's table
+int step2_issue(Ctx& cx, const Step2Args& a, bool reverse)
+{
+    if (cx.batch) {
+        if (!cx.issue) cx.stab.push_back(a);
+        return CKFWI_OK;
+    }
+    const int tok = cx.begin(reverse ? PC_ADJ : PC_FWD);
+    cx.count[reverse ? PC_ADJ : PC_FWD] += a.T - 1;     // counted by step
+    CK_TRY(launch_step2(a, cx.tile(reverse), cx.m->K, reverse, cx.st));
+    cx.end(tok);
+    ++cx.launches;
+    return CKFWI_OK;
+}
+
+int step2_batch(Ctx& cx, int T, bool reverse)
+{
+    if (!cx.batch) return CKFWI_OK;
+    if (cx.issue) {
+        const int tok = cx.begin(reverse ? PC_ADJ : PC_FWD);
+        cx.count[reverse ? PC_ADJ : PC_FWD] += T - 1;
+        const std::vector<int>& g = cx.grp[reverse ? 1 : 0];
+        const int* start = reverse ? cx.astart_d : cx.fstart_d;
+        for (size_t k = 0; k + 1 < g.size(); ++k) {
+            // a group's own offsets follow those of the groups before it
+            const int l0 = g[k], n = g[k + 1] - l0;
+            long long blocks = 0;
+            for (int l = l0; l < l0 + n; ++l) blocks += tiles_of(cx.lane(l)->fg, cx.tile(reverse));
+            const BatchLaunch<Step2Args> b{cx.stab_d + cx.si + l0, start + l0 + k, n, 2, blocks};
+            CK_TRY(launch_step2_batch(b, cx.tile(reverse), cx.m->K, reverse, cx.st));
+            ++cx.launches;
+        }
+        cx.end(tok);
+    }
+    cx.si += cx.nl();
+    return CKFWI_OK;
+}
+
+// Forward steps n .. n + T - 1 of every lane from (u, up); e32 / e16: where
+// levels go as FP32 fields and as checkpoint fields of type ck.
+int fwd_steps2(Ctx& cx, const Role& u, const Role& up, int n, int T, bool record, const Emits& e32, const Emits& e16,
+               int ck)
+{
+    for (int l = 0; l < cx.nl(); ++l) {
+        ckfwi_model* m = cx.lane(l);
+        Step2Args a;
+        ST_TRY(step2_args(m, cx.tile(false), false, T, &a));
+        a.f1 = cx.fptr(l, u);
+        a.f2 = cx.fptr(l, up);
+        a.src.series = m->shot.wavelet.as<float>() + n;
+        for (const auto& e : e32) ST_TRY(step2_dst(&a, e.first, cx.ptr(l, e.second), CK_FP32));
+        for (const auto& e : e16) ST_TRY(step2_dst(&a, e.first, cx.ptr(l, e.second), ck));
+        if (cx.debug) {
+            ST_TRY(check_field(m, CKFWI_STORE_FP32, u, a.f1, "forward steps: u^n"));
+            ST_TRY(check_field(m, CKFWI_STORE_FP32, up, a.f2, "forward steps: u^{n-1}"));
+            for (const auto& e : e32) {
+                ST_TRY(check_field(m, CKFWI_STORE_FP32, e.second, cx.ptr(l, e.second), "forward steps: a level"));
+                ST_TRY(check_distinct(e.second, u, "forward steps: a level"));
+                ST_TRY(check_distinct(e.second, up, "forward steps: a level"));
+            }
+            for (const auto& e : e16) {
+                ST_TRY(check_field(m, CKFWI_STORE_FP16, e.second, cx.ptr(l, e.second), "forward steps: checkpoint"));
+                ST_TRY(check_distinct(e.second, u, "forward steps: checkpoint"));
+                ST_TRY(check_distinct(e.second, up, "forward steps: checkpoint"));
+            }
+        }
+        if (record) {
+            a.smp = sample_of(m, n);
+            a.rzx = m->shot.rzx.as<int2>();
+        }
+        ST_TRY(step2_issue(cx, a, false));
+    }
+    return step2_batch(cx, T, false);
+}
+
+// Reverse steps j, j - 1, .. j - T + 1 of every lane; us[i] (type uts[i])
+// holds u^{j-1-i}; lam^{j-T} goes to o0, lam^{j-T+1} to o1 (T > 1).
+int adj_steps2(Ctx& cx, const Role& l1, const Role& l2, const Role& o0, const Role& o1, const Role* us, const int* uts,
+               int j, int T)
+{
+    for (int l = 0; l < cx.nl(); ++l) {
+        ckfwi_model* m = cx.lane(l);
+        Step2Args a;
+        ST_TRY(step2_args(m, cx.tile(true), true, T, &a));
+        a.f1 = cx.fptr(l, l1);
+        a.f2 = cx.fptr(l, l2);
+        ST_TRY(step2_dst(&a, T, cx.ptr(l, o0), CK_FP32));
+        if (T > 1) ST_TRY(step2_dst(&a, T - 1, cx.ptr(l, o1), CK_FP32));
+        a.adj = m->shot.adj.view;
+        a.adj.series = m->shot.resid.as<float>() + (size_t)j * m->shot.nrec;
+        a.adj_stride = m->shot.nrec;
+        a.src.series = m->shot.wavelet.as<float>() + (j - 1);
+        a.gacc = org(m->gacc, m->fg);
+        for (int i = 0; i < T; ++i) {
+            a.u[i] = cx.ptr(l, us[i]);
+            a.ut[i] = (unsigned char)uts[i];
+        }
+        if (cx.debug) {
+            ST_TRY(check_field(m, CKFWI_STORE_FP32, l1, a.f1, "reverse steps: lambda^j"));
+            ST_TRY(check_field(m, CKFWI_STORE_FP32, l2, a.f2, "reverse steps: lambda^{j+1}"));
+            ST_TRY(check_field(m, CKFWI_STORE_FP32, o0, a.dst[T][0], "reverse steps: lambda"));
+            ST_TRY(check_distinct(o0, l1, "reverse steps: lambda"));
+            ST_TRY(check_distinct(o0, l2, "reverse steps: lambda"));
+            if (T > 1) {
+                ST_TRY(check_field(m, CKFWI_STORE_FP32, o1, a.dst[T - 1][0], "reverse steps: lambda"));
+                ST_TRY(check_distinct(o1, l1, "reverse steps: lambda"));
+                ST_TRY(check_distinct(o1, l2, "reverse steps: lambda"));
+                ST_TRY(check_distinct(o1, o0, "reverse steps: lambda"));
+            }
+            for (int i = 0; i < T; ++i)
+                ST_TRY(check_field(m, uts[i] == U_FP32 ? CKFWI_STORE_FP32 : CKFWI_STORE_FP16, us[i], a.u[i],
+                                   "reverse steps: u"));
+        }
+        ST_TRY(step2_issue(cx, a, true));
+    }
+    return step2_batch(cx, T, true);
+}
+
 // One fused reverse step j of every lane: lam^{j-1} from lam^j, lam^{j+1}
 // and the residual row j; gacc += lam^{j-1} (lap u^{j-1} + source^{j-1}).
 int adj_step(Ctx& cx, const Role& l1, const Role& l2, const Role& l0, const Role& u, int utype, int j)
 {
     const int NL = cx.nl();
+    if (cx.several(true)) return adj_steps2(cx, l1, l2, l0, NONE_R, &u, &utype, j, 1);
     for (int l = 0; l < NL; ++l) {
         ckfwi_model* m = cx.lane(l);
         AdjArgs a = adj_args(m);
@@ -1334,7 +1611,8 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         if (nf < 5) u.vec = 1;
         if (nf < 6) u.pf = 0;
         if ((u.ver == 5 || u.ver == 6) != (m->ot == 4)) return false;
-        const bool okv = u.ver == 8   ? tma_ok && tq_supported(f.dims, m->K, u) && v3_fits(f, m->K)
+        const bool okv = u.ver == 9   ? m->ot == 2 && step2_supported(f.dims, m->K, u, reverse) && tiles_of(f, u) <= nsm
+                         : u.ver == 8 ? tma_ok && tq_supported(f.dims, m->K, u) && v3_fits(f, m->K)
                          : u.ver == 7 ? v5_supported(f.dims, m->K, u) && v3_fits(f, m->K)
                          : u.ver == 6 ? ot4v_supported(f.dims, m->K, u, reverse) && v3_fits(f, m->K)
                          : u.ver == 5 ? ot4_supported(f.dims, m->K, u)
@@ -1346,7 +1624,13 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         *t = u;
         return true;
     };
-    const bool ff = forced("CKFWI_TILE_FWD", &m->tf, false), fa = forced("CKFWI_TILE_ADJ", &m->ta, true);
+    bool ff = forced("CKFWI_TILE_FWD", &m->tf, false), fa = forced("CKFWI_TILE_ADJ", &m->ta, true);
+    // a 2D grid that fits the SMs takes the kernels of many steps a launch:
+    // nothing to time (281 x 281 and 464 x 1104: 1.8 and 3.1 us a forward
+    // step, against 3.3 and 5.1 us of kernel time for one step a launch, and
+    // 6.3 us when the host launches it)
+    ff = ff || step2_tile({m}, false, &m->tf);
+    fa = fa || step2_tile({m}, true, &m->ta);
     const bool verbose = std::getenv("CKFWI_VERBOSE") != nullptr;
     // time one candidate: the median of `rounds` timings of `reps` launches
     auto time_of = [&](const Tile& t, int pass, int rounds, float* out) -> int {
@@ -1365,7 +1649,7 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         return CKFWI_OK;
     };
     // bring the clocks up before anything is timed
-    if (!cands.empty()) {
+    if (!cands.empty() && !(ff && fa)) {
         for (int k = 0; k < 30; ++k) ST_TRY(go(cands[0], k & 1));
         CK_TRY(cudaStreamSynchronize(st));
     }
@@ -1403,8 +1687,13 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    // exchange buffers, before any recording (allocating is not recorded)
+    Step2Args x2;
+    if (m->tf.ver == 9) ST_TRY(step2_exchange(m, m->tf, false, &x2));
+    if (m->ta.ver == 9) ST_TRY(step2_exchange(m, m->ta, true, &x2));
     // the probe runs wrote into working buffers; clear them
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 4; ++i) {
+        if (!m->work[i].p) continue;
         CK_TRY(cudaMemsetAsync(m->work[i].p, 0, m->work[i].bytes, st));
         CK_TRY(cudaMemsetAsync(m->lam[i].p, 0, m->lam[i].bytes, st));
     }
@@ -1432,6 +1721,12 @@ int read_flags(ckfwi_model* m, cudaStream_t st, int* fl)
     if (h[1] & 2) *fl = CKFWI_POOL_OVERFLOW;
     else if (h[1] & 4) *fl = CKFWI_CORRUPT;
     else if (h[0] & 8) *fl = CKFWI_TIMEOUT;
+    // a launch of many steps that gave up leaves its tiles at different steps
+    if (h[0] & 8)
+        for (auto& x : m->xch) {
+            CK_TRY(cudaMemset(x.second.buf.p, 0, x.second.buf.bytes));
+            CK_TRY(cudaMemset(x.second.epoch.p, 0, x.second.epoch.bytes));
+        }
     else if ((h[0] & 1) || (h[1] & 1)) *fl = CKFWI_NONFINITE;
     return CKFWI_OK;
 }
@@ -1469,15 +1764,17 @@ CodecView field_view(const FieldGeom& f)
     return v;
 }
 
-// Fields a codec call names by index: the zero state, then the working fields
-int codec_field(const Role& r) { return r.kind == R_WORK ? 1 + r.idx : 0; }
+// Fields a codec call names by index: the zero state, the working fields,
+// the restored states
+int codec_field(const Role& r) { return r.kind == R_WORK ? 1 + r.idx : r.kind == R_URES ? 5 + r.idx : 0; }
 
 CodecLane codec_lane(ckfwi_model* m)
 {
     CodecLane a{};
     a.v = field_view(m->fg);
     a.f[0] = org(m->zero, m->fg);
-    for (int i = 0; i < 3; ++i) a.f[1 + i] = org(m->work[i], m->fg);
+    for (int i = 0; i < 4 && m->work[i].p; ++i) a.f[1 + i] = org(m->work[i], m->fg);
+    for (int i = 0; i < CODEC_NF && m->ures[i].p; ++i) a.f[5 + i] = org(m->ures[i], m->fg);
     a.pool = m->pool.as<uint32_t>();
     a.cap_words = m->cap_words;
     a.base = m->slotbase.as<long long>();
@@ -1505,12 +1802,40 @@ CodecCall codec_call(const Ctx& cx, const RunCfg& rc, int nf)
     return c;
 }
 
-// a working field that holds neither the current nor the previous state
-Role pick_free(const State& s)
+// the fields of a codec call decoded on every lane
+int decompress(Ctx& cx, const RunCfg& rc, const CodecCall& c)
 {
-    for (int i = 0; i < 3; ++i)
-        if (work_r(i) != s.cur && work_r(i) != s.prev) return work_r(i);
+    if (!cx.issue) return CKFWI_OK;
+    const int tok = cx.begin(PC_DECOMP);
+    cx.count[PC_DECOMP] += c.nf - 1;   // counted by field
+    if (rc.rate) CK_TRY(codec_rate_decompress_dev(c, cx.st));
+    else CK_TRY(codec_decompress_dev(c, cx.st));
+    cx.end(tok);
+    ++cx.launches;
+    return CKFWI_OK;
+}
+
+// a working field that holds neither the current nor the previous state (nor
+// `other`: a fourth field, in 2D)
+Role pick_free(const State& s, const Role& other = NONE_R)
+{
+    for (int i = 0; i < 4; ++i)
+        if (work_r(i) != s.cur && work_r(i) != s.prev && work_r(i) != other) return work_r(i);
     return NONE_R;
+}
+Role pick_lam(const Role& a, const Role& b, const Role& other = NONE_R)
+{
+    for (int i = 0; i < 4; ++i)
+        if (lam_r(i) != a && lam_r(i) != b && lam_r(i) != other) return lam_r(i);
+    return NONE_R;
+}
+
+// steps of the next launch when `left` are to do, at most `most` a launch: a
+// run is split evenly, so that no launch has more halo than it needs
+int block_of(int left, int most)
+{
+    const int nb = (left + most - 1) / most;
+    return (left + nb - 1) / nb;
 }
 
 // An NVTX range for the lifetime of the object (a no-op without a tool
@@ -1533,6 +1858,24 @@ struct NvtxRange {
 };
 const char* const kActionRange[4] = {"ckfwi advance", "ckfwi takeshot", "ckfwi restore", "ckfwi youturn"};
 
+// All forward steps with their receivers (no checkpoints), and d^N.
+int forward_sweep(Ctx& cx)
+{
+    State sv{ZERO_R, ZERO_R, U_FP32, U_FP32};
+    const int N = cx.m->g.nt;
+    for (int n = 0; n < N;) {
+        const int T = cx.several(false) ? block_of(N - n, STEP2_MAX) : 1;
+        const Role out = pick_free(sv), out2 = T > 1 ? pick_free(sv, out) : sv.cur;
+        if (T > 1)
+            ST_TRY(fwd_steps2(cx, sv.cur, sv.prev, n, T, true, Emits{{T, out}, {T - 1, out2}}, Emits(), CK_NONE));
+        else
+            ST_TRY(fwd_step(cx, sv.cur, sv.prev, out, n, true, CK_NONE, NONE_R, NONE_R));
+        sv = State{out, out2, U_FP32, U_FP32};
+        n += T;
+    }
+    return sample_last(cx, sv.cur);
+}
+
 // The recorded part of a gradient: everything between "inputs staged" and
 // "outputs ready" (this is what a CUDA graph captures).  Runs every lane of
 // the context through the same schedule.
@@ -1544,23 +1887,47 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
     if (cx.issue) {
         for (int l = 0; l < NL; ++l) {
             ckfwi_model* m = cx.lane(l);
-            for (int i = 0; i < 3; ++i) CK_TRY(cudaMemsetAsync(m->lam[i].p, 0, m->lam[i].bytes, cx.st));
+            for (int i = 0; i < 4; ++i)
+                if (m->lam[i].p) CK_TRY(cudaMemsetAsync(m->lam[i].p, 0, m->lam[i].bytes, cx.st));
             CK_TRY(cudaMemsetAsync(m->gacc.p, 0, m->gacc.bytes, cx.st));
             CK_TRY(cudaMemsetAsync(m->shot.dsim.p, 0, m->shot.dsim.bytes, cx.st));
             CK_TRY(cudaMemsetAsync(m->phi.as<double>() + 1, 0, sizeof(double), cx.st));
         }
     }
-    int li = 0;   // lam rotation: lam[li] = lam^{j}, lam[(li+1)%3] = lam^{j+1}
+    Role lc = lam_r(0), lp = lam_r(1);   // lam^j, lam^{j+1}
     auto reverse = [&](int s, const Role& u, int ut) -> int {
-        ST_TRY(adj_step(cx, lam_r(li), lam_r((li + 1) % 3), lam_r((li + 2) % 3), u, ut, s + 1));
-        li = (li + 2) % 3;   // new lam^{j} = old lam^{j-1}, lam^{j+1} = old lam^{j}
+        const Role o = pick_lam(lc, lp);
+        ST_TRY(adj_step(cx, lc, lp, o, u, ut, s + 1));
+        lp = lc;
+        lc = o;
+        return CKFWI_OK;
+    };
+    // reverse steps of states s, s - 1, .. (u's in that order), several a launch (2D)
+    auto reverse_run = [&](int s, const std::vector<Role>& us, const std::vector<int>& uts) -> int {
+        for (size_t i = 0; i < us.size();) {
+            const int T = block_of((int)(us.size() - i), STEP2_MAX);
+            const Role o0 = pick_lam(lc, lp), o1 = T > 1 ? pick_lam(lc, lp, o0) : NONE_R;
+            ST_TRY(adj_steps2(cx, lc, lp, o0, o1, us.data() + i, uts.data() + i, s + 1 - (int)i, T));
+            lp = T > 1 ? o1 : lc;
+            lc = o0;
+            i += T;
+        }
         return CKFWI_OK;
     };
     long long fsteps = 0;
     if (rc.store_all) {
         {
             NvtxRange range(kActionRange[ACT_ADVANCE], 0);
-            for (int n = 0; n < N; ++n) {
+            for (int n = 0; n < N && cx.several(false);) {
+                const int T = block_of(N - n, STEP2_MAX);
+                Emits out;
+                for (int i = 1; i <= T; ++i) out.emplace_back(i, n + i < N ? traj_r(n + i) : UN_R);
+                ST_TRY(fwd_steps2(cx, n == 0 ? ZERO_R : traj_r(n), n <= 1 ? ZERO_R : traj_r(n - 1), n, T, true, out,
+                                  Emits(), CK_NONE));
+                fsteps += T;
+                n += T;
+            }
+            for (int n = 0; n < N && !cx.several(false); ++n) {
                 const Role u = n == 0 ? ZERO_R : traj_r(n);
                 const Role up = n <= 1 ? ZERO_R : traj_r(n - 1);
                 const Role out = (n + 1 < N) ? traj_r(n + 1) : UN_R;
@@ -1572,6 +1939,13 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
             ST_TRY(residual(cx));
         }
         NvtxRange range(kActionRange[ACT_YOUTURN], N - 1);
+        if (cx.several(true)) {
+            std::vector<Role> us;
+            for (int s = N - 1; s >= 0; --s) us.push_back(s == 0 ? ZERO_R : traj_r(s));
+            ST_TRY(reverse_run(N - 1, us, std::vector<int>(us.size(), U_FP32)));
+            counters[0] = fsteps;
+            return CKFWI_OK;
+        }
         for (int s = N - 1; s >= 0; --s) ST_TRY(reverse(s, s == 0 ? ZERO_R : traj_r(s), U_FP32));
         counters[0] = fsteps;
         return CKFWI_OK;
@@ -1596,10 +1970,66 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
         NvtxRange range(kActionRange[A.op & 3], A.a);
         const bool next_take = ai + 1 < acts.size() && acts[ai + 1].op == ACT_TAKESHOT;
         const bool next_turn = ai + 1 < acts.size() && acts[ai + 1].op == ACT_YOUTURN;
-        if (A.op == ACT_ADVANCE) {
+        if (A.op == ACT_ADVANCE && cx.several(false) && !cx.stage) {
+            // A run of forward steps with the checkpoints taken on the way
+            // (compressed ones end it: they read the state afterwards), in
+            // launches of several steps.  A checkpoint of state s takes level
+            // s and level s - 1 of the launch that makes level s.
+            const int n0 = A.a;
+            int len = A.b;
+            std::vector<std::pair<int, int>> takes;      // (level, slot), ascending
+            while (!rc.codec && ai + 1 < acts.size()) {
+                const Action& B = acts[ai + 1];
+                if (B.op == ACT_TAKESHOT) takes.emplace_back(B.a - n0, B.b);
+                else if (B.op == ACT_ADVANCE) len += B.b;
+                else break;
+                ++ai;
+            }
+            const int ck = rc.mode == CKFWI_STORE_BF16 ? CK_BF16 : rc.mode == CKFWI_STORE_FP16 ? CK_FP16 : CK_FP32;
+            for (int i = 0; i < len;) {
+                const int T = block_of(len - i, STEP2_MAX);
+                Emits e32, e16;
+                Role out = pick_free(st), out2 = T > 1 ? pick_free(st, out) : st.cur;
+                for (const auto& t : takes) {
+                    if (t.first <= i || t.first > i + T) continue;
+                    const int lv = t.first - i;
+                    if (ck != CK_FP32) {
+                        e16.emplace_back(lv, slot_r(t.second, 0));
+                        e16.emplace_back(lv - 1, slot_r(t.second, 1));
+                    } else {
+                        e32.emplace_back(lv, slot_r(t.second, 0));
+                        e32.emplace_back(lv - 1, slot_r(t.second, 1));
+                        if (lv == T) {                   // the slot is the state from here on
+                            out = slot_r(t.second, 0);
+                            out2 = slot_r(t.second, 1);
+                        }
+                    }
+                }
+                if (out.kind == R_WORK) {
+                    e32.emplace_back(T, out);
+                    if (T > 1) e32.emplace_back(T - 1, out2);
+                }
+                ST_TRY(fwd_steps2(cx, st.cur, st.prev, n0 + i, T, first_sweep, e32, e16, ck));
+                fsteps += T;
+                st = State{out, out2, U_FP32, U_FP32};
+                i += T;
+            }
+        } else if (A.op == ACT_ADVANCE) {
             for (int i = 0; i < A.b; ++i) {
                 const int n = A.a + i;
                 const bool last = i == A.b - 1;
+                const int plain = A.b - i - (next_take ? 1 : 0);    // steps before one that writes a checkpoint
+                if (cx.several(false) && plain > 1) {
+                    const int T = block_of(plain, STEP2_MAX);
+                    const Role o0 = pick_free(st), o1 = T > 1 ? pick_free(st, o0) : st.cur;
+                    Emits e32{{T, o0}};
+                    if (T > 1) e32.emplace_back(T - 1, o1);
+                    ST_TRY(fwd_steps2(cx, st.cur, st.prev, n, T, first_sweep, e32, Emits(), CK_NONE));
+                    fsteps += T;
+                    st = State{o0, o1, U_FP32, U_FP32};
+                    i += T - 1;
+                    continue;
+                }
                 int ck = CK_NONE;
                 Role cku = NONE_R, ckup = NONE_R;
                 Role out = pick_free(st);
@@ -1752,20 +2182,13 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
             } else if (rc.mode == CKFWI_STORE_FP32) {
                 st = State{slot_r(A.b, 0), slot_r(A.b, 1), U_FP32, U_FP32};   // the slot is the state
             } else if (rc.codec) {
-                if (cx.issue) {
-                    // a reverse step needs u^s only
-                    CodecCall c = codec_call(cx, rc, next_turn ? 1 : 2);
-                    c.src[0] = codec_field(work_r(0));
-                    c.src[1] = codec_field(work_r(1));
-                    c.from[0] = A.b;
-                    c.from[1] = rc.M + 1 + A.b;
-                    const int tok = cx.begin(PC_DECOMP);
-                    cx.count[PC_DECOMP] += c.nf - 1;   // counted by field
-                    if (rc.rate) CK_TRY(codec_rate_decompress_dev(c, cx.st));
-                    else CK_TRY(codec_decompress_dev(c, cx.st));
-                    cx.end(tok);
-                    ++cx.launches;
-                }
+                // a reverse step needs u^s only
+                CodecCall c = codec_call(cx, rc, next_turn ? 1 : 2);
+                c.src[0] = codec_field(work_r(0));
+                c.src[1] = codec_field(work_r(1));
+                c.from[0] = A.b;
+                c.from[1] = rc.M + 1 + A.b;
+                ST_TRY(decompress(cx, rc, c));
                 st = State{work_r(0), work_r(1), U_FP32, U_FP32};
             } else if (next_turn) {
                 // a reverse step needs u^s only: up-cast that field.  (The
@@ -1808,7 +2231,40 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 ST_TRY(residual(cx));
                 first_sweep = false;
             }
-            ST_TRY(reverse(A.a, st.cur, st.tcur));
+            if (!cx.several(true) || cx.stage) {
+                ST_TRY(reverse(A.a, st.cur, st.tcur));
+                continue;
+            }
+            // A run of reverse steps whose states need no recomputation: the
+            // current state, then checkpoint after checkpoint, each read where
+            // it lies (FP32 and 16-bit) or decoded for its launch
+            std::vector<Role> us{st.cur};
+            std::vector<int> uts{st.tcur}, slots{-1};
+            while (ai + 2 < acts.size() && acts[ai + 1].op == ACT_RESTORE && acts[ai + 2].op == ACT_YOUTURN) {
+                const int b = acts[ai + 1].b;
+                us.push_back(b == 0 ? ZERO_R : rc.codec ? NONE_R : slot_r(b, 0));
+                uts.push_back(b == 0 ? U_FP32 : ut_slot);
+                slots.push_back(b);
+                ai += 2;
+            }
+            if (!rc.codec) {
+                ST_TRY(reverse_run(A.a, us, uts));
+                continue;
+            }
+            for (size_t i = 0; i < us.size();) {
+                const int T = block_of((int)(us.size() - i), CODEC_NF);
+                CodecCall c = codec_call(cx, rc, 0);
+                for (int k = 0; k < T; ++k) {
+                    if (us[i + k] != NONE_R) continue;
+                    us[i + k] = ures_r(c.nf);
+                    c.src[c.nf] = codec_field(us[i + k]);
+                    c.from[c.nf++] = slots[i + k];
+                }
+                if (c.nf > 0) ST_TRY(decompress(cx, rc, c));
+                ST_TRY(reverse_run(A.a - (int)i, std::vector<Role>(us.begin() + i, us.begin() + i + T),
+                                   std::vector<int>(uts.begin() + i, uts.begin() + i + T)));
+                i += T;
+            }
         }
     }
     // join the copy stream: no checkpoint copy or prefetch outlives the gradient
@@ -1838,16 +2294,16 @@ double storage_bytes(const FieldGeom& f, const RunCfg& rc, const ckfwi_grad_opts
 int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
 {
     const FieldGeom& f = m->fg;
-    const void* before[7] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d,
+    const void* before[8] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d, m->ures[0].p,
                              reinterpret_cast<const void*>((intptr_t)m->host_slots)};
     struct Bump {
         ckfwi_model* m;
         const void* const* b;
         ~Bump()
         {
-            const void* after[7] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d,
+            const void* after[8] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d, m->ures[0].p,
                                     reinterpret_cast<const void*>((intptr_t)m->host_slots)};
-            for (int i = 0; i < 7; ++i)
+            for (int i = 0; i < 8; ++i)
                 if (after[i] != b[i]) ++m->gen;
         }
     } bump{m, before};
@@ -1923,6 +2379,7 @@ int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
             CK_TRY(e);
         }
         CK_TRY(m->statw.alloc(sizeof(unsigned long long) * (size_t)(4 * rc.N + 8)));
+        for (int i = 0; m->work[3].p && i < CODEC_NF; ++i) CK_TRY(m->ures[i].alloc(field_bytes(f)));
     }
     return CKFWI_OK;
 }
@@ -2296,8 +2753,17 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
     float best[2] = {1e30f, 1e30f};
     bool warmed = false;
     BatchTiles bt;
+    // 2D lanes that fit the SMs, in groups or together: as for one model
+    bool many[2] = {false, false};
+    if (!want || want == 9) {
+        many[0] = step2_tile(lanes, false, &bt.tf);
+        many[1] = step2_tile(lanes, true, &bt.ta);
+        if (many[0]) bt.zf.assign(NL, bt.tf.zlen);
+        if (many[1]) bt.za.assign(NL, bt.ta.zlen);
+    }
     int rs = CKFWI_OK;
     for (const Cand& c : cands) {
+        if (many[0] && many[1]) break;
         long long total = 0;
         const std::vector<int> s = lane_starts(lanes, c.t, c.z, &total);
         if (total > 0x7fffffffLL) continue;
@@ -2313,6 +2779,7 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
         }
         for (int pass = 0; pass < 2 && rs == CKFWI_OK; ++pass) {
             if (pass == 1 && c.t.ver == 4) continue;    // generation 4 has no batched reverse step
+            if (many[pass]) continue;
             if (want && c.t.ver != want && !(want == 4 && pass == 1 && c.t.ver == 3)) continue;
             auto go = [&]() {
                 const BatchLaunch<FwdArgs> bf{ftab, dst.as<int>(), NL, dims, total};
@@ -2371,7 +2838,8 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
     if (bt.zf.empty() || bt.za.empty()) return CKFWI_EINVAL;
     // the probes wrote into working buffers; clear them
     for (ckfwi_model* L : lanes) {
-        for (int i = 0; i < 3; ++i) {
+        for (int i = 0; i < 4; ++i) {
+            if (!L->work[i].p) continue;
             CK_TRY(cudaMemsetAsync(L->work[i].p, 0, L->work[i].bytes, st));
             CK_TRY(cudaMemsetAsync(L->lam[i].p, 0, L->lam[i].bytes, st));
         }
@@ -2421,8 +2889,23 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
     cx.ba = bt->ta;
     cx.zf = bt->zf;
     cx.za = bt->za;
-    const std::vector<int> fs = lane_starts(lanes, cx.bf, cx.zf, &cx.fblocks);
-    const std::vector<int> as = lane_starts(lanes, cx.ba, cx.za, &cx.ablocks);
+    std::vector<int> fs = lane_starts(lanes, cx.bf, cx.zf, &cx.fblocks);
+    std::vector<int> as = lane_starts(lanes, cx.ba, cx.za, &cx.ablocks);
+    for (int r = 0; r < 2; ++r) {
+        if (!cx.several(r == 1)) continue;
+        // every group's own offsets (its lanes + 1 entries) one after the other
+        int nsm = 0, dev = 0;
+        CK_TRY(cudaGetDevice(&dev));
+        CK_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        cx.grp[r] = step2_groups(lanes, cx.tile(r == 1), nsm);
+        std::vector<int>& s = r ? as : fs;
+        s.clear();
+        for (size_t k = 0; k + 1 < cx.grp[r].size(); ++k) {
+            int at = 0;
+            s.push_back(0);
+            for (int l = cx.grp[r][k]; l < cx.grp[r][k + 1]; ++l) s.push_back(at += (int)tiles_of(lanes[l]->fg, cx.tile(r == 1)));
+        }
+    }
     if (cx.fblocks > 0x7fffffffLL || cx.ablocks > 0x7fffffffLL) return CKFWI_EINVAL;
     long long counters[2] = {0, 0};
     const bool graph = o->use_graph != 0 && !o->profile;
@@ -2448,11 +2931,12 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
         DevMem& tabs = graph ? bg.tabs : m0->btabs;
         const size_t fb = ((sizeof(FwdArgs) * cx.ftab.size() + 255) / 256) * 256;
         const size_t ab = ((sizeof(AdjArgs) * cx.atab.size() + 255) / 256) * 256;
-        const size_t sb = sizeof(int) * 2 * (NL + 1);
+        const size_t sb = sizeof(int) * (fs.size() + as.size());
+        const size_t s2 = ((sizeof(Step2Args) * cx.stab.size() + 255) / 256) * 256;
         std::vector<CodecLane> ctab;
         for (int l = 0; rc.codec && l < NL; ++l) ctab.push_back(codec_lane(lanes[l]));
         const size_t so = (sb + 255) / 256 * 256;
-        int rs = cuda_status_or_ok(tabs.alloc(fb + ab + so + sizeof(CodecLane) * ctab.size(), false));
+        int rs = cuda_status_or_ok(tabs.alloc(fb + ab + so + s2 + sizeof(CodecLane) * ctab.size(), false));
         if (rs == CKFWI_OK && !cx.ftab.empty())
             rs = cuda_status_or_ok(cudaMemcpy(tabs.p, cx.ftab.data(), sizeof(FwdArgs) * cx.ftab.size(),
                                               cudaMemcpyHostToDevice));
@@ -2465,18 +2949,22 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
             rs = cuda_status_or_ok(
                 cudaMemcpy(tabs.as<char>() + fb + ab, starts.data(), sb, cudaMemcpyHostToDevice));
         if (rs == CKFWI_OK && !ctab.empty())
-            rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so, ctab.data(),
+            rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so + s2, ctab.data(),
                                               sizeof(CodecLane) * ctab.size(), cudaMemcpyHostToDevice));
+        if (rs == CKFWI_OK && !cx.stab.empty())
+            rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so, cx.stab.data(),
+                                              sizeof(Step2Args) * cx.stab.size(), cudaMemcpyHostToDevice));
         if (rs != CKFWI_OK) {
             if (graph) m0->bgraphs.erase(key);
             return rs;
         }
-        cx.ctab_d = reinterpret_cast<const CodecLane*>(tabs.as<char>() + fb + ab + so);
+        cx.stab_d = reinterpret_cast<const Step2Args*>(tabs.as<char>() + fb + ab + so);
+        cx.ctab_d = reinterpret_cast<const CodecLane*>(tabs.as<char>() + fb + ab + so + s2);
         cx.ftab_d = tabs.as<FwdArgs>();
         cx.atab_d = reinterpret_cast<const AdjArgs*>(tabs.as<char>() + fb);
         cx.fstart_d = reinterpret_cast<const int*>(tabs.as<char>() + fb + ab);
-        cx.astart_d = cx.fstart_d + (NL + 1);
-        cx.fi = cx.ai = 0;
+        cx.astart_d = cx.fstart_d + fs.size();
+        cx.fi = cx.ai = cx.si = 0;
         cx.issue = true;
         // pass 2: issue (recorded into a graph when asked)
         if (graph) {
@@ -2630,7 +3118,7 @@ int ckfwi_create_model(const ckfwi_grid* g, ckfwi_model** out)
     CK_TRY(m->cvel.alloc((size_t)f.npts * sizeof(float)));
     CK_TRY(m->zero.alloc(field_bytes(f)));
     CK_TRY(m->uN.alloc(field_bytes(f)));
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < (g->dims == 2 && m->ot == 2 ? 4 : 3); ++i) {
         CK_TRY(m->work[i].alloc(field_bytes(f)));
         CK_TRY(m->lam[i].alloc(field_bytes(f)));
     }
@@ -2680,14 +3168,7 @@ int ckfwi_forward_shot(ckfwi_model* m, const ckfwi_shot* s, float* d_sim, int me
     ST_TRY(reset_flags(m, st));
     Ctx cx{m, st, 0};
     CK_TRY(cudaMemsetAsync(m->shot.dsim.p, 0, m->shot.dsim.bytes, st));
-    State sv{ZERO_R, ZERO_R, U_FP32, U_FP32};
-    for (int n = 0; n < m->g.nt; ++n) {
-        const Role out = pick_free(sv);
-        ST_TRY(fwd_step(cx, sv.cur, sv.prev, out, n, true, CK_NONE, NONE_R, NONE_R));
-        sv.prev = sv.cur;
-        sv.cur = out;
-    }
-    ST_TRY(sample_last(cx, sv.cur));
+    ST_TRY(forward_sweep(cx));
     const size_t nd = (size_t)(m->g.nt + 1) * m->shot.nrec;
     CK_TRY(cudaMemcpyAsync(d_sim, m->shot.dsim.p, nd * sizeof(float),
                            mem == CKFWI_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
@@ -2710,14 +3191,7 @@ int ckfwi_misfit(ckfwi_model* m, const ckfwi_shot* s, const float* d_obs, int me
     CK_TRY(cudaMemcpyAsync(m->shot.dobs.p, d_obs, nd * sizeof(float),
                            mem == CKFWI_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
     CK_TRY(cudaMemsetAsync(m->shot.dsim.p, 0, m->shot.dsim.bytes, st));
-    State sv{ZERO_R, ZERO_R, U_FP32, U_FP32};
-    for (int n = 0; n < m->g.nt; ++n) {
-        const Role out = pick_free(sv);
-        ST_TRY(fwd_step(cx, sv.cur, sv.prev, out, n, true, CK_NONE, NONE_R, NONE_R));
-        sv.prev = sv.cur;
-        sv.cur = out;
-    }
-    ST_TRY(sample_last(cx, sv.cur));
+    ST_TRY(forward_sweep(cx));
     ST_TRY(residual(cx));
     if (d_sim)
         CK_TRY(cudaMemcpyAsync(d_sim, m->shot.dsim.p, nd * sizeof(float),

@@ -181,8 +181,8 @@ __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t
 // item blockIdx.y of a call: lane and field
 __device__ __forceinline__ const CodecLane& item_of(const CodecCall& c, int& k)
 {
-    const int l = c.nf == 2 ? blockIdx.y >> 1 : blockIdx.y;
-    k = c.nf == 2 ? blockIdx.y & 1 : 0;
+    const int l = blockIdx.y / (unsigned)c.nf;
+    k = blockIdx.y - l * c.nf;
     return c.tab ? c.tab[l] : c.one;
 }
 

@@ -127,6 +127,38 @@ struct Ot4GradArgs {
     Inj src;              // Q^T s^{j-1}
 };
 
+// Many time steps of a 2D grid in one launch (stencil_2d.cu).
+constexpr int STEP2_MAX = 64;
+struct Step2Args {
+    FieldGeom g;
+    int T;                // steps
+    int bx, bz;           // tile
+    const float* f1;      // u^n (reverse: lam^j)
+    const float* f2;      // u^{n-1} (reverse: lam^{j+1})
+    const float* w;
+    const float* eta;
+    float hdt;
+    float c[MAXK + 1];
+    Inj src;              // forward: step i takes series + i; reverse: series - i
+    // destinations of level n + i and their CkMode (reverse: [i][0], lam^{j-i}, FP32)
+    void* dst[STEP2_MAX + 1][3];
+    unsigned char dtype[STEP2_MAX + 1][3];
+    unsigned levels[STEP2_MAX / 32 + 1];    // bit l: level n + l has a destination
+    int* err;
+    uint4* xbuf;          // the tiles' exchange buffer
+    unsigned* epoch;      // and each tile's step count
+    long long wait_limit; // looks at a neighbour's edge before giving up
+    // forward
+    Sample smp;           // receivers: level n + i goes to out + i n
+    const int2* rzx;      // each receiver's first point (z, x)
+    // reverse
+    Inj adj;              // step i takes series - i adj_stride
+    long long adj_stride;
+    const void* u[STEP2_MAX];       // u^{j-1-i} and its UType
+    unsigned char ut[STEP2_MAX];
+    float* gacc;
+};
+
 enum CkMode { CK_NONE = 0, CK_FP32 = 1, CK_BF16 = 2, CK_FP16 = 3 };
 enum UType { U_FP32 = 0, U_BF16 = 1, U_FP16 = 2 };
 
@@ -139,7 +171,8 @@ struct Tile {
                           // 6: the same vector-blocked (3D), 7: the lean async-copy
                           // OT2 kernels (3D, one or two planes per step), 8: the
                           // forward step fed by tensor copies and the reverse step split
-                          // in two launches (3D)
+                          // in two launches (3D), 9: many steps a launch (2D; bx x zlen
+                          // points a tile)
     int vec = 1;          // ver 3, 4: x points per thread (2 or 4)
     int pf = 0;           // ver 4: planes of prefetch (0 = the default, 2); ver 7: planes per step (1, 2);
                           // ver 8: planes of prefetch (1, 2; 0 reads as 1)
@@ -189,6 +222,13 @@ cudaError_t launch_adj5_batch(const BatchLaunch<AdjArgs>& b, const Tile& t, int 
 // batch_v3.cu (every lane's geometry must pass v3_fits)
 cudaError_t launch_fwd3_batch(const BatchLaunch<FwdArgs>& b, const Tile& t, int K, int ck, cudaStream_t s);
 cudaError_t launch_adj3_batch(const BatchLaunch<AdjArgs>& b, const Tile& t, int K, int ut, cudaStream_t s);
+
+// stencil_2d.cu: many steps a launch (Tile.ver 9)
+bool step2_supported(int dims, int K, const Tile& t, bool reverse);
+size_t step2_exchange_bytes(int K, const Tile& t, long long tiles);
+cudaError_t launch_step2(const Step2Args& a, const Tile& t, int K, bool reverse, cudaStream_t s);
+// the lanes' tiles (b.blocks) must be resident together
+cudaError_t launch_step2_batch(const BatchLaunch<Step2Args>& b, const Tile& t, int K, bool reverse, cudaStream_t s);
 
 // ot4.cu
 bool ot4_supported(int dims, int K, const Tile& t);
@@ -263,7 +303,8 @@ long long codec_scratch_zero_bytes(int dims, int nz, int ny, int nx);
 
 // One lane's side of a codec call: the fields it may name, the stream pool
 // and the table of word offsets into it (device).
-constexpr int CODEC_FIELDS = 6;
+constexpr int CODEC_NF = 8;              // most fields of a lane a call takes
+constexpr int CODEC_FIELDS = 5 + CODEC_NF;
 struct CodecLane {
     CodecView v;
     float* f[CODEC_FIELDS];
@@ -274,8 +315,8 @@ struct CodecLane {
     int* err;                      // bits: 1 NONFINITE, 2 OVERFLOW, 4 CORRUPT
     unsigned long long* stat;      // words of each stream, or null
 };
-// One launch group for all lanes: field k (of nf, 1 or 2) of every lane is
-// f[src[k]].  Compression: the streams follow one another in the pool, field
+// One launch group for all lanes: field k of nf of every lane is f[src[k]].
+// Compression (nf 1 or 2): the streams follow one another in the pool, field
 // 0's from the word in base[from[0]]; field 0's end goes to base[from[1]]
 // (nf = 2), the last field's to base[to].  Decompression: field k's stream
 // starts at the word in base[from[k]].  One lane is passed by value, several
@@ -284,7 +325,7 @@ struct CodecCall {
     CodecLane one;
     const CodecLane* tab;          // null: `one` alone
     int lanes, nf, dims;
-    int src[2], from[2], to;
+    int src[CODEC_NF], from[CODEC_NF], to;
     long long stat0;               // the fields' first entry of stat
     long long blocks;              // 4^d blocks of the largest lane
     float tol_f;                   // fixed accuracy: the bound
