@@ -31,6 +31,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <initializer_list>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -365,6 +366,7 @@ struct ckfwi_model {
     DevMem gsum_comp;               // batch: compensation terms
     ShotDev shot;
     Tile tf{}, ta{};
+    Tile t4[5];                     // OT4 fed by tensor copies: the tile of each pass (ver 10 when tuned)
     bool tuned = false;
     int nparts = 128;
     long long gen = 0;              // bumped whenever a buffer a graph uses moves
@@ -856,13 +858,58 @@ Tile host_tile(const ckfwi_model* m)
     return t;
 }
 
+// The OT4 tile of a step that reads a field tensor maps do not cover (a host
+// slot, a 16-bit field): the vector-blocked passes
+Tile ot4_host_tile(const Tile& t)
+{
+    Tile v = t;
+    if (t.ver == 10) {
+        v.ver = 6;
+        v.pf = 0;
+    }
+    return v;
+}
+
+int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by, CUtensorMap* out);
+
 // OT4 steps (ot4.cu): forward, the pass computing w lap f, then the update;
 // reverse, w lap of lam^j and u^{j-1}, the update, the gradient pass.  The
 // reverse step j writes w lap u^{j-1} into z4[1 + j % 2] and pairs the one
 // of step j + 1 with lap lam^j.
+// A pass fed by tensor copies: the staged field, then the point fields
+int ot4q_pass(ckfwi_model* m, int op, const Ot4qArgs& a, std::initializer_list<const float*> points, const Tile& t,
+              int ck, cudaStream_t st)
+{
+    CUtensorMap mp[4];
+    ST_TRY(tensor_map(m, a.s, U_FP32, tq_box_x(m->K), tq_box_y(m->K), &mp[0]));
+    int k = 1;
+    for (const float* p : points) ST_TRY(tensor_map(m, p, U_FP32, 32, 16, &mp[k++]));
+    CK_TRY(launch_ot4q(op, a, mp, m->t4[op].ver == 10 ? m->t4[op] : t, m->K, ck, st));
+    return CKFWI_OK;
+}
+
+// pass 1 and the update, forward (a.u = u^n) or of the adjoint field (lam^j)
+int ot4q_update(ckfwi_model* m, const FwdArgs& a, const Tile& t, int ck, cudaStream_t st, const float* zu_next,
+                float* gacc)
+{
+    Ot4qArgs q{};
+    q.f = a;
+    q.s = a.u;
+    q.f.out = org(m->z4[0], m->fg);
+    q.gacc = gacc;
+    std::memcpy(q.c12, m->c12, sizeof(q.c12));
+    if (zu_next) ST_TRY(ot4q_pass(m, OT4Q_LAP_LAM, q, {a.w, zu_next, gacc}, t, CK_NONE, st));
+    else ST_TRY(ot4q_pass(m, OT4Q_LAP, q, {a.w}, t, CK_NONE, st));
+    q.f = a;
+    q.f.smp = Sample{};
+    q.s = org(m->z4[0], m->fg);
+    return ot4q_pass(m, OT4Q_UPDATE, q, {a.u, a.up, a.w}, t, ck, st);
+}
+
 int ot4_fwd_step(ckfwi_model* m, const FwdArgs& a, const Tile& t, int ck, cudaStream_t st)
 {
     const FieldGeom& f = m->fg;
+    if (t.ver == 10) return ot4q_update(m, a, t, ck, st, nullptr, nullptr);
     Ot4LapArgs la{};
     la.g = f;
     la.f0 = a.u;
@@ -885,6 +932,34 @@ int ot4_fwd_step(ckfwi_model* m, const FwdArgs& a, const Tile& t, int ck, cudaSt
 int ot4_adj_step(ckfwi_model* m, const AdjArgs& a, const Tile& t, int utype, int j, cudaStream_t st)
 {
     const FieldGeom& f = m->fg;
+    if (t.ver == 10) {
+        const float* u = static_cast<const float*>(a.u);
+        float* zu = org(m->z4[1 + (j & 1)], f);
+        FwdArgs la{};
+        la.g = f;
+        la.u = a.l1;
+        la.up = a.l2;
+        la.w = a.w;
+        la.out = a.l0;
+        la.eta = a.eta;
+        la.hdt = a.hdt;
+        std::memcpy(la.c, m->c, sizeof(la.c));
+        la.src = a.adj;
+        la.err = a.err;
+        la.wait_limit = a.wait_limit;
+        ST_TRY(ot4q_update(m, la, t, CK_NONE, st, j < m->g.nt ? org(m->z4[1 + ((j + 1) & 1)], f) : nullptr, a.gacc));
+        Ot4qArgs q{};
+        q.f = la;
+        q.f.src = a.src;
+        q.s = u;
+        q.f.out = zu;
+        q.lap = org(m->z4[0], f);          // Z_l is read by now
+        q.gacc = a.gacc;
+        std::memcpy(q.c12, m->c12, sizeof(q.c12));
+        ST_TRY(ot4q_pass(m, OT4Q_LAP_U, q, {a.w}, t, CK_NONE, st));
+        q.s = zu;
+        return ot4q_pass(m, OT4Q_GRAD, q, {q.lap, a.l0, a.gacc}, t, CK_NONE, st);
+    }
     // pass 1: Z_l, Z_u(j), and the deferred term of step j + 1
     Ot4LapArgs la{};
     la.g = f;
@@ -1023,7 +1098,7 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
         } else if (m->tf.ver == 7) {
             CK_TRY(launch_fwd5(a, m->tf, m->K, ck, cx.st));
         } else if (m->tf.ver >= 5) {
-            ST_TRY(ot4_fwd_step(m, a, m->tf, ck, cx.st));
+            ST_TRY(ot4_fwd_step(m, a, in_host(m, u) || in_host(m, up) ? ot4_host_tile(m->tf) : m->tf, ck, cx.st));
             ++cx.launches;
         } else if (m->tf.ver == 2 && in_host(m, u)) {
             CK_TRY(launch_fwd(a, host_tile(m), m->K, ck, cx.st));
@@ -1338,8 +1413,9 @@ int adj_step(Ctx& cx, const Role& l1, const Role& l2, const Role& l0, const Role
         } else if (m->ta.ver == 7) {
             CK_TRY(launch_adj5(a, m->ta, m->K, utype, cx.st));
         } else if (m->ta.ver >= 5) {
-            ST_TRY(ot4_adj_step(m, a, m->ta, utype, j, cx.st));
-            cx.launches += 2;
+            const Tile t = utype != U_FP32 || in_host(m, u) ? ot4_host_tile(m->ta) : m->ta;
+            ST_TRY(ot4_adj_step(m, a, t, utype, j, cx.st));
+            cx.launches += t.ver == 10 ? 3 : 2;
         } else if (m->ta.ver == 2 && in_host(m, u)) {
             CK_TRY(launch_adj(a, host_tile(m), m->K, utype, cx.st));
         } else if (m->ta.ver == 4) {
@@ -1493,6 +1569,12 @@ int autotune(ckfwi_model* m, cudaStream_t st)
             for (int z : zlens(cols)) {
                 t0.zlen = z;
                 cands.push_back(t0);
+                Tile tq = t0;                    // fed by tensor copies
+                tq.ver = 10;
+                for (int pf : {1, 2}) {
+                    tq.pf = pf;
+                    if (encode_fn() && ot4q_supported(f.dims, m->K, tq)) cands.push_back(tq);
+                }
             }
         }
     }
@@ -1610,8 +1692,9 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         if (nf < 4 || u.zlen < 1) return false;
         if (nf < 5) u.vec = 1;
         if (nf < 6) u.pf = 0;
-        if ((u.ver == 5 || u.ver == 6) != (m->ot == 4)) return false;
-        const bool okv = u.ver == 9   ? m->ot == 2 && step2_supported(f.dims, m->K, u, reverse) && tiles_of(f, u) <= nsm
+        if ((u.ver == 5 || u.ver == 6 || u.ver == 10) != (m->ot == 4)) return false;
+        const bool okv = u.ver == 10  ? encode_fn() && ot4q_supported(f.dims, m->K, u) && v3_fits(f, m->K)
+                         : u.ver == 9 ? m->ot == 2 && step2_supported(f.dims, m->K, u, reverse) && tiles_of(f, u) <= nsm
                          : u.ver == 8 ? tma_ok && tq_supported(f.dims, m->K, u) && v3_fits(f, m->K)
                          : u.ver == 7 ? v5_supported(f.dims, m->K, u) && v3_fits(f, m->K)
                          : u.ver == 6 ? ot4v_supported(f.dims, m->K, u, reverse) && v3_fits(f, m->K)
@@ -1684,6 +1767,49 @@ int autotune(ckfwi_model* m, cudaStream_t st)
                 (pass == 0 ? m->tf : m->ta) = t;
             }
         }
+    }
+    // The OT4 passes fed by tensor copies hold different numbers of CTAs an SM
+    // (three point fields against one), so each takes its own z run and
+    // prefetch: at 208^3 one run for all left the passes at 1.6 and 1.9 waves
+    // (forward 72.6 us, reverse 156.7 us a step).
+    if ((m->tf.ver == 10 && !ff) || (m->ta.ver == 10 && !fa)) {
+        Ot4qArgs q{};
+        q.f = a;
+        q.f.out = org(m->z4[0], f);
+        q.s = a.u;
+        q.lap = org(m->z4[1], f);
+        q.gacc = b.gacc;
+        std::memcpy(q.c12, m->c12, sizeof(q.c12));
+        Tile best[5];
+        for (int op = 0; op < 5; ++op) {
+            float bt = 1e30f;
+            for (const Tile& t : cands) {
+                if (t.ver != 10) continue;
+                m->t4[op] = t;
+                std::vector<float> v;
+                for (int r = 0; r < 4; ++r) {           // the first untimed
+                    CK_TRY(cudaEventRecord(e0, st));
+                    for (int k = 0; k < reps; ++k) {
+                        if (op == OT4Q_LAP || op == OT4Q_LAP_U) ST_TRY(ot4q_pass(m, op, q, {a.w}, t, CK_NONE, st));
+                        else ST_TRY(ot4q_pass(m, op, q, {a.w, a.up, b.gacc}, t, CK_NONE, st));
+                    }
+                    CK_TRY(cudaEventRecord(e1, st));
+                    CK_TRY(cudaEventSynchronize(e1));
+                    float ms = 0;
+                    CK_TRY(cudaEventElapsedTime(&ms, e0, e1));
+                    if (r) v.push_back(ms);
+                }
+                std::sort(v.begin(), v.end());
+                if (v[1] < bt) {
+                    bt = v[1];
+                    best[op] = t;
+                }
+            }
+            if (verbose)
+                std::fprintf(stderr, "ckfwi autotune OT4 pass %d zlen %d pf %d: %.1f us\n", op, best[op].zlen, best[op].pf,
+                             1000.0f * bt / reps);
+        }
+        for (int op = 0; op < 5; ++op) m->t4[op] = best[op];
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

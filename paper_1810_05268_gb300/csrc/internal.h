@@ -159,6 +159,18 @@ struct Step2Args {
     float* gacc;
 };
 
+// One pass of an OT4 step fed by tensor copies (ot4_tq.cu): s the staged
+// field; f.out the pass's result (Z, or the next level), f.src, f.smp, f.eta,
+// f.ck_* as the pass needs them; lap: where pass 3 leaves lap u.
+enum { OT4Q_LAP, OT4Q_LAP_LAM, OT4Q_LAP_U, OT4Q_UPDATE, OT4Q_GRAD };
+struct Ot4qArgs {
+    FwdArgs f;
+    const float* s;
+    float* lap;
+    float* gacc;
+    float c12[MAXK + 1];
+};
+
 enum CkMode { CK_NONE = 0, CK_FP32 = 1, CK_BF16 = 2, CK_FP16 = 3 };
 enum UType { U_FP32 = 0, U_BF16 = 1, U_FP16 = 2 };
 
@@ -172,7 +184,7 @@ struct Tile {
                           // OT2 kernels (3D, one or two planes per step), 8: the
                           // forward step fed by tensor copies and the reverse step split
                           // in two launches (3D), 9: many steps a launch (2D; bx x zlen
-                          // points a tile)
+                          // points a tile), 10: the OT4 passes fed by tensor copies (3D)
     int vec = 1;          // ver 3, 4: x points per thread (2 or 4)
     int pf = 0;           // ver 4: planes of prefetch (0 = the default, 2); ver 7: planes per step (1, 2);
                           // ver 8: planes of prefetch (1, 2; 0 reads as 1)
@@ -266,6 +278,10 @@ cudaError_t launch_fwdq(const FwdArgs& a, const CUtensorMap& tu, const CUtensorM
 // gradient half (maps 3-5: u^{j-1} with the u box, lam^{j-1} and g with
 // point boxes); FP32 u^{j-1} only
 cudaError_t launch_adjq(const AdjArgs& a, const CUtensorMap* maps, const Tile& t, int K, cudaStream_t s);
+// ot4_tq.cu: OT4 passes fed by tensor copies (Tile.ver 10; maps: the staged
+// field with the u box, then the pass's point fields with 32 x 16 boxes)
+bool ot4q_supported(int dims, int K, const Tile& t);
+cudaError_t launch_ot4q(int op, const Ot4qArgs& A, const CUtensorMap* maps, const Tile& t, int K, int ck, cudaStream_t s);
 
 // aux.cu
 cudaError_t launch_sample(const float* u, const Sample& smp, cudaStream_t s);

@@ -61,35 +61,6 @@ struct VStage {
     }
 };
 
-// leapfrog4() for a pair of points: c + ((1 - e)(c - p) + Z + w s) / (1 + e).
-// The product (1 - e)(c - p) is formed with the scalar __fmul_rn, which is
-// never merged into a multiply-add: the packed multiply feeding the packed
-// addition of Z was contracted into one FFMA2, whose single rounding differs
-// from the two of the scalar kernels inside the damping layer (1 - e != 1).
-__device__ __forceinline__ float2 leap4v(float2 c, float2 p, float2 w, float2 zc, float2 s, float2 eta, float hdt)
-{
-    const float2 be = __ffma2_rn(f2(-eta.x, -eta.y), f2(hdt, hdt), f2(1.0f, 1.0f));
-    const float2 d = __ffma2_rn(p, f2(-1.0f, -1.0f), c);
-    const float2 bd = f2(__fmul_rn(be.x, d.x), __fmul_rn(be.y, d.y));
-    float2 t = __ffma2_rn(w, s, __fadd2_rn(zc, bd));
-    t.x = eta.x != 0.0f ? __fdividef(t.x, __fmaf_rn(eta.x, hdt, 1.0f)) : t.x;
-    t.y = eta.y != 0.0f ? __fdividef(t.y, __fmaf_rn(eta.y, hdt, 1.0f)) : t.y;
-    return __fadd2_rn(c, t);
-}
-
-// store V values at offset o of a row whose first vector point is x0
-template <int V>
-__device__ __forceinline__ void vput(float* p, long long o, const float (&v)[V], bool full, int x0, int nx)
-{
-    if (full) {
-        vst<V>(p + o, v);
-    } else {
-#pragma unroll
-        for (int i = 0; i < V; ++i)
-            if (x0 + i < nx) p[o + i] = v[i];
-    }
-}
-
 // Common per-thread geometry of a vector-blocked step.
 struct Pos3 {
     int tx, ty, nz, ny, nx, px, pxy, x0, y, col, xb;
