@@ -760,6 +760,13 @@ struct Ctx {
     std::vector<FwdArgs> ftab;      // one row per lane and step, in launch order
     std::vector<AdjArgs> atab;
     std::vector<Step2Args> stab;    // rows of the launches of several 2D steps
+    // batched tensor-copy steps: the lanes' tensor maps (a row's tm is 1 +
+    // the map's place until the table is on the device), and the rows of the
+    // reverse steps' lambda halves
+    std::vector<CUtensorMap> maps;
+    std::map<std::tuple<const void*, int>, size_t> map_at;
+    std::vector<FwdArgs> qtab;
+    const FwdArgs* qtab_d = nullptr;
     size_t fi = 0, ai = 0, si = 0;  // next row
     const Step2Args* stab_d = nullptr;
     const CodecLane* ctab_d = nullptr;   // the lanes' codec sides
@@ -1027,6 +1034,43 @@ int fwd_steps2(Ctx& cx, const Role& u, const Role& up, int n, int T, bool record
 int adj_steps2(Ctx& cx, const Role& l1, const Role& l2, const Role& o0, const Role& o1, const Role* us, const int* uts,
                int j, int T);
 
+int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by, CUtensorMap* out);
+
+// place (1, 2, ..) of a field's map in the context's table, as a row's tm
+// holds it before the upload; staged: with the u box, else a point box
+int map_place(Ctx& cx, ckfwi_model* m, const void* field, bool staged, const void** tm)
+{
+    const auto key = std::make_tuple(field, staged ? 1 : 0);
+    auto it = cx.map_at.find(key);
+    if (it == cx.map_at.end()) {
+        CUtensorMap t;
+        ST_TRY(tensor_map(m, field, U_FP32, staged ? tq_box_x(m->K) : 32, staged ? tq_box_y(m->K) : 16, &t));
+        cx.maps.push_back(t);
+        it = cx.map_at.emplace(key, cx.maps.size()).first;
+    }
+    *tm = reinterpret_cast<const void*>(it->second);
+    return CKFWI_OK;
+}
+int fwd_places(Ctx& cx, ckfwi_model* m, FwdArgs* a)
+{
+    ST_TRY(map_place(cx, m, a->u, true, &a->tm[0]));
+    ST_TRY(map_place(cx, m, a->up, false, &a->tm[1]));
+    return map_place(cx, m, a->w, false, &a->tm[2]);
+}
+int grad_places(Ctx& cx, ckfwi_model* m, AdjArgs* a)
+{
+    ST_TRY(map_place(cx, m, a->u, true, &a->tm[0]));
+    ST_TRY(map_place(cx, m, a->l0, false, &a->tm[1]));
+    return map_place(cx, m, a->gacc, false, &a->tm[2]);
+}
+template <class A>
+void place_maps(std::vector<A>& rows, const CUtensorMap* base)
+{
+    for (A& a : rows)
+        for (const void*& p : a.tm)
+            if (p) p = base + (reinterpret_cast<size_t>(p) - 1);
+}
+
 int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, bool record, int ck,
              const Role& ck_u, const Role& ck_up)
 {
@@ -1077,6 +1121,7 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
         }
         if (cx.batch) {
             a.zlen = zlen;
+            if (!cx.issue && cx.bf.ver == 8) ST_TRY(fwd_places(cx, m, &a));
             if (!cx.issue) cx.ftab.push_back(a);
             continue;
         }
@@ -1120,7 +1165,8 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
         if (cx.issue) {
             const int tok = cx.begin(PC_FWD);
             BatchLaunch<FwdArgs> b{cx.ftab_d + cx.fi, cx.fstart_d, NL, cx.m->fg.dims, cx.fblocks};
-            if (cx.bf.ver == 7) CK_TRY(launch_fwd5_batch(b, cx.bf, cx.m->K, ck, cx.st));
+            if (cx.bf.ver == 8) CK_TRY(launch_fwdq_batch(b, cx.bf, cx.m->K, ck, cx.st));
+            else if (cx.bf.ver == 7) CK_TRY(launch_fwd5_batch(b, cx.bf, cx.m->K, ck, cx.st));
             else if (cx.bf.ver == 4) CK_TRY(launch_fwd4_batch(b, cx.bf, cx.m->K, ck, cx.st));
             else if (cx.bf.ver == 3) CK_TRY(launch_fwd3_batch(b, cx.bf, cx.m->K, ck, cx.st));
             else CK_TRY(launch_fwd_batch(b, cx.bf, cx.m->K, ck, cx.st));
@@ -1395,6 +1441,12 @@ int adj_step(Ctx& cx, const Role& l1, const Role& l2, const Role& l0, const Role
         a.src.series = m->shot.wavelet.as<float>() + (j - 1);
         if (cx.batch) {
             a.zlen = cx.za[l];
+            if (!cx.issue && cx.ba.ver == 8) {
+                FwdArgs f = lam_args(a);
+                ST_TRY(fwd_places(cx, m, &f));
+                cx.qtab.push_back(f);
+                if (utype == U_FP32) ST_TRY(grad_places(cx, m, &a));
+            }
             if (!cx.issue) cx.atab.push_back(a);
             continue;
         }
@@ -1438,7 +1490,17 @@ int adj_step(Ctx& cx, const Role& l1, const Role& l2, const Role& l0, const Role
         if (cx.issue) {
             const int tok = cx.begin(PC_ADJ);
             BatchLaunch<AdjArgs> b{cx.atab_d + cx.ai, cx.astart_d, NL, cx.m->fg.dims, cx.ablocks};
-            if (cx.ba.ver == 7) CK_TRY(launch_adj5_batch(b, cx.ba, cx.m->K, utype, cx.st));
+            if (cx.ba.ver == 8 && utype == U_FP32) {
+                const BatchLaunch<FwdArgs> q{cx.qtab_d + cx.ai, cx.astart_d, NL, cx.m->fg.dims, cx.ablocks};
+                CK_TRY(launch_adjq_batch(q, b, cx.ba, cx.m->K, cx.st));
+                ++cx.launches;
+            } else if (cx.ba.ver == 8) {
+                // tensor maps cover FP32 fields only: the lean kernel of the same tile
+                Tile t7 = cx.ba;
+                t7.ver = 7;
+                t7.pf = 1;
+                CK_TRY(launch_adj5_batch(b, t7, cx.m->K, utype, cx.st));
+            } else if (cx.ba.ver == 7) CK_TRY(launch_adj5_batch(b, cx.ba, cx.m->K, utype, cx.st));
             else if (cx.ba.ver == 3) CK_TRY(launch_adj3_batch(b, cx.ba, cx.m->K, utype, cx.st));
             else CK_TRY(launch_adj_batch(b, cx.ba, cx.m->K, utype, cx.st));
             cx.end(tok);
@@ -2820,6 +2882,12 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
             t7.pf = np;
             if (v5_supported(dims, K, t7)) shapes.push_back(t7);
         }
+        Tile t8 = t;                     // fed by tensor copies, one or two planes ahead
+        t8.ver = 8;
+        for (int pf : {1, 2}) {
+            t8.pf = pf;
+            if (encode_fn() && tq_supported(dims, K, t8)) shapes.push_back(t8);
+        }
     }
     // CKFWI_BATCH_VER restricts the timed candidates to one generation
     // (tests); generation 4 has no batched reverse step, which then takes
@@ -2834,6 +2902,20 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
             nzmax = std::max(nzmax, L->fg.nz);
         }
         std::vector<std::vector<int>> seen;
+        // the tensor-copy kernels also with runs of about the same length on
+        // every lane: lanes of 120 to 229 planes cut into equally many runs
+        // leave the short ones' SMs idle (windows of 1.7 to 15.5 M points:
+        // 170 us a forward step)
+        for (int zt = 16; t.ver == 8 && zt <= 96; zt += zt < 48 ? 4 : 16) {
+            std::vector<int> z(NL);
+            for (int l = 0; l < NL; ++l) {
+                const int nz = lanes[l]->fg.nz, runs = std::max(1, (nz + zt / 2) / zt);
+                z[l] = std::max(4, (nz + runs - 1) / runs);
+            }
+            if (std::find(seen.begin(), seen.end(), z) != seen.end()) continue;
+            seen.push_back(z);
+            cands.push_back(Cand{t, z});
+        }
         for (int target : {1, 2, 4, 8, 16}) {
             long long nzc = (target * (long long)nsm + cols - 1) / cols;
             nzc = std::max<long long>(1, std::min<long long>(nzc, nzmax));
@@ -2867,7 +2949,24 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
         aa[l].src = L->shot.src.view;
         aa[l].src.series = L->shot.wavelet.as<float>();
     }
-    DevMem dtab, dst;
+    // the tensor-copy kernels' maps, and the rows of their lambda half
+    DevMem dtab, dst, dmap, dlam;
+    std::vector<FwdArgs> la(NL);
+    Ctx mc{m0, st, 0};
+    if (fits3 && encode_fn()) {
+        for (int l = 0; l < NL; ++l) {
+            la[l] = lam_args(aa[l]);
+            ST_TRY(fwd_places(mc, lanes[l], &fa[l]));
+            ST_TRY(fwd_places(mc, lanes[l], &la[l]));
+            ST_TRY(grad_places(mc, lanes[l], &aa[l]));
+        }
+        CK_TRY(dmap.alloc(sizeof(CUtensorMap) * mc.maps.size(), false));
+        CK_TRY(cudaMemcpy(dmap.p, mc.maps.data(), sizeof(CUtensorMap) * mc.maps.size(), cudaMemcpyHostToDevice));
+        place_maps(fa, dmap.as<CUtensorMap>());
+        place_maps(la, dmap.as<CUtensorMap>());
+        place_maps(aa, dmap.as<CUtensorMap>());
+    }
+    CK_TRY(dlam.alloc(sizeof(FwdArgs) * NL, false));
     CK_TRY(dtab.alloc(sizeof(FwdArgs) * NL + sizeof(AdjArgs) * NL + 256, false));
     CK_TRY(dst.alloc(sizeof(int) * (NL + 1), false));
     FwdArgs* ftab = dtab.as<FwdArgs>();
@@ -2896,8 +2995,10 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
         for (int l = 0; l < NL; ++l) {
             fa[l].zlen = c.z[l];
             aa[l].zlen = c.z[l];
+            la[l].zlen = c.z[l];
         }
-        if (cudaMemcpy(ftab, fa.data(), sizeof(FwdArgs) * NL, cudaMemcpyHostToDevice) != cudaSuccess ||
+        if (cudaMemcpy(dlam.p, la.data(), sizeof(FwdArgs) * NL, cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(ftab, fa.data(), sizeof(FwdArgs) * NL, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(atab, aa.data(), sizeof(AdjArgs) * NL, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(dst.p, s.data(), sizeof(int) * (NL + 1), cudaMemcpyHostToDevice) != cudaSuccess) {
             rs = CKFWI_ECUDA;
@@ -2910,6 +3011,9 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
             auto go = [&]() {
                 const BatchLaunch<FwdArgs> bf{ftab, dst.as<int>(), NL, dims, total};
                 const BatchLaunch<AdjArgs> ba{atab, dst.as<int>(), NL, dims, total};
+                const BatchLaunch<FwdArgs> bq{dlam.as<FwdArgs>(), dst.as<int>(), NL, dims, total};
+                if (c.t.ver == 8)
+                    return pass == 0 ? launch_fwdq_batch(bf, c.t, K, CK_NONE, st) : launch_adjq_batch(bq, ba, c.t, K, st);
                 if (c.t.ver == 7)
                     return pass == 0 ? launch_fwd5_batch(bf, c.t, K, CK_NONE, st)
                                      : launch_adj5_batch(ba, c.t, K, U_FP32, st);
@@ -3013,6 +3117,14 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
     cx.batch = true;
     cx.bf = bt->tf;
     cx.ba = bt->ta;
+    // tensor maps cover device memory only: with host slots the lean kernels
+    // of the same tiles
+    for (ckfwi_model* L : lanes)
+        for (Tile* t : {&cx.bf, &cx.ba})
+            if (L->host_slots > 0 && t->ver == 8) {
+                t->ver = 7;
+                t->pf = 1;
+            }
     cx.zf = bt->zf;
     cx.za = bt->za;
     std::vector<int> fs = lane_starts(lanes, cx.bf, cx.zf, &cx.fblocks);
@@ -3059,10 +3171,23 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
         const size_t ab = ((sizeof(AdjArgs) * cx.atab.size() + 255) / 256) * 256;
         const size_t sb = sizeof(int) * (fs.size() + as.size());
         const size_t s2 = ((sizeof(Step2Args) * cx.stab.size() + 255) / 256) * 256;
+        const size_t tb = (sizeof(CUtensorMap) * cx.maps.size() + 255) / 256 * 256;
+        const size_t qb = ((sizeof(FwdArgs) * cx.qtab.size() + 255) / 256) * 256;
         std::vector<CodecLane> ctab;
         for (int l = 0; rc.codec && l < NL; ++l) ctab.push_back(codec_lane(lanes[l]));
         const size_t so = (sb + 255) / 256 * 256;
-        int rs = cuda_status_or_ok(tabs.alloc(fb + ab + so + s2 + sizeof(CodecLane) * ctab.size(), false));
+        int rs = cuda_status_or_ok(tabs.alloc(fb + ab + so + s2 + tb + qb + sizeof(CodecLane) * ctab.size(), false));
+        // the maps (after s2, 256-byte aligned: whole rows before them), then
+        // the rows that name them
+        char* const tmaps_d = tabs.as<char>() + fb + ab + so + s2;
+        place_maps(cx.ftab, reinterpret_cast<const CUtensorMap*>(tmaps_d));
+        place_maps(cx.atab, reinterpret_cast<const CUtensorMap*>(tmaps_d));
+        place_maps(cx.qtab, reinterpret_cast<const CUtensorMap*>(tmaps_d));
+        if (rs == CKFWI_OK && tb)
+            rs = cuda_status_or_ok(cudaMemcpy(tmaps_d, cx.maps.data(), sizeof(CUtensorMap) * cx.maps.size(), cudaMemcpyHostToDevice));
+        if (rs == CKFWI_OK && !cx.qtab.empty())
+            rs = cuda_status_or_ok(cudaMemcpy(tmaps_d + tb, cx.qtab.data(),
+                                              sizeof(FwdArgs) * cx.qtab.size(), cudaMemcpyHostToDevice));
         if (rs == CKFWI_OK && !cx.ftab.empty())
             rs = cuda_status_or_ok(cudaMemcpy(tabs.p, cx.ftab.data(), sizeof(FwdArgs) * cx.ftab.size(),
                                               cudaMemcpyHostToDevice));
@@ -3075,7 +3200,7 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
             rs = cuda_status_or_ok(
                 cudaMemcpy(tabs.as<char>() + fb + ab, starts.data(), sb, cudaMemcpyHostToDevice));
         if (rs == CKFWI_OK && !ctab.empty())
-            rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so + s2, ctab.data(),
+            rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so + s2 + tb + qb, ctab.data(),
                                               sizeof(CodecLane) * ctab.size(), cudaMemcpyHostToDevice));
         if (rs == CKFWI_OK && !cx.stab.empty())
             rs = cuda_status_or_ok(cudaMemcpy(tabs.as<char>() + fb + ab + so, cx.stab.data(),
@@ -3085,8 +3210,9 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
             return rs;
         }
         cx.stab_d = reinterpret_cast<const Step2Args*>(tabs.as<char>() + fb + ab + so);
-        cx.ctab_d = reinterpret_cast<const CodecLane*>(tabs.as<char>() + fb + ab + so + s2);
+        cx.ctab_d = reinterpret_cast<const CodecLane*>(tmaps_d + tb + qb);
         cx.ftab_d = tabs.as<FwdArgs>();
+        cx.qtab_d = reinterpret_cast<const FwdArgs*>(tmaps_d + tb);
         cx.atab_d = reinterpret_cast<const AdjArgs*>(tabs.as<char>() + fb);
         cx.fstart_d = reinterpret_cast<const int*>(tabs.as<char>() + fb + ab);
         cx.astart_d = cx.fstart_d + fs.size();

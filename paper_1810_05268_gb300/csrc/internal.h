@@ -67,6 +67,7 @@ struct FwdArgs {
     void* ck_up;
     int* err;             // error flags (bit 0: FP16 overflow, bit 3: a bounded wait ran out)
     long long wait_limit; // TMA kernels: back-off rounds of a plane's bounded wait (< 0: give up at once)
+    const void* tm[3];    // batched tensor-copy kernels: the tensor maps of u, up, w (device memory)
 };
 
 // Fused reverse step:
@@ -88,6 +89,7 @@ struct AdjArgs {
     Inj src;              // Q^T s^{j-1}
     int* err;             // error flags (bit 3: a bounded wait ran out)
     long long wait_limit; // TMA kernels: back-off rounds of a plane's bounded wait (< 0: give up at once)
+    const void* tm[3];    // batched tensor-copy kernels: the tensor maps of u, l0, gacc (device memory)
 };
 
 // OT4 kernel (Sec. 6): a forward step is two passes, Z = w lap f and then the
@@ -278,6 +280,12 @@ cudaError_t launch_fwdq(const FwdArgs& a, const CUtensorMap& tu, const CUtensorM
 // gradient half (maps 3-5: u^{j-1} with the u box, lam^{j-1} and g with
 // point boxes); FP32 u^{j-1} only
 cudaError_t launch_adjq(const AdjArgs& a, const CUtensorMap* maps, const Tile& t, int K, cudaStream_t s);
+FwdArgs lam_args(const AdjArgs& a);
+// batched forms (every lane's geometry must pass v3_fits and have its first
+// column at PX; rows carry their maps' addresses)
+cudaError_t launch_fwdq_batch(const BatchLaunch<FwdArgs>& b, const Tile& t, int K, int ck, cudaStream_t s);
+cudaError_t launch_adjq_batch(const BatchLaunch<FwdArgs>& lam, const BatchLaunch<AdjArgs>& b, const Tile& t, int K,
+                              cudaStream_t s);
 // ot4_tq.cu: OT4 passes fed by tensor copies (Tile.ver 10; maps: the staged
 // field with the u box, then the pass's point fields with 32 x 16 boxes)
 bool ot4q_supported(int dims, int K, const Tile& t);

@@ -38,10 +38,11 @@ namespace {
 // prefetch (31 KB of shared memory), five with two (39 KB)
 template <int K, int PF> constexpr int tq_min_blocks() { return K <= 4 ? (PF == 1 ? 6 : 5) : 1; }
 
+// Body of the forward step for CTA (bxi, byi, bzi) of a grid of gx x gy CTAs a
+// plane (one shot's, or one lane's of a batch)
 template <int K, int PF, int CK>
-__global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
-    fwdq_kernel(const FwdArgs a, const __grid_constant__ CUtensorMap tmu, const __grid_constant__ CUtensorMap tmp,
-                const __grid_constant__ CUtensorMap tmw)
+__device__ __forceinline__ void fwdq_body(const FwdArgs& a, const CUtensorMap* tmu, const CUtensorMap* tmp,
+                                          const CUtensorMap* tmw, int bxi, int byi, int bzi, int gx, int gy)
 {
     using Q = TQ<K, PF>;
     using G = typename Q::G;
@@ -54,7 +55,6 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
     float* wr = upr + RP * Q::PT;
     uint64_t* bar = reinterpret_cast<uint64_t*>(wr + RP * Q::PT);
 
-    const int bxi = blockIdx.x, byi = blockIdx.y, bzi = blockIdx.z;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nz = a.g.nz, ny = a.g.ny, nx = a.g.nx;
     const int px = (int)a.g.px, pxy = (int)a.g.pxy;
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
     const int y = yb + ty;
 
     if (a.smp.n > 0) {   // receiver sampling of u^n by the first threads of the grid
-        const int gt = ((bzi * gridDim.y + byi) * gridDim.x + bxi) * (TX * TY) + tid;
+        const int gt = ((bzi * gy + byi) * gx + bxi) * (TX * TY) + tid;
         if (gt < a.smp.n) {
             float acc = 0.0f;
             for (int i = 0; i < a.smp.nst; ++i)
@@ -98,11 +98,11 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
         uint64_t* b = bar + g % RU;
         const bool pts = g >= K;
         bar_expect(b, Q::UBYTES + (pts ? 2 * Q::PBYTES : 0));
-        tile3(ring + (g % RU) * Q::US, &tmu, xb, yb, min(z0 + g, zqmax) + K, b);
+        tile3(ring + (g % RU) * Q::US, tmu, xb, yb, min(z0 + g, zqmax) + K, b);
         if (pts) {
             const int zp = min(z0 + g - K, z1 - 1) + K, s = (g - K) % RP;
-            tile3(upr + s * Q::PT, &tmp, xb + G::PX, yb + K, zp, b);
-            tile3(wr + s * Q::PT, &tmw, xb + G::PX, yb + K, zp, b);
+            tile3(upr + s * Q::PT, tmp, xb + G::PX, yb + K, zp, b);
+            tile3(wr + s * Q::PT, tmw, xb + G::PX, yb + K, zp, b);
         }
     };
     auto wait_group = [&](int g) { return bar_wait(bar + g % RU, (unsigned)((g / RU) & 1), rounds); };
@@ -206,6 +206,36 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
 }
 
 template <int K, int PF, int CK>
+__global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
+    fwdq_kernel(const FwdArgs a, const __grid_constant__ CUtensorMap tmu, const __grid_constant__ CUtensorMap tmp,
+                const __grid_constant__ CUtensorMap tmw)
+{
+    fwdq_body<K, PF, CK>(a, &tmu, &tmp, &tmw, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y);
+}
+
+// Batched: a lane's maps lie in device memory (a.tm), written by the host
+// before the launch; the fence orders those writes before the copies' reads
+// of the maps.
+template <class A>
+__device__ __forceinline__ const CUtensorMap* lane_map(const A& a, int k)
+{
+    const CUtensorMap* m = static_cast<const CUtensorMap*>(a.tm[k]);
+    if (threadIdx.x == 0 && threadIdx.y == 0)
+        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(m) : "memory");
+    return m;
+}
+
+template <int K, int PF, int CK>
+__global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
+    fwdq_batch_kernel(const FwdArgs* __restrict__ tab, const int* __restrict__ start, int nl)
+{
+    __shared__ __align__(16) FwdArgs a;
+    const int b = stage_args(a, tab, start, nl);
+    const int gx = (a.g.nx + 31) / 32, gy = (a.g.ny + 15) / 16;
+    fwdq_body<K, PF, CK>(a, lane_map(a, 0), lane_map(a, 1), lane_map(a, 2), b % gx, (b / gx) % gy, b / (gx * gy), gx, gy);
+}
+
+template <int K, int PF, int CK>
 cudaError_t fwdq_go(const FwdArgs& a, const CUtensorMap& tu, const CUtensorMap& tp, const CUtensorMap& tw,
                     cudaStream_t s)
 {
@@ -247,9 +277,8 @@ cudaError_t fwdq_p(const FwdArgs& a, const CUtensorMap& tu, const CUtensorMap& t
 // the same Laplacian and injection order and one packed FMA, so g is
 // bitwise theirs.
 template <int K, int PF>
-__global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
-    gradq_kernel(const AdjArgs a, const __grid_constant__ CUtensorMap tmu, const __grid_constant__ CUtensorMap tml,
-                 const __grid_constant__ CUtensorMap tmg)
+__device__ __forceinline__ void gradq_body(const AdjArgs& a, const CUtensorMap* tmu, const CUtensorMap* tml,
+                                           const CUtensorMap* tmg, int bxi, int byi, int bzi)
 {
     using Q = TQ<K, PF>;
     using G = typename Q::G;
@@ -262,7 +291,6 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
     float* gr = lr + RP * Q::PT;
     uint64_t* bar = reinterpret_cast<uint64_t*>(gr + RP * Q::PT);
 
-    const int bxi = blockIdx.x, byi = blockIdx.y, bzi = blockIdx.z;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int nz = a.g.nz, ny = a.g.ny, nx = a.g.nx;
     const int px = (int)a.g.px, pxy = (int)a.g.pxy;
@@ -289,11 +317,11 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
         uint64_t* b = bar + g % RU;
         const bool pts = g >= K;
         bar_expect(b, Q::UBYTES + (pts ? 2 * Q::PBYTES : 0));
-        tile3(ring + (g % RU) * Q::US, &tmu, xb, yb, min(z0 + g, zqmax) + K, b);
+        tile3(ring + (g % RU) * Q::US, tmu, xb, yb, min(z0 + g, zqmax) + K, b);
         if (pts) {
             const int zp = min(z0 + g - K, z1 - 1) + K, sl = (g - K) % RP;
-            tile3(lr + sl * Q::PT, &tml, xb + G::PX, yb + K, zp, b);
-            tile3(gr + sl * Q::PT, &tmg, xb + G::PX, yb + K, zp, b);
+            tile3(lr + sl * Q::PT, tml, xb + G::PX, yb + K, zp, b);
+            tile3(gr + sl * Q::PT, tmg, xb + G::PX, yb + K, zp, b);
         }
     };
     auto wait_group = [&](int g) { return bar_wait(bar + g % RU, (unsigned)((g / RU) & 1), rounds); };
@@ -372,6 +400,56 @@ __global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
 }
 
 template <int K, int PF>
+__global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
+    gradq_kernel(const AdjArgs a, const __grid_constant__ CUtensorMap tmu, const __grid_constant__ CUtensorMap tml,
+                 const __grid_constant__ CUtensorMap tmg)
+{
+    gradq_body<K, PF>(a, &tmu, &tml, &tmg, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+template <int K, int PF>
+__global__ void __launch_bounds__(128, tq_min_blocks<K, PF>())
+    gradq_batch_kernel(const AdjArgs* __restrict__ tab, const int* __restrict__ start, int nl)
+{
+    __shared__ __align__(16) AdjArgs a;
+    const int b = stage_args(a, tab, start, nl);
+    const int gx = (a.g.nx + 31) / 32, gy = (a.g.ny + 15) / 16;
+    gradq_body<K, PF>(a, lane_map(a, 0), lane_map(a, 1), lane_map(a, 2), b % gx, (b / gx) % gy, b / (gx * gy));
+}
+
+template <int K, int PF, int CK>
+cudaError_t fwdqb_ck(const BatchLaunch<FwdArgs>& b, cudaStream_t s)
+{
+    using Q = TQ<K, PF>;
+    cudaError_t e = cudaFuncSetAttribute(fwdq_batch_kernel<K, PF, CK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SMEM);
+    if (e != cudaSuccess) return e;
+    fwdq_batch_kernel<K, PF, CK><<<dim3((unsigned)b.blocks), dim3(Q::TX, Q::TY), Q::SMEM, s>>>(b.tab, b.start, b.lanes);
+    return cudaGetLastError();
+}
+
+template <int K, int PF>
+cudaError_t fwdqb_go(const BatchLaunch<FwdArgs>& b, int ck, cudaStream_t s)
+{
+    switch (ck) {
+    case CK_NONE: return fwdqb_ck<K, PF, CK_NONE>(b, s);
+    case CK_FP32: return fwdqb_ck<K, PF, CK_FP32>(b, s);
+    case CK_BF16: return fwdqb_ck<K, PF, CK_BF16>(b, s);
+    case CK_FP16: return fwdqb_ck<K, PF, CK_FP16>(b, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+template <int K, int PF>
+cudaError_t gradqb_go(const BatchLaunch<AdjArgs>& b, cudaStream_t s)
+{
+    using Q = TQ<K, PF>;
+    cudaError_t e = cudaFuncSetAttribute(gradq_batch_kernel<K, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SMEM);
+    if (e != cudaSuccess) return e;
+    gradq_batch_kernel<K, PF><<<dim3((unsigned)b.blocks), dim3(Q::TX, Q::TY), Q::SMEM, s>>>(b.tab, b.start, b.lanes);
+    return cudaGetLastError();
+}
+
+template <int K, int PF>
 cudaError_t gradq_go(const AdjArgs& a, const CUtensorMap& tu, const CUtensorMap& tl, const CUtensorMap& tg,
                      cudaStream_t s)
 {
@@ -420,11 +498,9 @@ cudaError_t launch_fwdq(const FwdArgs& a, const CUtensorMap& tu, const CUtensorM
     }
 }
 
-cudaError_t launch_adjq(const AdjArgs& a, const CUtensorMap* maps, const Tile& t, int K, cudaStream_t s)
+// the lam half: a forward step of the adjoint field with the adjoint injection
+FwdArgs lam_args(const AdjArgs& a)
 {
-    if (!v3_fits(a.g, K) || !tq_supported(a.g.dims, K, t)) return cudaErrorInvalidValue;
-    if (a.g.X0 != (K <= 4 ? 4 : 8) || a.g.H != K) return cudaErrorInvalidValue;
-    // the lam half: a forward step of the adjoint field with the adjoint injection
     FwdArgs f{};
     f.g = a.g;
     f.u = a.l1;
@@ -434,12 +510,18 @@ cudaError_t launch_adjq(const AdjArgs& a, const CUtensorMap* maps, const Tile& t
     f.eta = a.eta;
     f.hdt = a.hdt;
     for (int j = 0; j <= MAXK; ++j) f.c[j] = a.c[j];
+    f.zlen = a.zlen;
     f.src = a.adj;
-    f.smp.n = 0;
-    f.ck_u = nullptr;
-    f.ck_up = nullptr;
     f.err = a.err;
     f.wait_limit = a.wait_limit;
+    return f;
+}
+
+cudaError_t launch_adjq(const AdjArgs& a, const CUtensorMap* maps, const Tile& t, int K, cudaStream_t s)
+{
+    if (!v3_fits(a.g, K) || !tq_supported(a.g.dims, K, t)) return cudaErrorInvalidValue;
+    if (a.g.X0 != (K <= 4 ? 4 : 8) || a.g.H != K) return cudaErrorInvalidValue;
+    const FwdArgs f = lam_args(a);
     cudaError_t e = launch_fwdq(f, maps[0], maps[1], maps[2], t, K, CK_NONE, s);
     if (e != cudaSuccess) return e;
     AdjArgs b = a;
@@ -449,6 +531,34 @@ cudaError_t launch_adjq(const AdjArgs& a, const CUtensorMap* maps, const Tile& t
     case 2: return gradq_p<2>(b, maps[3], maps[4], maps[5], t.pf, s);
     case 4: return gradq_p<4>(b, maps[3], maps[4], maps[5], t.pf, s);
     case 8: return gradq_p<8>(b, maps[3], maps[4], maps[5], t.pf, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_fwdq_batch(const BatchLaunch<FwdArgs>& b, const Tile& t, int K, int ck, cudaStream_t s)
+{
+    if (!tq_supported(b.dims, K, t)) return cudaErrorInvalidValue;
+    const bool two = t.pf == 2;
+    switch (K) {
+    case 1: return two ? fwdqb_go<1, 2>(b, ck, s) : fwdqb_go<1, 1>(b, ck, s);
+    case 2: return two ? fwdqb_go<2, 2>(b, ck, s) : fwdqb_go<2, 1>(b, ck, s);
+    case 4: return two ? fwdqb_go<4, 2>(b, ck, s) : fwdqb_go<4, 1>(b, ck, s);
+    case 8: return two ? fwdqb_go<8, 2>(b, ck, s) : fwdqb_go<8, 1>(b, ck, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_adjq_batch(const BatchLaunch<FwdArgs>& lam, const BatchLaunch<AdjArgs>& b, const Tile& t, int K,
+                              cudaStream_t s)
+{
+    cudaError_t e = launch_fwdq_batch(lam, t, K, CK_NONE, s);
+    if (e != cudaSuccess) return e;
+    const bool two = t.pf == 2;
+    switch (K) {
+    case 1: return two ? gradqb_go<1, 2>(b, s) : gradqb_go<1, 1>(b, s);
+    case 2: return two ? gradqb_go<2, 2>(b, s) : gradqb_go<2, 1>(b, s);
+    case 4: return two ? gradqb_go<4, 2>(b, s) : gradqb_go<4, 1>(b, s);
+    case 8: return two ? gradqb_go<8, 2>(b, s) : gradqb_go<8, 1>(b, s);
     default: return cudaErrorInvalidValue;
     }
 }
