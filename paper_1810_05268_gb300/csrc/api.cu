@@ -1608,7 +1608,12 @@ int autotune(ckfwi_model* m, cudaStream_t st)
             nzc = std::max<long long>(1, std::min<long long>(nzc, f.nz));
             add((int)((f.nz + nzc - 1) / nzc));
         }
-        for (int z = 4; z <= 32; ++z) add(z);
+        // (an order-16 run reads 16 planes beyond its own: short ones never win)
+        for (int z = m->K > 4 ? 12 : 4; z <= 32; ++z) add(z);
+        // columns cut into two to eight equal runs (the lean reverse step of
+        // order 8 at 208^3, three CTAs an SM: 69.2 us at runs of 42, 71.9 at
+        // 21, the best below 33)
+        for (int r = 2; r <= 8; ++r) add((f.nz + r - 1) / r);
         return zl;
     };
     // the OT4 kernel has its own two-pass kernels, tried alone

@@ -37,7 +37,7 @@ struct Maps4 {
 
 // CTAs an SM at order <= 8: shared memory and registers of one point field
 // allow one more than those of three
-template <int K, int PF, int OP> constexpr int ot4q_min_blocks() { return K > 4 ? 1 : (points_of(OP) == 1 ? 7 : 6) - PF; }
+template <int K, int PF, int OP> constexpr int ot4q_min_blocks() { return K > 4 ? (PF == 1 ? 4 : 3) : (points_of(OP) == 1 ? 7 : 6) - PF; }
 
 template <int K, int PF, int OP, int CK>
 __global__ void __launch_bounds__(128, ot4q_min_blocks<K, PF, OP>())
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(128, ot4q_min_blocks<K, PF, OP>())
     constexpr int NP = points_of(OP);
     using Q = TQ<K, PF, NP>;
     using G = typename Q::G;
-    constexpr int V = Q::V, TX = Q::TX, TY = Q::TY, D = Q::D, RU = Q::RU, RP = Q::RP;
+    constexpr int V = Q::V, TX = Q::TX, TY = Q::TY, D = Q::D, RU = Q::RU, RP = Q::RP, LD = Q::LEAD;
     extern __shared__ unsigned char smq_raw[];
     __shared__ int abort_s[2];                  // a wait gave up at a step of this parity
     unsigned char* sm0 = align128(smq_raw);
@@ -98,11 +98,11 @@ __global__ void __launch_bounds__(128, ot4q_min_blocks<K, PF, OP>())
     // point planes z0 + g - K (see stencil_tq.cu)
     auto issue = [&](int g) {
         uint64_t* b = bar + g % RU;
-        const bool pt = g >= K;
+        const bool pt = g >= LD;
         bar_expect(b, Q::UBYTES + (pt ? NP * Q::PBYTES : 0));
         tile3(ring + (g % RU) * Q::US, &M.f, xb, yb, min(z0 + g, zqmax) + K, b);
         if (pt) {
-            const int zp = min(z0 + g - K, z1 - 1) + K, s = (g - K) % RP;
+            const int zp = min(z0 + g - LD, z1 - 1) + K, s = (g - LD) % RP;
 #pragma unroll
             for (int k = 0; k < NP; ++k) tile3(pts + (k * RP + s) * Q::PT, &M.p[k], xb + G::PX, yb + K, zp, b);
         }
@@ -113,36 +113,46 @@ __global__ void __launch_bounds__(128, ot4q_min_blocks<K, PF, OP>())
         abort_s[0] = abort_s[1] = 0;
         for (int s = 0; s < RU; ++s) bar_init(bar + s);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (int g = 0; g < K + D; ++g) issue(g);
+        for (int g = 0; g < LD + D; ++g) issue(g);
     }
     __syncthreads();
-    int issued = K + D;
-    float q[2 * K + 1][V];
+    int issued = LD + D;
+    float q[2 * K + 1][V], nq[V];
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
+    for (int i = 0; i < (Q::COL ? 2 * K : K); ++i) {
         if (cload) gld<V>(q[i], A.s + (z0 - K + i) * pxy + col);
         else vzero<V>(q[i]);
     }
+    if constexpr (Q::COL) {
+        if (cload) gld<V>(nq, A.s + (z0 + K) * pxy + col);
+        else vzero<V>(nq);
+    }
     int g0 = 0;
-    while (g0 < K && wait_group(g0)) ++g0;
-    if (g0 < K) abort_s[0] = 1;
+    while (g0 < LD && wait_group(g0)) ++g0;
+    if (g0 < LD) abort_s[0] = 1;
     bool aborted = false;                        // the same in every thread: read after one barrier
     int confirmed = g0;
 #pragma unroll
-    for (int i = 0; i < K; ++i) sld<V>(q[K + i], ring + i * Q::US + cs);
+    for (int i = 0; i < LD; ++i) sld<V>(q[K + i], ring + i * Q::US + cs);
 
     for (int step = 0; step < nstep; ++step) {
         const int z = z0 + step;
-        if (!wait_group(step + K)) abort_s[step & 1] = 1;
+        if (!wait_group(step + LD)) abort_s[step & 1] = 1;
         __syncthreads();                        // every thread is past step - 1: its slots are free
         if (abort_s[step & 1]) {
             aborted = true;
             break;
         }
-        confirmed = step + K + 1;
-        if (tid == 0) issue(step + K + D);
-        issued = step + K + D + 1;
-        sld<V>(q[2 * K], ring + ((step + K) % RU) * Q::US + cs);
+        confirmed = step + LD + 1;
+        if (tid == 0) issue(step + LD + D);
+        issued = step + LD + D + 1;
+        if constexpr (Q::COL) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) q[2 * K][k] = nq[k];
+            if (cload) gld<V>(nq, A.s + min(z + K + 1, zqmax) * pxy + col);
+        } else {
+            sld<V>(q[2 * K], ring + ((step + K) % RU) * Q::US + cs);
+        }
         const float* sm = ring + (step % RU) * Q::US;
         if (cload) {
             float pv[NP][V], r[V], l[V];

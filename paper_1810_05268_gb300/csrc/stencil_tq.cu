@@ -36,7 +36,7 @@ namespace {
 
 // CTAs an SM at order <= 8, set by the register cap: six with one plane of
 // prefetch (31 KB of shared memory), five with two (39 KB)
-template <int K, int PF> constexpr int tq_min_blocks() { return K <= 4 ? (PF == 1 ? 6 : 5) : 1; }
+template <int K, int PF> constexpr int tq_min_blocks() { return K <= 4 ? (PF == 1 ? 6 : 5) : (PF == 1 ? 4 : 3); }
 
 // Body of the forward step for CTA (bxi, byi, bzi) of a grid of gx x gy CTAs a
 // plane (one shot's, or one lane's of a batch)
@@ -46,7 +46,7 @@ __device__ __forceinline__ void fwdq_body(const FwdArgs& a, const CUtensorMap* t
 {
     using Q = TQ<K, PF>;
     using G = typename Q::G;
-    constexpr int V = Q::V, TX = Q::TX, TY = Q::TY, D = Q::D, RU = Q::RU, RP = Q::RP;
+    constexpr int V = Q::V, TX = Q::TX, TY = Q::TY, D = Q::D, RU = Q::RU, RP = Q::RP, LD = Q::LEAD;
     extern __shared__ unsigned char smq_raw[];
     __shared__ int abort_s[2];                  // a wait gave up at a step of this parity
     unsigned char* sm0 = align128(smq_raw);
@@ -96,11 +96,11 @@ __device__ __forceinline__ void fwdq_body(const FwdArgs& a, const CUtensorMap* t
     // on barrier g % RU, whose phase (g / RU) it completes.
     auto issue = [&](int g) {
         uint64_t* b = bar + g % RU;
-        const bool pts = g >= K;
+        const bool pts = g >= LD;
         bar_expect(b, Q::UBYTES + (pts ? 2 * Q::PBYTES : 0));
         tile3(ring + (g % RU) * Q::US, tmu, xb, yb, min(z0 + g, zqmax) + K, b);
         if (pts) {
-            const int zp = min(z0 + g - K, z1 - 1) + K, s = (g - K) % RP;
+            const int zp = min(z0 + g - LD, z1 - 1) + K, s = (g - LD) % RP;
             tile3(upr + s * Q::PT, tmp, xb + G::PX, yb + K, zp, b);
             tile3(wr + s * Q::PT, tmw, xb + G::PX, yb + K, zp, b);
         }
@@ -111,26 +111,30 @@ __device__ __forceinline__ void fwdq_body(const FwdArgs& a, const CUtensorMap* t
         abort_s[0] = abort_s[1] = 0;
         for (int s = 0; s < RU; ++s) bar_init(bar + s);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (int g = 0; g < K + D; ++g) issue(g);
+        for (int g = 0; g < LD + D; ++g) issue(g);
     }
     __syncthreads();
-    int issued = K + D;                          // groups 0 .. issued - 1 are in flight or done
+    int issued = LD + D;                          // groups 0 .. issued - 1 are in flight or done
 
     // the queue: planes z0 - K .. z0 - 1 straight from global memory, planes
     // z0 .. z0 + K - 1 from the ring once their groups land
-    float q[2 * K + 1][V];
+    float q[2 * K + 1][V], nq[V];
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
+    for (int i = 0; i < (Q::COL ? 2 * K : K); ++i) {
         if (cload) gld<V>(q[i], a.u + (z0 - K + i) * pxy + col);
         else vzero<V>(q[i]);
     }
+    if constexpr (Q::COL) {
+        if (cload) gld<V>(nq, a.u + (z0 + K) * pxy + col);
+        else vzero<V>(nq);
+    }
     int g0 = 0;
-    while (g0 < K && wait_group(g0)) ++g0;
-    if (g0 < K) abort_s[0] = 1;
+    while (g0 < LD && wait_group(g0)) ++g0;
+    if (g0 < LD) abort_s[0] = 1;
     bool aborted = false;                        // the same in every thread: read after one barrier
     int confirmed = g0;                          // groups 0 .. confirmed - 1 are known complete
 #pragma unroll
-    for (int i = 0; i < K; ++i) sld<V>(q[K + i], ring + i * Q::US + cs);
+    for (int i = 0; i < LD; ++i) sld<V>(q[K + i], ring + i * Q::US + cs);
 
     int step = 0;
     for (; step < nstep; ++step) {
@@ -138,16 +142,22 @@ __device__ __forceinline__ void fwdq_body(const FwdArgs& a, const CUtensorMap* t
         // the group of u plane z + K and point plane z
         // a wait that gave up flags this step's slot (step & 1): a thread one
         // step ahead writes the other slot, so all leave at the same step
-        if (!wait_group(step + K)) abort_s[step & 1] = 1;
+        if (!wait_group(step + LD)) abort_s[step & 1] = 1;
         __syncthreads();                        // every thread is past step - 1: its slots are free
         if (abort_s[step & 1]) {
             aborted = true;
             break;
         }
-        confirmed = step + K + 1;
-        if (tid == 0) issue(step + K + D);      // into the slots step - 1 read
-        issued = step + K + D + 1;
-        sld<V>(q[2 * K], ring + ((step + K) % RU) * Q::US + cs);
+        confirmed = step + LD + 1;
+        if (tid == 0) issue(step + LD + D);      // into the slots step - 1 read
+        issued = step + LD + D + 1;
+        if constexpr (Q::COL) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) q[2 * K][k] = nq[k];
+            if (cload) gld<V>(nq, a.u + min(z + K + 1, zqmax) * pxy + col);
+        } else {
+            sld<V>(q[2 * K], ring + ((step + K) % RU) * Q::US + cs);
+        }
         const float* sm = ring + (step % RU) * Q::US;
         if (cload) {
             float upv[V], wv[V];
@@ -282,7 +292,7 @@ __device__ __forceinline__ void gradq_body(const AdjArgs& a, const CUtensorMap* 
 {
     using Q = TQ<K, PF>;
     using G = typename Q::G;
-    constexpr int V = Q::V, TX = Q::TX, TY = Q::TY, D = Q::D, RU = Q::RU, RP = Q::RP;
+    constexpr int V = Q::V, TX = Q::TX, TY = Q::TY, D = Q::D, RU = Q::RU, RP = Q::RP, LD = Q::LEAD;
     extern __shared__ unsigned char smq_raw[];
     __shared__ int abort_s[2];                  // a wait gave up at a step of this parity
     unsigned char* sm0 = align128(smq_raw);
@@ -315,11 +325,11 @@ __device__ __forceinline__ void gradq_body(const AdjArgs& a, const CUtensorMap* 
 
     auto issue = [&](int g) {
         uint64_t* b = bar + g % RU;
-        const bool pts = g >= K;
+        const bool pts = g >= LD;
         bar_expect(b, Q::UBYTES + (pts ? 2 * Q::PBYTES : 0));
         tile3(ring + (g % RU) * Q::US, tmu, xb, yb, min(z0 + g, zqmax) + K, b);
         if (pts) {
-            const int zp = min(z0 + g - K, z1 - 1) + K, sl = (g - K) % RP;
+            const int zp = min(z0 + g - LD, z1 - 1) + K, sl = (g - LD) % RP;
             tile3(lr + sl * Q::PT, tml, xb + G::PX, yb + K, zp, b);
             tile3(gr + sl * Q::PT, tmg, xb + G::PX, yb + K, zp, b);
         }
@@ -330,36 +340,46 @@ __device__ __forceinline__ void gradq_body(const AdjArgs& a, const CUtensorMap* 
         abort_s[0] = abort_s[1] = 0;
         for (int sl = 0; sl < RU; ++sl) bar_init(bar + sl);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (int g = 0; g < K + D; ++g) issue(g);
+        for (int g = 0; g < LD + D; ++g) issue(g);
     }
     __syncthreads();
-    int issued = K + D;
-    float q[2 * K + 1][V];
+    int issued = LD + D;
+    float q[2 * K + 1][V], nq[V];
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
+    for (int i = 0; i < (Q::COL ? 2 * K : K); ++i) {
         if (cload) gld<V>(q[i], u + (z0 - K + i) * pxy + col);
         else vzero<V>(q[i]);
     }
+    if constexpr (Q::COL) {
+        if (cload) gld<V>(nq, u + (z0 + K) * pxy + col);
+        else vzero<V>(nq);
+    }
     int g0 = 0;
-    while (g0 < K && wait_group(g0)) ++g0;
-    if (g0 < K) abort_s[0] = 1;
+    while (g0 < LD && wait_group(g0)) ++g0;
+    if (g0 < LD) abort_s[0] = 1;
     bool aborted = false;                        // the same in every thread: read after one barrier
     int confirmed = g0;
 #pragma unroll
-    for (int i = 0; i < K; ++i) sld<V>(q[K + i], ring + i * Q::US + cs);
+    for (int i = 0; i < LD; ++i) sld<V>(q[K + i], ring + i * Q::US + cs);
 
     for (int step = 0; step < nstep; ++step) {
         const int z = z0 + step;
-        if (!wait_group(step + K)) abort_s[step & 1] = 1;
+        if (!wait_group(step + LD)) abort_s[step & 1] = 1;
         __syncthreads();
         if (abort_s[step & 1]) {
             aborted = true;
             break;
         }
-        confirmed = step + K + 1;
-        if (tid == 0) issue(step + K + D);
-        issued = step + K + D + 1;
-        sld<V>(q[2 * K], ring + ((step + K) % RU) * Q::US + cs);
+        confirmed = step + LD + 1;
+        if (tid == 0) issue(step + LD + D);
+        issued = step + LD + D + 1;
+        if constexpr (Q::COL) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) q[2 * K][k] = nq[k];
+            if (cload) gld<V>(nq, u + min(z + K + 1, zqmax) * pxy + col);
+        } else {
+            sld<V>(q[2 * K], ring + ((step + K) % RU) * Q::US + cs);
+        }
         const float* sm = ring + (step % RU) * Q::US;
         if (cload) {
             float lv[V], gv[V];

@@ -62,7 +62,16 @@ template <int K, int PF, int NP = 2>
 struct TQ {
     static constexpr int V = 4, TX = 8, TY = 16, D = PF;
     using G = G3<K, V, TX, TY>;
-    static constexpr int RU = K + D + 1;                       // u tiles in the ring
+    // A tile of the staged field waits in the ring from when its column feeds
+    // the queue (K planes ahead) until it is the centre plane.  At order 16
+    // that is 67 KB a CTA, two or three CTAs an SM; there the queue loads its
+    // column itself (the tile's copy finds it in L2) and the ring holds the
+    // planes of the prefetch only: four CTAs an SM with one plane of it.  At
+    // 300 x 600 x 600 a forward step takes 523 us (595 with the long ring, 554
+    // the lean kernel), the split reverse step 985 us (1118).
+    static constexpr bool COL = K > 4;
+    static constexpr int LEAD = COL ? 0 : K;                   // planes from a group's u tile to its point tiles
+    static constexpr int RU = LEAD + D + 1;                    // u tiles in the ring
     static constexpr int RP = D + 1;                           // point tiles of each point field
     static constexpr int UBYTES = G::TILE * 4;                 // one u box
     static constexpr int US = (UBYTES + 127) / 128 * 32;       // ring slot stride [floats], 128-byte multiple
