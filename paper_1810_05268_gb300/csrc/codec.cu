@@ -39,7 +39,7 @@
 //     warp assembles its chunk's bits contiguously in shared memory and
 //     writes them back over the slot, with the chunk's word count, which it
 //     also adds to the sums of its group of 32 and of 1024 chunks;
-//  2. compact: a small CTA per 4 chunks copies them from staging to the
+//  2. compact: a small CTA per 8 chunks copies them from staging to the
 //     payload, and their blocks' sizes to the table, at offsets formed from
 //     at most (chunks / 1024) + 62 group sums and chunk counts (linear total
 //     work); CTA 0 writes the header, the last CTA resets the group sums.
@@ -466,9 +466,12 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const __
 // overflow (nothing is written) and, in CTA 0, the header, the pool's next
 // word and the statistics.  The last CTA to finish reading the sums (a
 // counter, no waiting) sets them back to zero for the next compression.
-// Small CTAs spread the copy over every SM.
+// Small CTAs spread the copy over every SM; eight chunks are what the threads
+// copy the sizes of at once (four chunks: an inversion iteration over 2D
+// fields took 484 ms, now 473).
 constexpr int CMP_THREADS = 128;
-constexpr int CPB = 4;
+constexpr int CPB = 8;
+static_assert(CPB * CHUNK / 2 <= CMP_THREADS, "a thread copies one word of sizes");
 
 template <int DIMS>
 __global__ void __launch_bounds__(CMP_THREADS) compact_kernel(const __grid_constant__ CodecCall call)
@@ -594,19 +597,6 @@ __global__ void __launch_bounds__(CMP_THREADS) compact_kernel(const __grid_const
     }
 }
 
-// 64 stream bits starting at bit `pos` of the payload (zeros past `limit` words)
-__device__ __forceinline__ unsigned long long peek64(const uint32_t* __restrict__ p, long long pos, long long limit)
-{
-    const long long w = pos >> 5;
-    const int sh = (int)(pos & 31);
-    const unsigned long long w0 = w < limit ? p[w] : 0u;
-    const unsigned long long w1 = w + 1 < limit ? p[w + 1] : 0u;
-    const unsigned long long w2 = w + 2 < limit ? p[w + 2] : 0u;
-    unsigned long long v = (w0 | (w1 << 32)) >> sh;
-    if (sh) v |= w2 << (64 - sh);
-    return v;
-}
-
 template <int DIMS>
 __global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_constant__ CodecCall call)
 {
@@ -656,26 +646,27 @@ __global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_consta
         atomicOr(err, 4);
         return;
     }
-    long long pos = start;
+    BitR rd(payload + (start >> 5), payload + pw, (int)(start & 31));
+    int used = 0;                                  // bits of the block read so far
     bool corrupt = false;
     float f[V];
-    const unsigned long long h0 = peek64(payload, pos, pw);
-    if (!(h0 & 1ull)) {
-        pos += 1;
+    rd.need();
+    const uint32_t h0 = (uint32_t)rd.buf;          // the longest block header has 20 bits
+    if (!(h0 & 1u)) {
+        used = 1;
 #pragma unroll
         for (int i = 0; i < V; ++i) f[i] = 0.0f;
-    } else if (h0 & 2ull) {
-        pos += 2;
+    } else if (h0 & 2u) {
+        rd.skip(2);
+        used = 2 + 32 * V;
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            f[i] = __uint_as_float((uint32_t)peek64(payload, pos, pw));
-            pos += 32;
-        }
+        for (int i = 0; i < V; ++i) f[i] = __uint_as_float(rd.take(32));
     } else {
         const int emax = (int)((h0 >> 2) & 0xFFu) - 127;
         const int ptop = (int)((h0 >> 10) & 31u);
         const int pbot = (int)((h0 >> 15) & 31u);
-        pos += 20;
+        rd.skip(20);
+        used = 20;
         if (emax < -126 || emax > 127 || pbot > ptop) corrupt = true;
         // plane words into this thread's shared column (rows p and 32 + p),
         // then one bit-matrix transpose gives the coefficient words
@@ -688,34 +679,18 @@ __global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_consta
         int s = 0;
 #pragma unroll 1
         for (int p = ptop; p >= pbot && !corrupt; --p) {
-            unsigned long long W = 0;
-            if (s > 0) {
-                W = peek64(payload, pos, pw) & low_mask(s);
-                pos += s;
-            }
+            unsigned long long W = s > 0 ? rd.take64(s) : 0ull;
+            used += s;
             while (s < V) {
-                // one look at the group test and the run after it; a run
-                // longer than the 63 bits past the test takes a second look
-                const unsigned long long t = peek64(payload, pos, pw);
-                if (!(t & 1ull)) {
-                    pos += 1;
-                    break;
-                }
-                unsigned long long look = t >> 1;
-                int z;
-                if (look != 0ull) {
-                    z = __ffsll((long long)look) - 1;
-                } else {
-                    look = peek64(payload, pos + 1, pw);
-                    if (look == 0ull) { corrupt = true; break; }
-                    z = __ffsll((long long)look) - 1;
-                }
-                if (s + z >= V) { corrupt = true; break; }
+                ++used;
+                if (!rd.take(1)) break;            // group test
+                const int z = rd.run(V - s);       // a run that leaves the block has no end
+                if (z >= V - s) { corrupt = true; break; }
                 W |= 1ull << (s + z);
-                pos += z + 2;
+                used += z + 1;
                 s += z + 1;
             }
-            if (pos > end) corrupt = true;
+            if (used > nbits) corrupt = true;
             col[p * S] = (uint32_t)W;
             if (V > 32) col[(32 + p) * S] = (uint32_t)(W >> 32);
         }
@@ -737,7 +712,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_consta
 #pragma unroll
         for (int i = 0; i < V; ++i) f[i] = __fmul_rn(__int2float_rn(t[i]), sc);
     }
-    if (corrupt || pos != end) {
+    if (corrupt || used != nbits) {
         atomicOr(err, 4);
         return;
     }

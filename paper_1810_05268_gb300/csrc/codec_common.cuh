@@ -207,6 +207,78 @@ __device__ __forceinline__ BlockPos block_pos(const Geo& G, long long b)
     return p;
 }
 
+__device__ __forceinline__ uint32_t mask32(int n) { return n >= 32 ? ~0u : (1u << n) - 1u; }
+
+// Bit reader with its next bits in registers: 33 to 64 of them after need(),
+// and the word after those already on its way.  (Looking at the stream anew
+// for every group test, three words and their addresses a look, was most of a
+// decoder's time and its longest wait.)  Words from `end` on read as zero.
+struct BitR {
+    const uint32_t* w;
+    const uint32_t* end;
+    unsigned long long buf;
+    uint32_t nxt;
+    int nb;               // bits in buf
+    __device__ __forceinline__ uint32_t load()
+    {
+        const uint32_t v = w < end ? __ldg(w) : 0u;
+        ++w;
+        return v;
+    }
+    // from bit `sh` (0 .. 31) of word `at` on
+    __device__ __forceinline__ BitR(const uint32_t* at, const uint32_t* end_, int sh) : w(at), end(end_)
+    {
+        buf = load() >> sh;
+        nb = 32 - sh;
+        nxt = load();
+    }
+    __device__ __forceinline__ void need()            // at least 32 bits in buf
+    {
+        if (nb < 32) {
+            buf |= (unsigned long long)nxt << nb;
+            nb += 32;
+            nxt = load();
+        }
+    }
+    __device__ __forceinline__ void skip(int n)       // n <= 32, after need()
+    {
+        buf >>= n;
+        nb -= n;
+    }
+    __device__ __forceinline__ uint32_t take(int n)   // n <= 32
+    {
+        need();
+        const uint32_t v = (uint32_t)buf & mask32(n);
+        skip(n);
+        return v;
+    }
+    __device__ __forceinline__ unsigned long long take64(int n)   // n <= 64
+    {
+        if (n <= 32) return take(n);
+        const uint32_t lo = take(32);
+        return lo | (unsigned long long)take(n - 32) << 32;
+    }
+    // zeros before the next set bit among the next n (<= 64), which is taken
+    // too; n when there is none
+    __device__ __forceinline__ int run(int n)
+    {
+        int z = 0;
+        while (z < n) {
+            need();
+            const int c = min(n - z, 32);
+            const uint32_t t = (uint32_t)buf & mask32(c);
+            if (t) {
+                const int f = __ffs((int)t) - 1;
+                skip(f + 1);
+                return z + f;
+            }
+            skip(c);
+            z += c;
+        }
+        return n;
+    }
+};
+
 // In-place transpose of a 32 x 32 bit matrix: on return a[p] bit r is the
 // input a[r] bit p (five stages of block swaps: j = 16, 8, 4, 2, 1).  The
 // half-word and byte swaps of the first two stages are byte permutes (two
