@@ -406,7 +406,7 @@ def codec_compress(x, tol, stream=None):
     dims = x.dim()
     nz, ny, nx = _shape3(tuple(x.shape))
     cap = codec_bound_words(dims, nz, ny, nx)
-    out = torch.zeros(cap, dtype=torch.int32, device=x.device)
+    out = torch.empty(cap, dtype=torch.int32, device=x.device)
     used = ctypes.c_longlong(0)
     flags = ctypes.c_int(0)
     with torch.cuda.device(x.device):
@@ -457,7 +457,7 @@ def codec_compress_rate(x, rate, stream=None):
     dims = x.dim()
     nz, ny, nx = _shape3(tuple(x.shape))
     cap = codec_rate_words(dims, nz, ny, nx, rate)
-    out = torch.zeros(cap, dtype=torch.int32, device=x.device)
+    out = torch.empty(cap, dtype=torch.int32, device=x.device)
     used = ctypes.c_longlong(0)
     flags = ctypes.c_int(0)
     _check(lib().ckfwi_codec_compress_rate(ctypes.c_void_p(x.data_ptr()), dims, nz, ny, nx, int(rate),
@@ -472,7 +472,7 @@ def codec_decompress(stream_words, shape, stream=None):
         raise ValueError("codec_decompress needs a contiguous CUDA tensor of 32-bit stream words")
     dims = len(shape)
     nz, ny, nx = _shape3(tuple(shape))
-    out = torch.zeros(tuple(shape), dtype=torch.float32, device=stream_words.device)
+    out = torch.empty(tuple(shape), dtype=torch.float32, device=stream_words.device)
     with torch.cuda.device(stream_words.device):
         _check(lib().ckfwi_codec_decompress(ctypes.c_void_p(stream_words.data_ptr()), stream_words.numel(), dims,
                                             nz, ny, nx, ctypes.c_void_p(out.data_ptr()), _stream(stream)),

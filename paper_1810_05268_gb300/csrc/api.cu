@@ -3716,9 +3716,48 @@ long long ckfwi_codec_bound_words(int dims, int nz, int ny, int nx)
 }  // extern "C"
 
 namespace {
+// What the standalone calls keep per device (under the mutex; every call ends
+// with the stream synchronised): the scratch of the last layout, eight words
+// on the device (the stream's start, always 0, its end, error bits) and their
+// pinned copy.  Both must start a call as a finished one leaves them: zero
+// counters (for the same layout of the scratch) and no error bits; what is not
+// known to be so is cleared.
+struct CodecDev {
+    DevMem scratch, scal;
+    HostMem pin;
+    long long layout[4] = {0, 0, 0, 0};   // of the field whose compression left the scratch's counters zero
+    bool clean = false;                   // the words hold no error bits
+};
 std::mutex g_codec_mu;
-DevMem* g_codec_scratch[64] = {};
-DevMem* g_codec_scal[64] = {};
+CodecDev* g_codec[64] = {};
+
+int codec_dev(cudaStream_t st, CodecDev** out)
+{
+    int dev = 0;
+    CK_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return CKFWI_EINVAL;
+    if (!g_codec[dev]) g_codec[dev] = new (std::nothrow) CodecDev();
+    CodecDev* c = g_codec[dev];
+    if (!c) return CKFWI_ENOMEM;
+    CK_TRY(c->scal.alloc(64, true));
+    CK_TRY(c->pin.alloc(64));
+    if (!c->clean) CK_TRY(cudaMemsetAsync(c->scal.p, 0, 64, st));
+    c->clean = false;                     // until the call has ended without an error
+    *out = c;
+    return CKFWI_OK;
+}
+
+// wait for the call; the stream's end and the error bits
+int codec_wait(CodecDev* c, cudaStream_t st, long long* end, int* err)
+{
+    CK_TRY(cudaMemcpyAsync(c->pin.p, c->scal.p, 40, cudaMemcpyDeviceToHost, st));
+    CK_TRY(cudaStreamSynchronize(st));
+    const long long* h = static_cast<const long long*>(c->pin.p);
+    *end = h[1];
+    *err = (int)(h[4] & 0xffffffff);
+    c->clean = *err == 0;
+    return CKFWI_OK;
+}
 
 // A call on one dense field: its stream in `pool` from the word in sc[0] on,
 // the end of a compressed stream to sc[1], error bits at sc[4]
@@ -3750,34 +3789,33 @@ extern "C" int ckfwi_codec_compress(const float* x, int dims, int nz, int ny, in
     if ((dims != 2 && dims != 3) || nz < 1 || ny < 1 || nx < 1 || (dims == 2 && ny != 1)) return CKFWI_EINVAL;
     if (!(tol >= std::ldexp(1.0, -90)) || !std::isfinite(tol)) return CKFWI_EINVAL;
     cudaStream_t st = S(stream);
-    int dev = 0;
-    CK_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return CKFWI_EINVAL;
     std::lock_guard<std::mutex> lk(g_codec_mu);
-    if (!g_codec_scratch[dev]) g_codec_scratch[dev] = new DevMem();
-    if (!g_codec_scal[dev]) g_codec_scal[dev] = new DevMem();
-    DevMem& scr = *g_codec_scratch[dev];
-    DevMem& scal = *g_codec_scal[dev];
+    CodecDev* d = nullptr;
+    ST_TRY(codec_dev(st, &d));
     const size_t need = (size_t)codec_scratch_bytes(dims, nz, ny, nx, 1);
-    if (scr.bytes < need) CK_TRY(scr.alloc(need, false));
-    CK_TRY(scal.alloc(64, true));
-    CK_TRY(cudaMemsetAsync(scal.p, 0, 64, st));
     // the scratch serves fields of any size here: its counter and group sums
-    // are cleared for this one's layout
-    CK_TRY(cudaMemsetAsync(scr.p, 0, (size_t)codec_scratch_zero_bytes(dims, nz, ny, nx), st));
-    long long* sc = scal.as<long long>();
+    // are cleared when this one's layout is not the last one's
+    const long long lay[4] = {dims, nz, ny, nx};
+    bool same = std::equal(lay, lay + 4, d->layout);
+    if (d->scratch.bytes < need) {
+        CK_TRY(d->scratch.alloc(need, false));
+        same = false;
+    }
+    if (!same) CK_TRY(cudaMemsetAsync(d->scratch.p, 0, (size_t)codec_scratch_zero_bytes(dims, nz, ny, nx), st));
+    d->layout[0] = 0;
+    long long* sc = d->scal.as<long long>();
     CodecCall c = dense_call(const_cast<float*>(x), dims, nz, ny, nx, out, cap, sc);
-    c.one.scratch = scr.p;
+    c.one.scratch = d->scratch.p;
     c.tol_f = tol_float(tol);
     CK_TRY(codec_compress_dev(c, st));
-    long long h[5];
-    CK_TRY(cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st));
-    CK_TRY(cudaStreamSynchronize(st));
-    const int e = (int)(h[4] & 0xffffffff);
+    long long end = 0;
+    int e = 0;
+    ST_TRY(codec_wait(d, st, &end, &e));
+    std::copy(lay, lay + 4, d->layout);
     if (flags) *flags = (e & 1) ? 1 : 0;
     if (e & 2) return CKFWI_POOL_OVERFLOW;
     if (e & 4) return CKFWI_CORRUPT;          // a chunk the compaction refused: the stream is incomplete
-    if (used_words) *used_words = h[1];
+    if (used_words) *used_words = end;
     return CKFWI_OK;
 }
 
@@ -3795,25 +3833,18 @@ extern "C" int ckfwi_codec_compress_rate(const float* x, int dims, int nz, int n
     if ((dims != 2 && dims != 3) || nz < 1 || ny < 1 || nx < 1 || (dims == 2 && ny != 1)) return CKFWI_EINVAL;
     if (rate < 1 || rate > 32) return CKFWI_EINVAL;
     cudaStream_t st = S(stream);
-    int dev = 0;
-    CK_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return CKFWI_EINVAL;
     std::lock_guard<std::mutex> lk(g_codec_mu);
-    if (!g_codec_scal[dev]) g_codec_scal[dev] = new DevMem();
-    DevMem& scal = *g_codec_scal[dev];
-    CK_TRY(scal.alloc(64, true));
-    CK_TRY(cudaMemsetAsync(scal.p, 0, 64, st));
-    long long* sc = scal.as<long long>();
-    CodecCall c = dense_call(const_cast<float*>(x), dims, nz, ny, nx, out, cap, sc);
+    CodecDev* d = nullptr;
+    ST_TRY(codec_dev(st, &d));
+    CodecCall c = dense_call(const_cast<float*>(x), dims, nz, ny, nx, out, cap, d->scal.as<long long>());
     c.rate = rate;
     CK_TRY(codec_rate_compress_dev(c, st));
-    long long h[5];
-    CK_TRY(cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st));
-    CK_TRY(cudaStreamSynchronize(st));
-    const int e = (int)(h[4] & 0xffffffff);
+    long long end = 0;
+    int e = 0;
+    ST_TRY(codec_wait(d, st, &end, &e));
     if (flags) *flags = (e & 1) ? 1 : 0;
     if (e & 2) return CKFWI_POOL_OVERFLOW;
-    if (used_words) *used_words = h[1];
+    if (used_words) *used_words = end;
     return CKFWI_OK;
 }
 
@@ -3823,32 +3854,20 @@ extern "C" int ckfwi_codec_decompress(const uint32_t* in, long long nwords, int 
     if (!in || !x || nwords <= 0) return CKFWI_EINVAL;
     if ((dims != 2 && dims != 3) || nz < 1 || ny < 1 || nx < 1 || (dims == 2 && ny != 1)) return CKFWI_EINVAL;
     cudaStream_t st = S(stream);
-    int dev = 0;
-    CK_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return CKFWI_EINVAL;
-    std::lock_guard<std::mutex> lk(g_codec_mu);
-    if (!g_codec_scal[dev]) g_codec_scal[dev] = new DevMem();
-    DevMem& scal = *g_codec_scal[dev];
-    CK_TRY(scal.alloc(64, true));
-    CK_TRY(cudaMemsetAsync(scal.p, 0, 64, st));
-    long long* sc = scal.as<long long>();
-    CodecCall c = dense_call(x, dims, nz, ny, nx, const_cast<uint32_t*>(in), nwords, sc);
-    int* err = c.one.err;
-    // the header's version word says which mode wrote the stream
-    uint32_t hv[9] = {};
     if (nwords < 16) return CKFWI_CORRUPT;
-    CK_TRY(cudaMemcpyAsync(hv, in, sizeof(hv), cudaMemcpyDeviceToHost, st));
-    CK_TRY(cudaStreamSynchronize(st));
-    if ((hv[1] >> 8) == 2u) {
-        if (hv[8] < 1u || hv[8] > 32u) return CKFWI_CORRUPT;   // the rate word of a fixed-rate stream
-        c.rate = (int)hv[8];
-        CK_TRY(codec_rate_decompress_dev(c, st));
-    } else {
-        CK_TRY(codec_decompress_dev(c, st));
-    }
+    std::lock_guard<std::mutex> lk(g_codec_mu);
+    CodecDev* d = nullptr;
+    ST_TRY(codec_dev(st, &d));
+    CodecCall c = dense_call(x, dims, nz, ny, nx, const_cast<uint32_t*>(in), nwords, d->scal.as<long long>());
+    // the header's version word says which mode wrote the stream: each mode's
+    // decoder leaves the other's alone (asking the header first would cost a
+    // round trip to the host)
+    c.any = true;
+    CK_TRY(codec_decompress_dev(c, st));
+    CK_TRY(codec_rate_decompress_dev(c, st));
+    long long end = 0;
     int e = 0;
-    CK_TRY(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK_TRY(cudaStreamSynchronize(st));
+    ST_TRY(codec_wait(d, st, &end, &e));
     if (e & 4) return CKFWI_CORRUPT;
     return CKFWI_OK;
 }

@@ -63,7 +63,7 @@
 namespace ckfwi {
 namespace {
 
-constexpr uint32_t VERSION = 1u;
+constexpr uint32_t VERSION = VERSION_ACCURACY;
 constexpr int GUARD = 1;
 constexpr int ENC_THREADS = 64;
 constexpr int DEC_THREADS = 128;
@@ -622,6 +622,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_consta
         return;
     }
     const uint32_t* hdr = in + base;
+    if (call.any && (hdr[1] >> 8) == VERSION_RATE) return;
     if (hdr[0] != MAGIC || hdr[1] != ((uint32_t)G.dims | (VERSION << 8)) || hdr[2] != (uint32_t)G.nz ||
         hdr[3] != (uint32_t)G.ny || hdr[4] != (uint32_t)G.nx || hdr[5] != (uint32_t)G.nblocks ||
         hdr[6] != (uint32_t)G.nchunks || base + G.table_words + (long long)hdr[7] > cap_words) {

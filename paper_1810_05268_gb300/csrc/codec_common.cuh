@@ -12,6 +12,7 @@ namespace {
 
 constexpr uint32_t MAGIC = 0x31435442u;
 constexpr int HDR = 16;
+constexpr uint32_t VERSION_ACCURACY = 1u, VERSION_RATE = 2u;     // header word 1, bits 8 up
 constexpr int CHUNK = 32;
 
 template <int DIMS> struct Cfg {

@@ -31,7 +31,7 @@
 namespace ckfwi {
 namespace {
 
-constexpr uint32_t RATE_VERSION = 2u;
+constexpr uint32_t RATE_VERSION = VERSION_RATE;
 constexpr int RATE_EMIN = -100;
 constexpr int RT = 64;                 // threads (blocks) per CTA
 
@@ -242,12 +242,21 @@ __global__ void __launch_bounds__(RT) rate_dec_kernel(const __grid_constant__ Co
     float* __restrict__ x = A.f[call.src[fld]];
     int* err = A.err;
     const long long cap_words = A.cap_words;
-    const int rate = call.rate;
     const int tid = threadIdx.x;
     const long long b = (long long)blockIdx.x * RT + tid;
     if (b >= G.nblocks) return;
-    const int W = (int)rate_block_words(DIMS, rate);
     const long long base = A.base[call.from[fld]];
+    int rate = call.rate;
+    if (call.any) {                                  // a whole stream from the first word on: the header is there
+        if ((__ldg(in + base + 1) >> 8) != RATE_VERSION) return;
+        const uint32_t r = __ldg(in + base + 8);
+        if (r < 1u || r > 32u) {
+            atomicOr(err, 4);
+            return;
+        }
+        rate = (int)r;
+    }
+    const int W = (int)rate_block_words(DIMS, rate);
     if (base < 0 || base + HDR + G.nblocks * W > cap_words) {
         atomicOr(err, 4);
         return;
@@ -362,7 +371,7 @@ cudaError_t codec_rate_compress_dev(const CodecCall& c, cudaStream_t s)
 
 cudaError_t codec_rate_decompress_dev(const CodecCall& c, cudaStream_t s)
 {
-    if (c.rate < 1 || c.rate > 32) return cudaErrorInvalidValue;
+    if (!c.any && (c.rate < 1 || c.rate > 32)) return cudaErrorInvalidValue;
     const dim3 grd((unsigned)((c.blocks + RT - 1) / RT), (unsigned)(c.lanes * c.nf));
     if (c.dims == 3) rate_dec_kernel<3><<<grd, RT, 0, s>>>(c);
     else rate_dec_kernel<2><<<grd, RT, 0, s>>>(c);

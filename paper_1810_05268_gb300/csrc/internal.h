@@ -353,7 +353,8 @@ struct CodecCall {
     long long stat0;               // the fields' first entry of stat
     long long blocks;              // 4^d blocks of the largest lane
     float tol_f;                   // fixed accuracy: the bound
-    int rate;                      // fixed rate: bits per value
+    int rate;                      // fixed rate: bits per value; 0 in a decompression: as the stream says
+    bool any;                      // decompression: leave streams of the other mode alone
 };
 long long codec_blocks(int dims, int nz, int ny, int nx);
 cudaError_t codec_compress_dev(const CodecCall& c, cudaStream_t s);
