@@ -2156,6 +2156,35 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
     }
     long long ncomp = 0;   // compressions per lane
 
+    // a compressed checkpoint of (u, up) into a slot, on every lane
+    auto compress = [&](int slot, const Role& u, const Role& up) -> int {
+        if (cx.issue) {
+            // u^s and u^{s-1} of every lane; one field at a time where a
+            // lane's scratch serves only one
+            int nf = 2;
+            for (int l = 0; l < NL && !rc.rate; ++l) nf = std::min(nf, cx.lane(l)->scratch_fields);
+            const int fld[2] = {codec_field(u), codec_field(up)};
+            const int word[3] = {slot, rc.M + 1 + slot, slot + 1};
+            for (int k = 0; k < 2; k += nf) {
+                CodecCall c = codec_call(cx, rc, nf);
+                for (int i = 0; i < nf; ++i) {
+                    c.src[i] = fld[k + i];
+                    c.from[i] = word[k + i];
+                }
+                c.to = word[k + nf];
+                c.stat0 = ncomp + k;
+                const int tok = cx.begin(PC_COMP);
+                cx.count[PC_COMP] += nf - 1;   // counted by field
+                if (rc.rate) CK_TRY(codec_rate_compress_dev(c, cx.st));
+                else CK_TRY(codec_compress_dev(c, cx.st));
+                cx.end(tok);
+                cx.launches += 2;   // two launches in either mode
+            }
+        }
+        ncomp += 2;
+        return CKFWI_OK;
+    };
+
     State st{ZERO_R, ZERO_R, U_FP32, U_FP32};
     bool first_sweep = true;
     for (size_t ai = 0; ai < acts.size(); ++ai) {
@@ -2164,14 +2193,17 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
         const bool next_take = ai + 1 < acts.size() && acts[ai + 1].op == ACT_TAKESHOT;
         const bool next_turn = ai + 1 < acts.size() && acts[ai + 1].op == ACT_YOUTURN;
         if (A.op == ACT_ADVANCE && cx.several(false) && !cx.stage) {
-            // A run of forward steps with the checkpoints taken on the way
-            // (compressed ones end it: they read the state afterwards), in
+            // A run of forward steps with the checkpoints taken on the way, in
             // launches of several steps.  A checkpoint of state s takes level
-            // s and level s - 1 of the launch that makes level s.
+            // s and level s - 1 of the launch that makes level s; a compressed
+            // one takes them into the fields that restored states use in the
+            // reverse runs, and is coded when the launch is done.  (Launches
+            // that ended at every compressed checkpoint averaged 3.4 steps:
+            // half of their time was the state's way in and out.)
             const int n0 = A.a;
             int len = A.b;
             std::vector<std::pair<int, int>> takes;      // (level, slot), ascending
-            while (!rc.codec && ai + 1 < acts.size()) {
+            while (ai + 1 < acts.size()) {
                 const Action& B = acts[ai + 1];
                 if (B.op == ACT_TAKESHOT) takes.emplace_back(B.a - n0, B.b);
                 else if (B.op == ACT_ADVANCE) len += B.b;
@@ -2180,10 +2212,29 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
             }
             const int ck = rc.mode == CKFWI_STORE_BF16 ? CK_BF16 : rc.mode == CKFWI_STORE_FP16 ? CK_FP16 : CK_FP32;
             for (int i = 0; i < len;) {
-                const int T = block_of(len - i, STEP2_MAX);
+                int T = block_of(len - i, STEP2_MAX);
+                // levels (of the run) that compressed checkpoints take in this
+                // launch, in order; those before it are where the state is
+                std::vector<int> kept;
+                auto keep = [&](int lv) {
+                    if (lv > i && std::find(kept.begin(), kept.end(), lv) == kept.end()) kept.push_back(lv);
+                };
+                for (const auto& t : takes) {
+                    if (!rc.codec || t.first <= i || t.first > i + T) continue;
+                    std::vector<int> before = kept;
+                    keep(t.first - 1);
+                    keep(t.first);
+                    if (kept.size() > (size_t)CODEC_NF) {
+                        kept = before;
+                        T = t.first - 1 - i;             // up to, not including, this checkpoint
+                        break;
+                    }
+                }
                 Emits e32, e16;
                 Role out = pick_free(st), out2 = T > 1 ? pick_free(st, out) : st.cur;
+                for (size_t k = 0; k < kept.size(); ++k) e32.emplace_back(kept[k] - i, ures_r((int)k));
                 for (const auto& t : takes) {
+                    if (rc.codec) break;
                     if (t.first <= i || t.first > i + T) continue;
                     const int lv = t.first - i;
                     if (ck != CK_FP32) {
@@ -2204,6 +2255,13 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 }
                 ST_TRY(fwd_steps2(cx, st.cur, st.prev, n0 + i, T, first_sweep, e32, e16, ck));
                 fsteps += T;
+                auto level = [&](int lv) {
+                    const auto at = std::find(kept.begin(), kept.end(), lv);
+                    return at != kept.end() ? ures_r((int)(at - kept.begin())) : lv == i ? st.cur : st.prev;
+                };
+                for (const auto& t : takes)
+                    if (rc.codec && t.first > i && t.first <= i + T)
+                        ST_TRY(compress(t.second, level(t.first), level(t.first - 1)));
                 st = State{out, out2, U_FP32, U_FP32};
                 i += T;
             }
@@ -2275,32 +2333,7 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 st.tcur = U_FP32;
             }
         } else if (A.op == ACT_TAKESHOT) {
-            if (rc.codec) {
-                if (cx.issue) {
-                    // u^s and u^{s-1} of every lane; one field at a time where a
-                    // lane's scratch serves only one
-                    int nf = 2;
-                    for (int l = 0; l < NL && !rc.rate; ++l) nf = std::min(nf, cx.lane(l)->scratch_fields);
-                    const int fld[2] = {codec_field(st.cur), codec_field(st.prev)};
-                    const int word[3] = {A.b, rc.M + 1 + A.b, A.b + 1};
-                    for (int k = 0; k < 2; k += nf) {
-                        CodecCall c = codec_call(cx, rc, nf);
-                        for (int i = 0; i < nf; ++i) {
-                            c.src[i] = fld[k + i];
-                            c.from[i] = word[k + i];
-                        }
-                        c.to = word[k + nf];
-                        c.stat0 = ncomp + k;
-                        const int tok = cx.begin(PC_COMP);
-                        cx.count[PC_COMP] += nf - 1;   // counted by field
-                        if (rc.rate) CK_TRY(codec_rate_compress_dev(c, cx.st));
-                        else CK_TRY(codec_compress_dev(c, cx.st));
-                        cx.end(tok);
-                        cx.launches += 2;   // two launches in either mode
-                    }
-                }
-                ncomp += 2;
-            }
+            if (rc.codec) ST_TRY(compress(A.b, st.cur, st.prev));
         } else if (A.op == ACT_RESTORE) {
             if (A.b == 0) {
                 st = State{ZERO_R, ZERO_R, U_FP32, U_FP32};
