@@ -221,14 +221,10 @@ template <> __device__ __forceinline__ float up1<__nv_bfloat16>(__nv_bfloat16 v)
 template <class T>
 __global__ void upcast_kernel(const T* __restrict__ src, FieldGeom g, float* __restrict__ dst)
 {
-    const long long nvx = (g.nx + 3) / 4;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nvx * g.ny * g.nz) return;
-    const long long row = t / nvx;
-    const int x0 = (int)(t - row * nvx) * 4;
-    const long long y = row % g.ny, z = row / g.ny;
-    const long long o = z * g.pxy + y * g.px + x0;
-    if (x0 + 4 <= g.nx) {
+    const Quad q = quad_at(g, true);
+    if (!q.on) return;
+    const long long o = q.z * g.pxy + q.y * g.px + q.x0;
+    if (q.n == 4) {
         float4 r;
         if constexpr (sizeof(T) == 4) {
             r = __ldg(reinterpret_cast<const float4*>(src + o));
@@ -239,7 +235,7 @@ __global__ void upcast_kernel(const T* __restrict__ src, FieldGeom g, float* __r
         }
         *reinterpret_cast<float4*>(dst + o) = r;
     } else {
-        for (int i = 0; x0 + i < g.nx; ++i) dst[o + i] = up1<T>(src[o + i]);
+        for (int i = 0; i < q.n; ++i) dst[o + i] = up1<T>(src[o + i]);
     }
 }
 
