@@ -1776,7 +1776,7 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     };
     bool ff = forced("CKFWI_TILE_FWD", &m->tf, false), fa = forced("CKFWI_TILE_ADJ", &m->ta, true);
     // a 2D grid that fits the SMs takes the kernels of many steps a launch:
-    // nothing to time (281 x 281 and 464 x 1104: 1.8 and 3.1 us a forward
+    // nothing to time (281 x 281 and 464 x 1104: 1.5 and 3.1 us a forward
     // step, against 3.3 and 5.1 us of kernel time for one step a launch, and
     // 6.3 us when the host launches it)
     ff = ff || step2_tile({m}, false, &m->tf);

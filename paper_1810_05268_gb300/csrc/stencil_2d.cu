@@ -29,14 +29,16 @@
 // neighbours' waits then run out as well.
 //
 // Edge points are computed by the first half of the threads, four x points
-// each, interior points by the others, two rows at a time, straight from
-// shared memory.  The arithmetic is lap_at's and leapfrog's, on pairs of
+// each, interior points, the gradient's and the receivers by the threads
+// after them, straight from shared memory: a row each while there are threads
+// enough, else two rows at a time.  The arithmetic is lap_at's and leapfrog's, on pairs of
 // points (packed FP32x2, each lane rounding like the scalar operation), so
 // every value is bitwise the one the one-step kernels compute.  u^{n+1}
 // overwrites u^{n-1} point by point.
 //
 // Measured, from set_model to the data on one GB300: 281 x 281, 500 steps
-// 3.21 -> 1.01 ms; 464 x 1104, 2000 steps 12.5 -> 6.4 ms.  What bounds it: a
+// 3.21 -> 0.97 ms (1.5 us a step, a reverse step 2.7); 464 x 1104, 2000 steps
+// 12.5 -> 6.4 ms (3.1 and 6.5).  What bounds it: a
 // step's chain is an edge vector (about 1000 cycles: a lone warp issues an
 // instruction every 6 cycles), the exchange (1350 cycles between two CTAs
 // that do nothing else) and the interior beside it.  Two points a thread (1024
@@ -296,21 +298,25 @@ struct Cta2 {
     }
 };
 
-// `rows` rows of `nq` vectors as row pairs over all threads, the threads that
-// compute no edges first
-struct Pair2 {
-    int nq, rows, n, r, q;
-    __device__ __forceinline__ Pair2(int nq_, int rows_) : nq(max(nq_, 1)), rows(rows_)
+// `rows` rows of `nq` vectors over the threads from `start` on (all of them,
+// in turn): a row each while `idle` threads suffice, else row pairs (they
+// share their z neighbours)
+struct Rows2 {
+    int nq, rows, rp, n, start, r, q;
+    __device__ __forceinline__ Rows2(int nq_, int rows_, int start_, int idle) : nq(max(nq_, 1)), rows(rows_), start(start_)
     {
-        n = nq_ > 0 && rows_ > 0 ? (rows_ + 1) / 2 * nq_ : 0;
+        const int all = nq_ > 0 && rows_ > 0 ? nq_ * rows_ : 0;
+        rp = all <= idle ? 1 : 2;
+        n = rp == 1 ? all : (rows_ + 1) / 2 * nq_;
+        if (all == 0) n = 0;
         set(first());
     }
-    __device__ __forceinline__ static int first() { return (int)(threadIdx.x + NE2) % NT2; }
+    __device__ __forceinline__ int first() const { return ((int)threadIdx.x - start + NT2) % NT2; }
     __device__ __forceinline__ void set(int i)
     {
         const int p = i / nq;
         q = i - p * nq;
-        r = 2 * p;
+        r = rp * p;
     }
 };
 
@@ -397,16 +403,16 @@ struct Take2 {
 };
 
 // What every step repeats, worked out once: the thread's first edge vector,
-// its first vector to take and its first pair of interior rows
+// its first vector to take and its first interior rows
 template <int K>
 struct Plan2 {
     Cta2<K> ct;
     int nz, nx, n_edge, n_take;
     Edge2 edge;
     Take2 take;
-    Pair2 in;
+    Rows2 in;
     __device__ __forceinline__ Plan2(const Step2Args& a, int b)
-        : ct(a, b), nz(a.g.nz), nx(a.g.nx), in(ct.interior() ? ct.wq - 2 * ct.PQ : 0, ct.h - 2 * K)
+        : ct(a, b), nz(a.g.nz), nx(a.g.nx), in(ct.interior() ? ct.wq - 2 * ct.PQ : 0, ct.h - 2 * K, NE2, NT2 - NE2)
     {
         const int tid = threadIdx.x;
         n_edge = tid < NE2 ? ct.edges() : 0;
@@ -515,7 +521,17 @@ __device__ __forceinline__ void step2(const Plan2<K>& pl, const Step2Env<K>& ev,
     }
     // (Beside the interior the edges would share the issue slots with it and
     // leave twice as late: 1900 cycles against 950 at 464 x 1104.)
-    Pair2 pr = pl.in;
+    Rows2 pr = pl.in;
+    if (pr.rp == 1) {
+        if (pr.first() < pr.n) {                  // a row each: one round
+            float win[2 * K + 1][4], v[4];
+            const int r = pr.r + K, q = pr.q + ct.PQ;
+            window2<K, 1>(win, ev.b1, ct.t.pitch, r, q);
+            update2<K>(v, ct, win, ev, in, series, pl.nx, r, q);
+            emit(r, q, win[K], v);
+        }
+        return;
+    }
     for (int i = pr.first(); i < pr.n; i += NT2) {
         if (i >= NT2) pr.set(i);
         float win[2 * K + 2][4], v[4];
@@ -586,8 +602,9 @@ __device__ __forceinline__ void fwd2_body(const Step2Args& a, int b, float* sm)
     cp_wait();
     __syncthreads();
     const int listed = nrl;
+    const int spos = (tid - NE2 - pl.in.n % NT2 + 2 * NT2) % NT2;    // the threads after those of the interior sample
     for (int i = 0; i < a.T; ++i) {
-        // receivers of level n + i, by the threads that compute no edges
+        // receivers of level n + i
         auto sample = [&](int r) {
             const int2 at = a.rzx[r];
             const float* p = ev.b1 + (at.x - ct.zt + K) * t.pitch + at.y - ct.xt + ct.PX;
@@ -599,8 +616,7 @@ __device__ __forceinline__ void fwd2_body(const Step2Args& a, int b, float* sm)
             a.smp.out[(long long)i * a.smp.n + r] = acc;
         };
         if (listed <= RL2) {
-            for (int k = tid - NE2; k < listed; k += NT2 - NE2)
-                if (k >= 0) sample(rl[k]);
+            for (int k = spos; k < listed; k += NT2) sample(rl[k]);
         } else {
             for (int r = tid; r < a.smp.n; r += NT2)
                 if (mine(r)) sample(r);
@@ -660,7 +676,9 @@ __device__ __forceinline__ void adj2_body(const Step2Args& a, int b, float* sm)
     load_u(0);
     cp_wait();
     ev.damped = __syncthreads_or(damped);
-    const Pair2 gp0(ct.wq, ct.h);
+    // the gradient's rows by the threads after those of the interior (by the
+    // same ones, a small tile's step was the sum of both: 4.4 us at 281 x 281)
+    const Rows2 gp0(ct.wq, ct.h, (NE2 + pl.in.n) % NT2, NT2 - NE2 - pl.in.n);
     // Phase i: step i of lam, and the gradient of step i - 1, whose lam (now
     // b1) the barrier before has completed.  The u tile that phase i + 1 needs
     // replaces the one that the gradient of phase i - 1 has read.
@@ -678,7 +696,7 @@ __device__ __forceinline__ void adj2_body(const Step2Args& a, int b, float* sm)
                      });
         if (i > 0) {
             const float* ub = us + ((i - 1) & 1) * t.plane();
-            Pair2 pr = gp0;
+            Rows2 pr = gp0;
             for (int k = pr.first(); k < pr.n; k += NT2) {
                 if (k >= NT2) pr.set(k);
                 float win[2 * K + 2][4];
@@ -687,7 +705,7 @@ __device__ __forceinline__ void adj2_body(const Step2Args& a, int b, float* sm)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int r = pr.r + h, o = (K + r) * t.pitch + ct.PX + 4 * pr.q;
-                    if (r >= ct.h) break;
+                    if (h >= pr.rp || r >= ct.h) break;
                     float s[4], lv[4], gv[4];
                     sld<4>(lv, ev.b1 + o);
                     float* gp = gs + r * t.bx + 4 * pr.q;
