@@ -107,9 +107,9 @@ def roofline_block(H, nt, npts, peak, peak_kind, delta=0.0):
     per-call overhead `delta` [ms] that adds (measured on the store-all
     gradient against its graph replay) is taken off each call's time."""
     F = max(1.0, H["ratio_mean"] or 1.0)
-    # a step that writes an FP32 or 16-bit checkpoint writes 4 more B/pt
-    # (u^{n-1} in FP32, or both levels in 16 bits), W of the launches
-    ck_bytes = 4.0 if H["store_mode"] in ("fp32", "fp16", "bf16") and H["ckpt_slots"] < nt else 0.0
+    # a step that writes a 16-bit checkpoint writes 4 more B/pt (both levels
+    # in 16 bits), W of the launches; FP32 ones are written in place
+    ck_bytes = 4.0 if H["store_mode"] in ("fp16", "bf16") and H["ckpt_slots"] < nt else 0.0
     fwd_b = (FWD_BYTES + ck_bytes * H["W"] / max(1, H["fwd_launches"])) * npts
     classes = {
         "fwd": (H["fwd_ms"], H["fwd_launches"], fwd_b),
