@@ -2157,8 +2157,36 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
     long long ncomp = 0;   // compressions per lane
 
     // a compressed checkpoint of (u, up) into a slot, on every lane
-    auto compress = [&](int slot, const Role& u, const Role& up) -> int {
-        if (cx.issue) {
+    //
+    // A checkpoint one step after another, with nothing restored in between,
+    // holds that one's u^s as its u^{s-1}: the same field, so the same stream,
+    // which lies in the slot below as long as this one lives (slots are a
+    // stack).  It is not coded again.  (At 208^3, 500 steps and 116 slots 416
+    // of 471 checkpoints follow one another like that: the gradient takes 93.2
+    // ms against 100.4 with both fields coded every time.)
+    int took_slot = 0, took_level = -1;                    // the last checkpoint, of the state at hand
+    std::vector<int> prev_word((size_t)rc.M + 1, 0);       // the word where a slot's u^{s-1} starts
+    auto compress = [&](int slot, int level, const Role& u, const Role& up) -> int {
+        const bool follows = took_slot > 0 && took_slot == slot - 1 && took_level == level - 1;
+        prev_word[slot] = follows ? took_slot : rc.M + 1 + slot;
+        took_slot = slot;
+        took_level = level;
+        if (cx.issue && follows) {
+            CodecCall c = codec_call(cx, rc, 1);
+            c.src[0] = codec_field(u);
+            c.from[0] = slot;
+            c.from[1] = rc.M + 1 + slot;
+            c.to = slot + 1;
+            c.dup = slot - 1;
+            c.dup_end = rc.M + 1 + slot - 1;
+            c.stat0 = ncomp;
+            const int tok = cx.begin(PC_COMP);
+            cx.count[PC_COMP] += 1;                        // by field stored
+            if (rc.rate) CK_TRY(codec_rate_compress_dev(c, cx.st));
+            else CK_TRY(codec_compress_dev(c, cx.st));
+            cx.end(tok);
+            cx.launches += 2;
+        } else if (cx.issue) {
             // u^s and u^{s-1} of every lane; one field at a time where a
             // lane's scratch serves only one
             int nf = 2;
@@ -2269,7 +2297,7 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 };
                 for (const auto& t : takes)
                     if (rc.codec && t.first > i && t.first <= i + T)
-                        ST_TRY(compress(t.second, level(t.first), level(t.first - 1)));
+                        ST_TRY(compress(t.second, n0 + t.first, level(t.first), level(t.first - 1)));
                 st = State{out, out2, U_FP32, U_FP32};
                 i += T;
             }
@@ -2357,8 +2385,9 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 st.tcur = U_FP32;
             }
         } else if (A.op == ACT_TAKESHOT) {
-            if (rc.codec) ST_TRY(compress(A.b, st.cur, st.prev));
+            if (rc.codec) ST_TRY(compress(A.b, A.a, st.cur, st.prev));
         } else if (A.op == ACT_RESTORE) {
+            took_slot = 0;
             if (A.b == 0) {
                 st = State{ZERO_R, ZERO_R, U_FP32, U_FP32};
             } else if (rc.mode == CKFWI_STORE_FP32 && cx.stage && A.b <= cx.m->host_slots) {
@@ -2438,7 +2467,7 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 c.src[0] = codec_field(work_r(0));
                 c.src[1] = codec_field(work_r(1));
                 c.from[0] = A.b;
-                c.from[1] = rc.M + 1 + A.b;
+                c.from[1] = prev_word[A.b];
                 ST_TRY(decompress(cx, rc, c));
                 st = State{work_r(0), work_r(1), U_FP32, U_FP32};
             } else if (next_turn) {

@@ -555,7 +555,8 @@ __global__ void __launch_bounds__(CMP_THREADS) compact_kernel(const __grid_const
     const bool fits = end <= cap_words;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (!fits) atomicOr(A.err, 2);
-        A.base[fld + 1 < call.nf ? call.from[1] : call.to] = fits ? end : base;
+        if (fld + 1 < call.nf) A.base[call.from[1]] = fits ? end : base;
+        else end_streams(call, A, fits ? end : base);
         if (A.stat) atomicAdd(A.stat + call.stat0 + fld, (unsigned long long)(G.table_words + total));
     }
     if (!fits) return;                                 // overflow: nothing is written

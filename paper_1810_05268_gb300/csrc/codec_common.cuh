@@ -187,6 +187,20 @@ __device__ __forceinline__ const CodecLane& item_of(const CodecCall& c, int& k)
     return c.tab ? c.tab[l] : c.one;
 }
 
+// The pool's next word after a call's last stream, which ends at word e: a
+// stream that `dup` stands for keeps its room (and its overflow) as if written.
+__device__ __forceinline__ void end_streams(const CodecCall& c, const CodecLane& A, long long e)
+{
+    if (c.dup) {
+        const long long w = A.base[c.dup_end] - A.base[c.dup];
+        A.base[c.from[1]] = e;
+        if (A.stat) A.stat[c.stat0 + 1] = (unsigned long long)w;
+        if (e + w <= A.cap_words) e += w;
+        else atomicOr(A.err, 2);
+    }
+    A.base[c.to] = e;
+}
+
 // block coordinates and clamped sample positions
 struct BlockPos { int bz, by, bx; };
 __device__ __forceinline__ BlockPos block_pos(const Geo& G, long long b)

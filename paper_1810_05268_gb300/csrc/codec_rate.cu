@@ -91,7 +91,8 @@ __global__ void rate_header_kernel(const __grid_constant__ CodecCall c)
     const bool fits = base + total <= A.cap_words;
     if (threadIdx.x == 0) {
         if (!fits) atomicOr(A.err, 2);
-        A.base[fld + 1 < c.nf ? c.from[1] : c.to] = fits ? base + total : base;
+        if (fld + 1 < c.nf) A.base[c.from[1]] = fits ? base + total : base;
+        else end_streams(c, A, fits ? base + total : base);
         if (fits && A.stat) A.stat[c.stat0 + fld] = (unsigned long long)total;
     }
     if (fits && threadIdx.x < HDR) {

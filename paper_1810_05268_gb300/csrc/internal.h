@@ -343,13 +343,17 @@ struct CodecLane {
 // Compression (nf 1 or 2): the streams follow one another in the pool, field
 // 0's from the word in base[from[0]]; field 0's end goes to base[from[1]]
 // (nf = 2), the last field's to base[to].  Decompression: field k's stream
-// starts at the word in base[from[k]].  One lane is passed by value, several
-// by a device table.
+// starts at the word in base[from[k]].  A compression of one field with dup set
+// stands for two: the second is, word for word, the stream that lies from
+// base[dup] to base[dup_end].  Its room and statistics are counted, its words
+// are not written; readers start at base[dup].  One lane is passed by value,
+// several by a device table.
 struct CodecCall {
     CodecLane one;
     const CodecLane* tab;          // null: `one` alone
     int lanes, nf, dims;
     int src[CODEC_NF], from[CODEC_NF], to;
+    int dup, dup_end;              // compression of one field: see above; 0: no second stream
     long long stat0;               // the fields' first entry of stat
     long long blocks;              // 4^d blocks of the largest lane
     float tol_f;                   // fixed accuracy: the bound
