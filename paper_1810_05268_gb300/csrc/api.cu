@@ -877,6 +877,20 @@ Tile ot4_host_tile(const Tile& t)
     return v;
 }
 
+// The tile of a pass fed by tensor copies: its own when tuned, else the step's
+const Tile& ot4q_tile(const ckfwi_model* m, int op, const Tile& t) { return m->t4[op].ver == 10 ? m->t4[op] : t; }
+
+// The tile of the launch that samples a forward step's receivers (the step
+// reads u and up): an OT4 step's pass 1, which has a z run of its own, and
+// the stand-ins of steps that read host slots
+Tile sampling_tile(const ckfwi_model* m, const Role& u, const Role& up)
+{
+    if (m->tf.ver == 10)
+        return in_host(m, u) || in_host(m, up) ? ot4_host_tile(m->tf) : ot4q_tile(m, OT4Q_LAP, m->tf);
+    if (m->tf.ver == 2 && in_host(m, u)) return host_tile(m);
+    return m->tf;
+}
+
 int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by, CUtensorMap* out);
 
 // OT4 steps (ot4.cu): forward, the pass computing w lap f, then the update;
@@ -891,7 +905,7 @@ int ot4q_pass(ckfwi_model* m, int op, const Ot4qArgs& a, std::initializer_list<c
     ST_TRY(tensor_map(m, a.s, U_FP32, tq_box_x(m->K), tq_box_y(m->K), &mp[0]));
     int k = 1;
     for (const float* p : points) ST_TRY(tensor_map(m, p, U_FP32, 32, 16, &mp[k++]));
-    CK_TRY(launch_ot4q(op, a, mp, m->t4[op].ver == 10 ? m->t4[op] : t, m->K, ck, st));
+    CK_TRY(launch_ot4q(op, a, mp, ot4q_tile(m, op, t), m->K, ck, st));
     return CKFWI_OK;
 }
 
@@ -1107,8 +1121,8 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
                 ST_TRY(check_field(m, cm, ck_up, a.ck_up, "forward step: checkpoint u^{s-1}"));
             }
         }
-        const Tile& t = cx.batch ? cx.bf : m->tf;
-        const int zlen = cx.batch ? cx.zf[l] : m->tf.zlen;
+        const Tile t = cx.batch ? cx.bf : sampling_tile(m, u, up);
+        const int zlen = cx.batch ? cx.zf[l] : t.zlen;
         bool sep = false;
         if (record) {
             const Sample sm = sample_of(m, n);
@@ -1775,6 +1789,7 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         return true;
     };
     bool ff = forced("CKFWI_TILE_FWD", &m->tf, false), fa = forced("CKFWI_TILE_ADJ", &m->ta, true);
+    forced("CKFWI_TILE_OT4_LAP", &m->t4[OT4Q_LAP], false);   // pass 1 of an OT4 step, as tuning leaves it
     // a 2D grid that fits the SMs takes the kernels of many steps a launch:
     // nothing to time (281 x 281 and 464 x 1104: 1.5 and 3.1 us a forward
     // step, against 3.3 and 5.1 us of kernel time for one step a launch, and
