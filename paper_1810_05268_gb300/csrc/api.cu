@@ -1929,13 +1929,13 @@ int read_flags(ckfwi_model* m, cudaStream_t st, int* fl)
     if (h[1] & 2) *fl = CKFWI_POOL_OVERFLOW;
     else if (h[1] & 4) *fl = CKFWI_CORRUPT;
     else if (h[0] & 8) *fl = CKFWI_TIMEOUT;
+    else if ((h[0] & 1) || (h[1] & 1)) *fl = CKFWI_NONFINITE;
     // a launch of many steps that gave up leaves its tiles at different steps
     if (h[0] & 8)
         for (auto& x : m->xch) {
             CK_TRY(cudaMemset(x.second.buf.p, 0, x.second.buf.bytes));
             CK_TRY(cudaMemset(x.second.epoch.p, 0, x.second.epoch.bytes));
         }
-    else if ((h[0] & 1) || (h[1] & 1)) *fl = CKFWI_NONFINITE;
     return CKFWI_OK;
 }
 
