@@ -618,12 +618,15 @@ __global__ void __launch_bounds__(DEC_THREADS, 5) dec_kernel(const __grid_consta
     const long long c = b / CHUNK;
     if (c >= G.nchunks) return;                    // whole warp
     const long long base = A.base[call.from[fld]];
+    // a stream of the other mode is left alone before its length is looked at:
+    // it may be shorter than this mode's table (the caller has seen that it
+    // holds a header)
+    if (call.any && (in[base + 1] >> 8) == VERSION_RATE) return;
     if (base < 0 || base + G.table_words > cap_words) {
         if (lane == 0) atomicOr(err, 4);
         return;
     }
     const uint32_t* hdr = in + base;
-    if (call.any && (hdr[1] >> 8) == VERSION_RATE) return;
     if (hdr[0] != MAGIC || hdr[1] != ((uint32_t)G.dims | (VERSION << 8)) || hdr[2] != (uint32_t)G.nz ||
         hdr[3] != (uint32_t)G.ny || hdr[4] != (uint32_t)G.nx || hdr[5] != (uint32_t)G.nblocks ||
         hdr[6] != (uint32_t)G.nchunks || base + G.table_words + (long long)hdr[7] > cap_words) {
