@@ -302,6 +302,7 @@ struct GraphExec {
 };
 
 constexpr size_t MAX_GRAPHS = 8;   // recorded graphs kept per model
+constexpr long long WAIT_LIMIT = 1LL << 22;   // back-off rounds of a bounded wait in the kernels
 
 // Tile shape and per-lane z-run lengths of a batch of lanes.
 struct BatchTiles {
@@ -353,7 +354,7 @@ struct ckfwi_model {
     DevMem pool;                    // checkpoint pool
     HostMem hpool;                  // checkpoint slots in host memory (second level)
     int host_slots = 0;             // slots 1 .. host_slots live in hpool
-    long long wait_limit = 1LL << 22;   // TMA kernels: back-off rounds of a plane's wait
+    long long wait_limit = WAIT_LIMIT;
     size_t pool_cap_bytes = 0;
     int pool_tag = -1;              // storage mode whose layout the pool holds
     DevMem slotbase;                // codec: device word offsets of slots
@@ -1913,8 +1914,22 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     return CKFWI_OK;
 }
 
+// Bound of the kernels' waits: CKFWI_TMA_WAIT_LIMIT < 0 makes them run out at
+// once (the test of the CKFWI_TIMEOUT path; the copies in flight are still
+// waited for before a CTA leaves).  Read by every call; recorded graphs hold
+// the bound they were recorded with.
+void read_wait_limit(ckfwi_model* m)
+{
+    const char* v = std::getenv("CKFWI_TMA_WAIT_LIMIT");
+    const long long limit = v ? std::atoll(v) : WAIT_LIMIT;
+    if (limit != m->wait_limit) ++m->gen;
+    m->wait_limit = limit;
+}
+
+// start of a call's launches
 int reset_flags(ckfwi_model* m, cudaStream_t st)
 {
+    read_wait_limit(m);
     CK_TRY(cudaMemsetAsync(m->flags.p, 0, m->flags.bytes, st));
     return CKFWI_OK;
 }
@@ -1931,11 +1946,14 @@ int read_flags(ckfwi_model* m, cudaStream_t st, int* fl)
     else if (h[0] & 8) *fl = CKFWI_TIMEOUT;
     else if ((h[0] & 1) || (h[1] & 1)) *fl = CKFWI_NONFINITE;
     // a launch of many steps that gave up leaves its tiles at different steps
-    if (h[0] & 8)
+    // (waited for: the next call may come on any stream)
+    if (h[0] & 8) {
         for (auto& x : m->xch) {
-            CK_TRY(cudaMemset(x.second.buf.p, 0, x.second.buf.bytes));
-            CK_TRY(cudaMemset(x.second.epoch.p, 0, x.second.epoch.bytes));
+            CK_TRY(cudaMemsetAsync(x.second.buf.p, 0, x.second.buf.bytes, st));
+            CK_TRY(cudaMemsetAsync(x.second.epoch.p, 0, x.second.epoch.bytes, st));
         }
+        CK_TRY(cudaStreamSynchronize(st));
+    }
     return CKFWI_OK;
 }
 
@@ -3454,10 +3472,6 @@ int ckfwi_create_model(const ckfwi_grid* g, ckfwi_model** out)
     if (g->dims == 2) m->g.n[1] = 1;
     m->K = g->space_order / 2;
     m->fg = make_geom(g->dims, g->n[0], m->g.n[1], g->n[2], m->K);
-    // CKFWI_TMA_WAIT_LIMIT < 0 makes the TMA kernels' waits run out at once
-    // (the test of the CKFWI_TIMEOUT path; the copies in flight are still
-    // waited for before a CTA leaves)
-    if (const char* wl = std::getenv("CKFWI_TMA_WAIT_LIMIT")) m->wait_limit = std::atoll(wl);
     double c[MAXK + 1];
     fd_weights(m->K, c);
     const double ih2 = 1.0 / (g->h * g->h);
