@@ -341,8 +341,8 @@ struct ckfwi_model {
                                     // last two reverse steps (alternating by step parity)
     bool have_model = false;
     DevMem eta, w, cvel, zero, uN;
-    DevMem work[4], lam[4], gacc;   // the fourth: 2D, where a launch of several steps writes two levels
-    DevMem ures[CODEC_NF];          // 2D codec: restored states of one launch of reverse steps
+    DevMem work[4], lam[4], gacc;   // the fourth: grids that launches of several 2D steps take (they write two levels)
+    DevMem ures[CODEC_NF];          // codec, launches of several 2D steps: states kept for it, restored for them
     // 2D: the exchange buffer and step counts of launches of many steps, by
     // tile and direction (a buffer is only ever used with one tile: an old
     // value of another layout could look like an awaited one)
@@ -1229,10 +1229,8 @@ std::vector<int> step2_groups(const std::vector<ckfwi_model*>& lanes, const Tile
 // its launch).
 bool step2_tile(const std::vector<ckfwi_model*>& lanes, bool reverse, Tile* out)
 {
-    ckfwi_model* m = lanes[0];
+    const ckfwi_model* m = lanes[0];
     if (m->fg.dims != 2 || m->ot != 2) return false;
-    for (ckfwi_model* L : lanes)
-        if (!L->work[3].p) return false;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
@@ -1776,7 +1774,8 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         if (nf < 6) u.pf = 0;
         if ((u.ver == 5 || u.ver == 6 || u.ver == 10) != (m->ot == 4)) return false;
         const bool okv = u.ver == 10  ? encode_fn() && ot4q_supported(f.dims, m->K, u) && v3_fits(f, m->K)
-                         : u.ver == 9 ? m->ot == 2 && step2_supported(f.dims, m->K, u, reverse) && tiles_of(f, u) <= nsm
+                         : u.ver == 9 ? (reverse ? m->lam[3].p : m->work[3].p) &&
+                                            step2_supported(f.dims, m->K, u, reverse) && tiles_of(f, u) <= nsm
                          : u.ver == 8 ? tma_ok && tq_supported(f.dims, m->K, u) && v3_fits(f, m->K)
                          : u.ver == 7 ? v5_supported(f.dims, m->K, u) && v3_fits(f, m->K)
                          : u.ver == 6 ? ot4v_supported(f.dims, m->K, u, reverse) && v3_fits(f, m->K)
@@ -1901,11 +1900,8 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     if (m->tf.ver == 9) ST_TRY(step2_exchange(m, m->tf, false, &x2));
     if (m->ta.ver == 9) ST_TRY(step2_exchange(m, m->ta, true, &x2));
     // the probe runs wrote into working buffers; clear them
-    for (int i = 0; i < 4; ++i) {
-        if (!m->work[i].p) continue;
-        CK_TRY(cudaMemsetAsync(m->work[i].p, 0, m->work[i].bytes, st));
-        CK_TRY(cudaMemsetAsync(m->lam[i].p, 0, m->lam[i].bytes, st));
-    }
+    for (DevMem* d : {m->work, m->lam})
+        for (int i = 0; i < 4 && d[i].p; ++i) CK_TRY(cudaMemsetAsync(d[i].p, 0, d[i].bytes, st));
     CK_TRY(cudaMemsetAsync(m->gacc.p, 0, m->gacc.bytes, st));
     for (int i = 0; i < 3; ++i)
         if (m->z4[i].p) CK_TRY(cudaMemsetAsync(m->z4[i].p, 0, m->z4[i].bytes, st));
@@ -2607,16 +2603,16 @@ double storage_bytes(const FieldGeom& f, const RunCfg& rc, const ckfwi_grad_opts
 int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
 {
     const FieldGeom& f = m->fg;
-    const void* before[8] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d, m->ures[0].p,
+    const void* before[7] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d,
                              reinterpret_cast<const void*>((intptr_t)m->host_slots)};
     struct Bump {
         ckfwi_model* m;
         const void* const* b;
         ~Bump()
         {
-            const void* after[8] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d, m->ures[0].p,
+            const void* after[7] = {m->traj.p, m->pool.p, m->slotbase.p, m->scratch.p, m->statw.p, m->hpool.d,
                                     reinterpret_cast<const void*>((intptr_t)m->host_slots)};
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 7; ++i)
                 if (after[i] != b[i]) ++m->gen;
         }
     } bump{m, before};
@@ -2692,8 +2688,18 @@ int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
             CK_TRY(e);
         }
         CK_TRY(m->statw.alloc(sizeof(unsigned long long) * (size_t)(4 * rc.N + 8)));
-        for (int i = 0; m->work[3].p && i < CODEC_NF; ++i) CK_TRY(m->ures[i].alloc(field_bytes(f)));
     }
+    return CKFWI_OK;
+}
+
+// The fields that compressed states go through in launches of several 2D
+// steps, where the run's forward or reverse steps (tf, ta) are such launches
+int prepare_states(ckfwi_model* m, const RunCfg& rc, const Tile& tf, const Tile& ta)
+{
+    if (!rc.codec || rc.M <= 1 || (tf.ver != 9 && ta.ver != 9)) return CKFWI_OK;
+    const void* before = m->ures[0].p;
+    for (DevMem& d : m->ures) CK_TRY(d.alloc(field_bytes(m->fg)));
+    if (m->ures[0].p != before) ++m->gen;
     return CKFWI_OK;
 }
 
@@ -2847,6 +2853,7 @@ int gradient_one(ckfwi_model* m, const ckfwi_shot* s, const float* d_obs, int me
     const FieldGeom& f = m->fg;
     const RunCfg rc = run_cfg(m->g.nt, o);
     ST_TRY(prepare_storage(m, rc, o));
+    ST_TRY(prepare_states(m, rc, m->tf, m->ta));
     const size_t nd = (size_t)(rc.N + 1) * m->shot.nrec;
     CK_TRY(cudaMemcpyAsync(m->shot.dobs.p, d_obs, nd * sizeof(float),
                            mem == CKFWI_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
@@ -3193,11 +3200,8 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
     if (bt.zf.empty() || bt.za.empty()) return CKFWI_EINVAL;
     // the probes wrote into working buffers; clear them
     for (ckfwi_model* L : lanes) {
-        for (int i = 0; i < 4; ++i) {
-            if (!L->work[i].p) continue;
-            CK_TRY(cudaMemsetAsync(L->work[i].p, 0, L->work[i].bytes, st));
-            CK_TRY(cudaMemsetAsync(L->lam[i].p, 0, L->lam[i].bytes, st));
-        }
+        for (DevMem* d : {L->work, L->lam})
+            for (int i = 0; i < 4 && d[i].p; ++i) CK_TRY(cudaMemsetAsync(d[i].p, 0, d[i].bytes, st));
         CK_TRY(cudaMemsetAsync(L->gacc.p, 0, L->gacc.bytes, st));
     }
     CK_TRY(cudaStreamSynchronize(st));
@@ -3227,6 +3231,7 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
     const BatchTiles* bt = nullptr;
     ST_TRY(batch_tune(lanes, st, &bt));
     for (int l = 0; l < NL; ++l) {
+        ST_TRY(prepare_states(lanes[l], rc, bt->tf, bt->ta));
         ckfwi_model* L = lanes[l];
         const size_t nd = (size_t)(rc.N + 1) * L->shot.nrec;
         CK_TRY(cudaMemcpyAsync(L->shot.dobs.p, d_obs[l], nd * sizeof(float),
@@ -3437,18 +3442,33 @@ int ensure_clones(ckfwi_model* m, int k, cudaStream_t st)
     return CKFWI_OK;
 }
 
+// Device bytes of one more lane of a model: ten fields and the checkpoint
+// storage; where launches of several 2D steps take the grid, their fourth
+// fields, their exchange buffers and the fields compressed states go through.
+double lane_bytes(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
+{
+    double n = 10.0 * field_bytes(m->fg) + 8.0 * m->fg.npts + storage_bytes(m->fg, rc, o);
+    Tile t;
+    for (bool reverse : {false, true})
+        if (step2_tile({m}, reverse, &t))
+            n += (double)field_bytes(m->fg) + (double)step2_exchange_bytes(m->K, t, tiles_of(m->fg, t));
+    if (rc.codec && rc.M > 1 && (m->work[3].p || m->lam[3].p)) n += (double)CODEC_NF * field_bytes(m->fg);
+    return n;
+}
+
 // How many shots of one model run side by side: bounded by free device
-// memory (a lane holds ten fields and its checkpoint storage), by
-// CKFWI_MAX_LANES (default 64) and by the shot count.
+// memory (CKFWI_FREE_BYTES in its place), by CKFWI_MAX_LANES (default 64)
+// and by the shot count.
 int batch_width(ckfwi_model* m, int nshots, const ckfwi_grad_opts* o)
 {
     if (m->ot == 4) return 1;     // the OT4 kernels have no batched form: one shot at a time
     int cap = 64;
     if (const char* v = std::getenv("CKFWI_MAX_LANES")) cap = std::max(1, std::atoi(v));
     const RunCfg rc = run_cfg(m->g.nt, o);
-    const double lane = 10.0 * field_bytes(m->fg) + 8.0 * m->fg.npts + storage_bytes(m->fg, rc, o);
+    const double lane = lane_bytes(m, rc, o);
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return 1;
+    if (const char* v = std::getenv("CKFWI_FREE_BYTES")) fr = (size_t)std::max(0LL, std::atoll(v));
     const double extra = 0.8 * (double)fr / lane;
     const long long w = 1 + (long long)m->clones.size() + (long long)extra;
     return (int)std::max<long long>(1, std::min<long long>({(long long)nshots, (long long)cap, w}));
@@ -3491,10 +3511,13 @@ int ckfwi_create_model(const ckfwi_grid* g, ckfwi_model** out)
     CK_TRY(m->cvel.alloc((size_t)f.npts * sizeof(float)));
     CK_TRY(m->zero.alloc(field_bytes(f)));
     CK_TRY(m->uN.alloc(field_bytes(f)));
-    for (int i = 0; i < (g->dims == 2 && m->ot == 2 ? 4 : 3); ++i) {
-        CK_TRY(m->work[i].alloc(field_bytes(f)));
-        CK_TRY(m->lam[i].alloc(field_bytes(f)));
-    }
+    // the fourth fields where launches of many steps take the grid (a batch's
+    // lanes take them in its tile only if each takes them alone: the tile that
+    // is as small as a lane's count of columns and rows allows fits too)
+    Tile many;
+    const int nwork = step2_tile({m}, false, &many) ? 4 : 3, nlam = step2_tile({m}, true, &many) ? 4 : 3;
+    for (int i = 0; i < nwork; ++i) CK_TRY(m->work[i].alloc(field_bytes(f)));
+    for (int i = 0; i < nlam; ++i) CK_TRY(m->lam[i].alloc(field_bytes(f)));
     CK_TRY(m->gacc.alloc(field_bytes(f)));
     if (m->ot == 4)
         for (int i = 0; i < 3; ++i) CK_TRY(m->z4[i].alloc(field_bytes(f)));   // halos stay zero
