@@ -359,7 +359,7 @@ struct ckfwi_model {
     int pool_tag = -1;              // storage mode whose layout the pool holds
     DevMem slotbase;                // codec: device word offsets of slots
     DevMem scratch;                 // codec scratch
-    int scratch_fields = 0;         // fields it serves at once: 2 (a takeshot's pair), or 1 when memory is short
+    int scratch_fields = 0;         // fields it serves at once: 2 (a takeshot's pair), or 1 where memory served no more
     DevMem flags;                   // int error flags
     DevMem phi, partials;
     DevMem statw;                   // codec: words per compression
@@ -2677,13 +2677,24 @@ int prepare_storage(ckfwi_model* m, const RunCfg& rc, const ckfwi_grad_opts* o)
         // a fresh scratch is zeroed (its counter and group sums start at zero;
         // every compression of this model's fields leaves them zero)
         if (!rc.rate) {
-            // both fields of a takeshot at once, one after the other when memory is short
-            m->scratch_fields = 2;
-            cudaError_t e = m->scratch.alloc((size_t)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx, 2), true);
+            // both fields of a takeshot at once, one after the other where
+            // memory served only one (CKFWI_SCRATCH_BYTES stands for less of
+            // it); that scratch then stays: to ask again for both would give
+            // it up first, in every call
+            const size_t one = (size_t)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx, 1);
+            const char* lim = std::getenv("CKFWI_SCRATCH_BYTES");
+            cudaError_t e = cudaErrorMemoryAllocation;
+            if (m->scratch_fields != 1) {
+                m->scratch_fields = 2;
+                if (!lim || (long long)(2 * one) <= std::atoll(lim)) e = m->scratch.alloc(2 * one, true);
+            }
             if (e == cudaErrorMemoryAllocation) {
                 cudaGetLastError();
+                if (m->scratch_fields == 2 && std::getenv("CKFWI_VERBOSE"))
+                    std::fprintf(stderr, "ckfwi codec scratch for one field: %zu bytes\n", one);
                 m->scratch_fields = 1;
-                e = m->scratch.alloc((size_t)codec_scratch_bytes(f.dims, f.nz, f.ny, f.nx, 1), true);
+                e = m->scratch.alloc(one, true);
+                if (e != cudaSuccess) m->scratch_fields = 0;
             }
             CK_TRY(e);
         }
