@@ -1987,8 +1987,16 @@ CodecView field_view(const FieldGeom& f)
 }
 
 // Fields a codec call names by index: the zero state, the working fields,
-// the restored states
-int codec_field(const Role& r) { return r.kind == R_WORK ? 1 + r.idx : r.kind == R_URES ? 5 + r.idx : 0; }
+// the restored states; no other field is coded
+int codec_field(const Role& r, int* field)
+{
+    switch (r.kind) {
+    case R_ZERO: *field = 0; return CKFWI_OK;
+    case R_WORK: *field = 1 + r.idx; return CKFWI_OK;
+    case R_URES: *field = 5 + r.idx; return CKFWI_OK;
+    default: return CKFWI_EINVAL;
+    }
+}
 
 CodecLane codec_lane(ckfwi_model* m)
 {
@@ -2202,7 +2210,7 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
         took_level = level;
         if (cx.issue && follows) {
             CodecCall c = codec_call(cx, rc, 1);
-            c.src[0] = codec_field(u);
+            ST_TRY(codec_field(u, &c.src[0]));
             c.from[0] = slot;
             c.from[1] = rc.M + 1 + slot;
             c.to = slot + 1;
@@ -2220,7 +2228,9 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
             // lane's scratch serves only one
             int nf = 2;
             for (int l = 0; l < NL && !rc.rate; ++l) nf = std::min(nf, cx.lane(l)->scratch_fields);
-            const int fld[2] = {codec_field(u), codec_field(up)};
+            int fld[2];
+            ST_TRY(codec_field(u, &fld[0]));
+            ST_TRY(codec_field(up, &fld[1]));
             const int word[3] = {slot, rc.M + 1 + slot, slot + 1};
             for (int k = 0; k < 2; k += nf) {
                 CodecCall c = codec_call(cx, rc, nf);
@@ -2493,8 +2503,8 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
             } else if (rc.codec) {
                 // a reverse step needs u^s only
                 CodecCall c = codec_call(cx, rc, next_turn ? 1 : 2);
-                c.src[0] = codec_field(work_r(0));
-                c.src[1] = codec_field(work_r(1));
+                ST_TRY(codec_field(work_r(0), &c.src[0]));
+                ST_TRY(codec_field(work_r(1), &c.src[1]));
                 c.from[0] = A.b;
                 c.from[1] = prev_word[A.b];
                 ST_TRY(decompress(cx, rc, c));
@@ -2566,7 +2576,7 @@ int run_body(Ctx& cx, const RunCfg& rc, const std::vector<Action>& acts, long lo
                 for (int k = 0; k < T; ++k) {
                     if (us[i + k] != NONE_R) continue;
                     us[i + k] = ures_r(c.nf);
-                    c.src[c.nf] = codec_field(us[i + k]);
+                    ST_TRY(codec_field(us[i + k], &c.src[c.nf]));
                     c.from[c.nf++] = slots[i + k];
                 }
                 if (c.nf > 0) ST_TRY(decompress(cx, rc, c));
