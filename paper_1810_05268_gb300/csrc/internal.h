@@ -153,6 +153,8 @@ struct Step2Args {
     // forward
     Sample smp;           // receivers: level n + i goes to out + i n
     const int2* rzx;      // each receiver's first point (z, x)
+    const int* rlist;     // the receivers by tile (the one that holds their first point):
+    const int* rstart;    // tile b's are rlist[rstart[b]] .. rlist[rstart[b + 1] - 1]
     // reverse
     Inj adj;              // step i takes series - i adj_stride
     long long adj_stride;

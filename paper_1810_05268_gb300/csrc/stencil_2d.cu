@@ -61,7 +61,7 @@ namespace {
 
 constexpr int NT2 = 512;                          // threads
 constexpr int NE2 = 256;                          // of them, the ones that compute edges and exchange them
-constexpr int RL2 = 512;                          // receivers listed per tile; with more, every step looks at all
+constexpr int RL2 = 512;                          // receivers of a tile listed in shared memory; the rest stay in the lane's list
 constexpr int SLOTS2 = 4;                         // exchange buffers in turn
 
 // columns a strip between x neighbours has, and the x margin of a staged
@@ -573,7 +573,6 @@ __device__ __forceinline__ bool stage_state(const Cta2<K>& ct, float* b1, float*
 template <int K>
 __device__ __forceinline__ void fwd2_body(const Step2Args& a, int b, float* sm)
 {
-    __shared__ int nrl;
     const Plan2<K> pl(a, b);
     const Cta2<K>& ct = pl.ct;
     const Tile2& t = ct.t;
@@ -585,23 +584,15 @@ __device__ __forceinline__ void fwd2_body(const Step2Args& a, int b, float* sm)
     float* ezs = exs + t.bx;
     int* rl = reinterpret_cast<int*>(ezs + (t.bz + 3) / 4 * 4);
     const unsigned e0 = a.epoch[b];
-    if (tid == 0) nrl = 0;
     Step2Env<K> ev{b1, b2, w, ezs, exs, a.hdt, {}, false, pl.meets(a.src)};
 #pragma unroll
     for (int j = 0; j < K; ++j) ev.c[j] = a.c[j + 1];
     ev.damped = __syncthreads_or(stage_state<K>(ct, b1, b2, w, exs, ezs, a));
-    auto mine = [&](int r) {
-        const int2 at = a.rzx[r];
-        return at.x >= ct.zt && at.x < ct.zt + t.bz && at.y >= ct.xt && at.y < ct.xt + t.bx;
-    };
-    for (int r = tid; r < a.smp.n; r += NT2)
-        if (mine(r)) {
-            const int k = atomicAdd(&nrl, 1);
-            if (k < RL2) rl[k] = r;
-        }
+    const int* list = a.smp.n > 0 ? a.rlist + a.rstart[b] : nullptr;
+    const int listed = a.smp.n > 0 ? a.rstart[b + 1] - a.rstart[b] : 0;
+    for (int k = tid; k < min(listed, RL2); k += NT2) rl[k] = list[k];
     cp_wait();
     __syncthreads();
-    const int listed = nrl;
     const int spos = (tid - NE2 - pl.in.n % NT2 + 2 * NT2) % NT2;    // the threads after those of the interior sample
     for (int i = 0; i < a.T; ++i) {
         // receivers of level n + i
@@ -615,12 +606,7 @@ __device__ __forceinline__ void fwd2_body(const Step2Args& a, int b, float* sm)
             acc = __fmaf_rn(wt[3], p[t.pitch + 1], acc);
             a.smp.out[(long long)i * a.smp.n + r] = acc;
         };
-        if (listed <= RL2) {
-            for (int k = spos; k < listed; k += NT2) sample(rl[k]);
-        } else {
-            for (int r = tid; r < a.smp.n; r += NT2)
-                if (mine(r)) sample(r);
-        }
+        for (int k = spos; k < listed; k += NT2) sample(k < RL2 ? rl[k] : list[k]);
         const bool last = i + 1 == a.T;
         const unsigned e = e0 + 1u + i;
         const bool out0 = i == 0 && goes_out(a, 0), out = goes_out(a, i + 1);
