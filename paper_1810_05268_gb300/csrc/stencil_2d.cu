@@ -178,23 +178,25 @@ __device__ __forceinline__ void lap2(float (&out)[4], const float (*q)[4], const
     out[3] = acc[1].y;
 }
 
-// injection of four points of row z, where the box meets them (a Laplacian is
-// never -0, so adding a zero elsewhere, as the one-step kernels do, changes
-// nothing)
-__device__ __forceinline__ void inj4(float (&s)[4], const Inj& in, const float* series, int z, int x0)
+// injection of four points of row z: zero is added where nothing is injected
+// (`on`: somewhere in the tile), as the one-step kernels do (a Laplacian of
+// values near the smallest ones can round to -0, which that turns into +0)
+__device__ __forceinline__ void inj4(float (&s)[4], bool on, const Inj& in, const float* series, int z, int x0)
 {
-    if (z < in.z0 || z >= in.z1 || x0 + 4 <= in.x0 || x0 >= in.x1) return;
-    const int row = (z - in.z0) * (in.x1 - in.x0);
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (on && z >= in.z0 && z < in.z1 && x0 + 4 > in.x0 && x0 < in.x1) {
+        const int row = (z - in.z0) * (in.x1 - in.x0);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int x = x0 + i;
-        if (x < in.x0 || x >= in.x1) continue;
-        const int b = row + x - in.x0;
-        const int e1 = in.rowptr[b + 1];
-        float acc = 0.0f;
-        for (int e = in.rowptr[b]; e < e1; ++e) acc = __fmaf_rn(in.wt[e], series[in.col[e]], acc);
-        s[i] = __fadd_rn(s[i], acc);
+        for (int i = 0; i < 4; ++i) {
+            const int x = x0 + i;
+            if (x < in.x0 || x >= in.x1) continue;
+            const int b = row + x - in.x0;
+            const int e1 = in.rowptr[b + 1];
+            for (int e = in.rowptr[b]; e < e1; ++e) acc[i] = __fmaf_rn(in.wt[e], series[in.col[e]], acc[i]);
+        }
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] = __fadd_rn(s[i], acc[i]);
 }
 
 __device__ __forceinline__ void out32(float* p, long long o, const float* v, int x0, int nx)
@@ -468,7 +470,7 @@ __device__ __forceinline__ void update2(float (&v)[4], const Cta2<K>& ct, const 
     sld<4>(pv, ev.b2 + o);
     sld<4>(wv, ev.w + r * ct.t.bx + 4 * q);
     lap2<K>(s, qz, ev.b1 + o, ev.c);
-    if (ev.inject) inj4(s, in, series, ct.zt + r, x0);
+    inj4(s, ev.inject, in, series, ct.zt + r, x0);
     const float* uc = qz[K];
     float2 a0, a1;
     if (ev.damped) {
@@ -697,7 +699,7 @@ __device__ __forceinline__ void adj2_body(const Step2Args& a, int b, float* sm)
                     float* gp = gs + r * t.bx + 4 * pr.q;
                     sld<4>(gv, gp);
                     lap2<K>(s, win + h, ub + o, ev.c);
-                    if (src) inj4(s, a.src, a.src.series - (i - 1), ct.zt + r, x0);
+                    inj4(s, src, a.src, a.src.series - (i - 1), ct.zt + r, x0);
                     const float2 g0 = __ffma2_rn(f2(lv[0], lv[1]), f2(s[0], s[1]), f2(gv[0], gv[1]));
                     const float2 g1 = __ffma2_rn(f2(lv[2], lv[3]), f2(s[2], s[3]), f2(gv[2], gv[3]));
                     gv[0] = g0.x;

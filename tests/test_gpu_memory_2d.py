@@ -46,13 +46,15 @@ def test_grid_beyond_the_sms_takes_no_extra_fields():
 
 def test_batch_stays_within_the_memory_it_is_given(monkeypatch):
     import torch
-    shape, nt, shots, given = (464, 1104), 8, 12, 400 << 20
+    # a field just within two 2 MB allocation units, so that none is lost to rounding
+    shape, nt, shots, given = (928, 1104), 8, 12, 800 << 20
     vel = torch.full(shape, 2.0, device="cuda")
     rec = np.array([[100.0, 0.0, 400.0]])
     sh = [C.ShotSpec(src=(2000.0, 0.0, 300.0 * (i + 1)), rec=rec, f0=0.02) for i in range(shots)]
     dl = [torch.zeros((nt + 1, 1), device="cuda") for _ in sh]
     kw = dict(store_mode="codec", tol=1e-5, pool_bytes=2 << 20)
     monkeypatch.setenv("CKFWI_FREE_BYTES", str(given))
+    monkeypatch.setenv("CKFWI_BATCH_VER", "9")
     for counted in (False, True):
         m = C.Model(C.GridSpec(2, shape, 10, 10.0, 8, 0.8, nt, 3.0))
         m.set_model(vel)
