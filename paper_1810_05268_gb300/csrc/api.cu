@@ -375,6 +375,8 @@ struct ckfwi_model {
     DevMem gsum_comp;               // batch: compensation terms
     ShotDev shot;
     Tile tf{}, ta{};
+    Tile t1[2];                     // 2D: forward / reverse tile of one step a launch, beside launches of many (ver 9)
+    bool tuned1 = false;
     Tile t4[5];                     // OT4 fed by tensor copies: the tile of each pass (ver 10 when tuned)
     bool tuned = false;
     int nparts = 128;
@@ -793,6 +795,8 @@ struct Ctx {
     // the tile of the forward / reverse steps; launches of several 2D steps take ver 9
     const Tile& tile(bool reverse) const { return batch ? (reverse ? ba : bf) : (reverse ? m->ta : m->tf); }
     bool several(bool reverse) const { return tile(reverse).ver == 9; }
+    // the tile of a launch of one step
+    const Tile& step_tile(bool reverse) const { return stage && several(reverse) ? m->t1[reverse] : tile(reverse); }
     int nl() const { return lanes.empty() ? 1 : (int)lanes.size(); }
     ckfwi_model* lane(int l) const { return lanes.empty() ? m : lanes[l]; }
     void* ptr(int l, const Role& r) const { return rptr(lane(l), mode, r); }
@@ -890,15 +894,14 @@ Tile ot4_host_tile(const Tile& t)
 // The tile of a pass fed by tensor copies: its own when tuned, else the step's
 const Tile& ot4q_tile(const ckfwi_model* m, int op, const Tile& t) { return m->t4[op].ver == 10 ? m->t4[op] : t; }
 
-// The tile of the launch that samples a forward step's receivers (the step
-// reads u and up): an OT4 step's pass 1, which has a z run of its own, and
-// the stand-ins of steps that read host slots
-Tile sampling_tile(const ckfwi_model* m, const Role& u, const Role& up)
+// The tile of the launch that samples the receivers of a forward step of tile
+// t (the step reads u and up): an OT4 step's pass 1, which has a z run of its
+// own, and the stand-ins of steps that read host slots
+Tile sampling_tile(const ckfwi_model* m, const Tile& t, const Role& u, const Role& up)
 {
-    if (m->tf.ver == 10)
-        return in_host(m, u) || in_host(m, up) ? ot4_host_tile(m->tf) : ot4q_tile(m, OT4Q_LAP, m->tf);
-    if (m->tf.ver == 2 && in_host(m, u)) return host_tile(m);
-    return m->tf;
+    if (t.ver == 10) return in_host(m, u) || in_host(m, up) ? ot4_host_tile(t) : ot4q_tile(m, OT4Q_LAP, t);
+    if (t.ver == 2 && in_host(m, u)) return host_tile(m);
+    return t;
 }
 
 int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by, CUtensorMap* out);
@@ -1099,7 +1102,8 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
              const Role& ck_u, const Role& ck_up)
 {
     const int NL = cx.nl();
-    if (cx.several(false)) {
+    const Tile& ts = cx.step_tile(false);
+    if (ts.ver == 9) {
         // u^{n+1}, and the checkpoint's fields: u^{n+1} (16-bit) and u^n
         Emits e32{{1, out}}, e16;
         if (ck == CK_FP32) e32.emplace_back(0, ck_up);
@@ -1131,7 +1135,7 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
                 ST_TRY(check_field(m, cm, ck_up, a.ck_up, "forward step: checkpoint u^{s-1}"));
             }
         }
-        const Tile t = cx.batch ? cx.bf : sampling_tile(m, u, up);
+        const Tile t = cx.batch ? ts : sampling_tile(m, ts, u, up);
         const int zlen = cx.batch ? cx.zf[l] : t.zlen;
         bool sep = false;
         if (record) {
@@ -1150,10 +1154,10 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
             continue;
         }
         const int tok = cx.begin(PC_FWD);
-        if (m->tf.ver == 8) {
+        if (ts.ver == 8) {
             if (in_host(m, u) || in_host(m, up)) {
                 // tensor maps cover device memory only: the async-copy kernel of the same tile
-                Tile t4 = m->tf;
+                Tile t4 = ts;
                 t4.ver = 4;
                 t4.pf = m->K <= 4 ? 1 : 0;
                 CK_TRY(launch_fwd4(a, t4, m->K, ck, cx.st));
@@ -1162,25 +1166,25 @@ int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, boo
                 ST_TRY(tensor_map(m, a.u, U_FP32, tq_box_x(m->K), tq_box_y(m->K), &tu));
                 ST_TRY(tensor_map(m, a.up, U_FP32, 32, 16, &tp));
                 ST_TRY(tensor_map(m, a.w, U_FP32, 32, 16, &tw));
-                CK_TRY(launch_fwdq(a, tu, tp, tw, m->tf, m->K, ck, cx.st));
+                CK_TRY(launch_fwdq(a, tu, tp, tw, ts, m->K, ck, cx.st));
             }
-        } else if (m->tf.ver == 7) {
-            CK_TRY(launch_fwd5(a, m->tf, m->K, ck, cx.st));
-        } else if (m->tf.ver >= 5) {
-            ST_TRY(ot4_fwd_step(m, a, in_host(m, u) || in_host(m, up) ? ot4_host_tile(m->tf) : m->tf, ck, cx.st));
+        } else if (ts.ver == 7) {
+            CK_TRY(launch_fwd5(a, ts, m->K, ck, cx.st));
+        } else if (ts.ver >= 5) {
+            ST_TRY(ot4_fwd_step(m, a, in_host(m, u) || in_host(m, up) ? ot4_host_tile(ts) : ts, ck, cx.st));
             ++cx.launches;
-        } else if (m->tf.ver == 2 && in_host(m, u)) {
+        } else if (ts.ver == 2 && in_host(m, u)) {
             CK_TRY(launch_fwd(a, host_tile(m), m->K, ck, cx.st));
-        } else if (m->tf.ver == 4) {
-            CK_TRY(launch_fwd4(a, m->tf, m->K, ck, cx.st));
-        } else if (m->tf.ver == 3) {
-            CK_TRY(launch_fwd3(a, m->tf, m->K, ck, cx.st));
-        } else if (m->tf.ver == 2) {
+        } else if (ts.ver == 4) {
+            CK_TRY(launch_fwd4(a, ts, m->K, ck, cx.st));
+        } else if (ts.ver == 3) {
+            CK_TRY(launch_fwd3(a, ts, m->K, ck, cx.st));
+        } else if (ts.ver == 2) {
             CUtensorMap tm;
-            ST_TRY(tensor_map(m, a.u, U_FP32, tma_tile_x() + 2 * tma_halo_x(m->K), m->tf.by + 2 * m->K, &tm));
-            CK_TRY(launch_fwd_tma(a, tm, m->tf, m->K, ck, cx.st));
+            ST_TRY(tensor_map(m, a.u, U_FP32, tma_tile_x() + 2 * tma_halo_x(m->K), ts.by + 2 * m->K, &tm));
+            CK_TRY(launch_fwd_tma(a, tm, ts, m->K, ck, cx.st));
         } else {
-            CK_TRY(launch_fwd(a, m->tf, m->K, ck, cx.st));
+            CK_TRY(launch_fwd(a, ts, m->K, ck, cx.st));
         }
         cx.end(tok);
         ++cx.launches;
@@ -1470,7 +1474,8 @@ int adj_steps2(Ctx& cx, const Role& l1, const Role& l2, const Role& o0, const Ro
 int adj_step(Ctx& cx, const Role& l1, const Role& l2, const Role& l0, const Role& u, int utype, int j)
 {
     const int NL = cx.nl();
-    if (cx.several(true)) return adj_steps2(cx, l1, l2, l0, NONE_R, &u, &utype, j, 1);
+    const Tile& ts = cx.step_tile(true);
+    if (ts.ver == 9) return adj_steps2(cx, l1, l2, l0, NONE_R, &u, &utype, j, 1);
     for (int l = 0; l < NL; ++l) {
         ckfwi_model* m = cx.lane(l);
         AdjArgs a = adj_args(m);
@@ -1503,37 +1508,37 @@ int adj_step(Ctx& cx, const Role& l1, const Role& l2, const Role& l0, const Role
             continue;
         }
         const int tok = cx.begin(PC_ADJ);
-        if (m->ta.ver == 8 && (utype != U_FP32 || in_host(m, u))) {
+        if (ts.ver == 8 && (utype != U_FP32 || in_host(m, u))) {
             // tensor maps cover FP32 device fields only: the lean kernel of the same tile
-            Tile t7 = m->ta;
+            Tile t7 = ts;
             t7.ver = 7;
             t7.pf = 1;
             CK_TRY(launch_adj5(a, t7, m->K, utype, cx.st));
-        } else if (m->ta.ver == 8) {
+        } else if (ts.ver == 8) {
             CUtensorMap mp[6];
             ST_TRY(adjq_maps(m, a, mp));
-            CK_TRY(launch_adjq(a, mp, m->ta, m->K, cx.st));
+            CK_TRY(launch_adjq(a, mp, ts, m->K, cx.st));
             ++cx.launches;
-        } else if (m->ta.ver == 7) {
-            CK_TRY(launch_adj5(a, m->ta, m->K, utype, cx.st));
-        } else if (m->ta.ver >= 5) {
-            const Tile t = utype != U_FP32 || in_host(m, u) ? ot4_host_tile(m->ta) : m->ta;
+        } else if (ts.ver == 7) {
+            CK_TRY(launch_adj5(a, ts, m->K, utype, cx.st));
+        } else if (ts.ver >= 5) {
+            const Tile t = utype != U_FP32 || in_host(m, u) ? ot4_host_tile(ts) : ts;
             ST_TRY(ot4_adj_step(m, a, t, utype, j, cx.st));
             cx.launches += t.ver == 10 ? 3 : 2;
-        } else if (m->ta.ver == 2 && in_host(m, u)) {
+        } else if (ts.ver == 2 && in_host(m, u)) {
             CK_TRY(launch_adj(a, host_tile(m), m->K, utype, cx.st));
-        } else if (m->ta.ver == 4) {
-            CK_TRY(launch_adj4(a, m->ta, m->K, utype, cx.st));
-        } else if (m->ta.ver == 3) {
-            CK_TRY(launch_adj3(a, m->ta, m->K, utype, cx.st));
-        } else if (m->ta.ver == 2) {
+        } else if (ts.ver == 4) {
+            CK_TRY(launch_adj4(a, ts, m->K, utype, cx.st));
+        } else if (ts.ver == 3) {
+            CK_TRY(launch_adj3(a, ts, m->K, utype, cx.st));
+        } else if (ts.ver == 2) {
             CUtensorMap tl, tu;
-            const int bx = tma_tile_x() + 2 * tma_halo_x(m->K), by = m->ta.by + 2 * m->K;
+            const int bx = tma_tile_x() + 2 * tma_halo_x(m->K), by = ts.by + 2 * m->K;
             ST_TRY(tensor_map(m, a.l1, U_FP32, bx, by, &tl));
             ST_TRY(tensor_map(m, a.u, utype, bx, by, &tu));
-            CK_TRY(launch_adj_tma(a, tl, tu, m->ta, m->K, utype, cx.st));
+            CK_TRY(launch_adj_tma(a, tl, tu, ts, m->K, utype, cx.st));
         } else {
-            CK_TRY(launch_adj(a, m->ta, m->K, utype, cx.st));
+            CK_TRY(launch_adj(a, ts, m->K, utype, cx.st));
         }
         cx.end(tok);
         ++cx.launches;
@@ -1635,9 +1640,13 @@ int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by
 }
 
 // --------------------------------------------------------------- autotune
-int autotune(ckfwi_model* m, cudaStream_t st)
+// (one_step: the tiles of one step a launch where the model's are of many)
+int autotune(ckfwi_model* m, cudaStream_t st, bool one_step = false)
 {
-    if (m->tuned) return CKFWI_OK;
+    bool& tuned = one_step ? m->tuned1 : m->tuned;
+    if (tuned) return CKFWI_OK;
+    Tile& tf = one_step ? m->t1[0] : m->tf;
+    Tile& ta = one_step ? m->t1[1] : m->ta;
     const FieldGeom& f = m->fg;
     // candidate z-run lengths: whole columns, and runs giving >= 4 CTAs per SM
     int dev = 0;
@@ -1827,14 +1836,15 @@ int autotune(ckfwi_model* m, cudaStream_t st)
         *t = u;
         return true;
     };
-    bool ff = forced("CKFWI_TILE_FWD", &m->tf, false), fa = forced("CKFWI_TILE_ADJ", &m->ta, true);
+    bool ff = one_step ? m->tf.ver != 9 : forced("CKFWI_TILE_FWD", &tf, false);
+    bool fa = one_step ? m->ta.ver != 9 : forced("CKFWI_TILE_ADJ", &ta, true);
     forced("CKFWI_TILE_OT4_LAP", &m->t4[OT4Q_LAP], false);   // pass 1 of an OT4 step, as tuning leaves it
     // a 2D grid that fits the SMs takes the kernels of many steps a launch:
     // nothing to time (281 x 281 and 464 x 1104: 1.5 and 3.1 us a forward
     // step, against 3.3 and 5.1 us of kernel time for one step a launch, and
     // 6.3 us when the host launches it)
-    ff = ff || step2_tile({m}, false, &m->tf);
-    fa = fa || step2_tile({m}, true, &m->ta);
+    ff = ff || (!one_step && step2_tile({m}, false, &tf));
+    fa = fa || (!one_step && step2_tile({m}, true, &ta));
     const bool verbose = std::getenv("CKFWI_VERBOSE") != nullptr;
     // time one candidate: the median of `rounds` timings of `reps` launches
     auto time_of = [&](const Tile& t, int pass, int rounds, float* out) -> int {
@@ -1885,7 +1895,7 @@ int autotune(ckfwi_model* m, cudaStream_t st)
                              pass ? "adj" : "fwd", t.ver, t.bx, t.by, t.vec, t.zlen, t.pf, 1000.0f * ms);
             if (ms < best) {
                 best = ms;
-                (pass == 0 ? m->tf : m->ta) = t;
+                (pass == 0 ? tf : ta) = t;
             }
         }
     }
@@ -1893,7 +1903,7 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     // (three point fields against one), so each takes its own z run and
     // prefetch: at 208^3 one run for all left the passes at 1.6 and 1.9 waves
     // (forward 72.6 us, reverse 156.7 us a step).
-    if ((m->tf.ver == 10 && !ff) || (m->ta.ver == 10 && !fa)) {
+    if ((tf.ver == 10 && !ff) || (ta.ver == 10 && !fa)) {
         Ot4qArgs q{};
         q.f = a;
         q.f.out = org(m->z4[0], f);
@@ -1936,8 +1946,8 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     cudaEventDestroy(e1);
     // exchange buffers, before any recording (allocating is not recorded)
     Step2Args x2;
-    if (m->tf.ver == 9) ST_TRY(step2_exchange(m, m->tf, false, &x2));
-    if (m->ta.ver == 9) ST_TRY(step2_exchange(m, m->ta, true, &x2));
+    if (tf.ver == 9) ST_TRY(step2_exchange(m, tf, false, &x2));
+    if (ta.ver == 9) ST_TRY(step2_exchange(m, ta, true, &x2));
     // the probe runs wrote into working buffers; clear them
     for (DevMem* d : {m->work, m->lam})
         for (int i = 0; i < 4 && d[i].p; ++i) CK_TRY(cudaMemsetAsync(d[i].p, 0, d[i].bytes, st));
@@ -1945,7 +1955,7 @@ int autotune(ckfwi_model* m, cudaStream_t st)
     for (int i = 0; i < 3; ++i)
         if (m->z4[i].p) CK_TRY(cudaMemsetAsync(m->z4[i].p, 0, m->z4[i].bytes, st));
     CK_TRY(cudaStreamSynchronize(st));
-    m->tuned = true;
+    tuned = true;
     return CKFWI_OK;
 }
 
@@ -2915,6 +2925,13 @@ int gradient_one(ckfwi_model* m, const ckfwi_shot* s, const float* d_obs, int me
     ST_TRY(prepare_storage(m, rc, o));
     ST_TRY(prepare_states(m, rc, m->tf, m->ta));
     ST_TRY(step2_receivers(m, m->tf));
+    // staged host slots: a step that makes a checkpoint and every reverse step
+    // is a launch of its own, and a launch of one step is better the one-step
+    // kernels' (the many-step ones move the state in and out of the tiles for
+    // it: 464 x 1104, 300 steps, half of 20 slots on the host: 7.9 ms with
+    // them alone, 5.2 with one-step launches alone, 4.9 with both)
+    const bool stage = rc.mode == CKFWI_STORE_FP32 && !rc.codec && !rc.store_all && m->host_slots > 0 && m->side;
+    if (stage && (m->tf.ver == 9 || m->ta.ver == 9)) ST_TRY(autotune(m, st, true));
     const size_t nd = (size_t)(rc.N + 1) * m->shot.nrec;
     CK_TRY(cudaMemcpyAsync(m->shot.dobs.p, d_obs, nd * sizeof(float),
                            mem == CKFWI_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
@@ -2924,7 +2941,7 @@ int gradient_one(ckfwi_model* m, const ckfwi_shot* s, const float* d_obs, int me
     make_schedule(m, rc, acts, cnt);
     Ctx cx{m, st, 0};
     cx.mode = rc.mode;
-    cx.stage = rc.mode == CKFWI_STORE_FP32 && !rc.codec && !rc.store_all && m->host_slots > 0 && m->side;
+    cx.stage = stage;
     long long counters[2] = {0, 0};
     const bool graph = o->use_graph != 0 && !o->profile;
     if (o->profile) {
