@@ -3049,14 +3049,115 @@ std::vector<long long> lane_ids(const std::vector<ckfwi_model*>& lanes, bool wit
     return v;
 }
 
+// Steps of an average launch of many 2D steps, forward and reverse, in a
+// schedule: its steps over its runs (forward steps past checkpoints, reverse
+// steps of states that need no recomputation), as a power of two from below
+struct RunSteps {
+    int s[2];
+};
+RunSteps run_steps(const RunCfg& rc, const std::vector<Action>& acts)
+{
+    long long steps[2] = {0, 0}, launches[2] = {0, 0};
+    const int most[2] = {STEP2_MAX, rc.codec ? CODEC_NF : STEP2_MAX};
+    auto run = [&](int r, long long len) {
+        steps[r] += len;
+        launches[r] += (len + most[r] - 1) / most[r];
+    };
+    if (rc.store_all) run(0, rc.N), run(1, rc.N);
+    for (size_t i = 0; i < acts.size(); ++i) {
+        long long len = 0;
+        if (acts[i].op == ACT_ADVANCE) {
+            for (; i < acts.size() && (acts[i].op == ACT_ADVANCE || acts[i].op == ACT_TAKESHOT); ++i)
+                if (acts[i].op == ACT_ADVANCE) len += acts[i].b;
+            --i;
+            run(0, len);
+        } else if (acts[i].op == ACT_YOUTURN) {
+            for (len = 1; i + 2 < acts.size() && acts[i + 1].op == ACT_RESTORE && acts[i + 2].op == ACT_YOUTURN; i += 2) ++len;
+            run(1, len);
+        }
+    }
+    RunSteps rs{{1, 1}};
+    for (int r = 0; r < 2; ++r)
+        while (launches[r] > 0 && 2LL * rs.s[r] * launches[r] <= steps[r]) rs.s[r] *= 2;
+    return rs;
+}
+
+// Time of one step [us] of every lane in launches of T 2D steps, on the lanes'
+// working buffers
+int step2_time(const std::vector<ckfwi_model*>& lanes, const Tile& t, bool reverse, int T, cudaStream_t st,
+               cudaEvent_t e0, cudaEvent_t e1, float* us)
+{
+    const int NL = (int)lanes.size(), K = lanes[0]->K;
+    int dev = 0, nsm = 0;
+    CK_TRY(cudaGetDevice(&dev));
+    CK_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    std::vector<Step2Args> rows(NL);
+    for (int l = 0; l < NL; ++l) {
+        ckfwi_model* L = lanes[l];
+        const FieldGeom& f = L->fg;
+        Step2Args& a = rows[l];
+        ST_TRY(step2_args(L, t, reverse, T, &a));
+        DevMem* const d = reverse ? L->lam : L->work;
+        a.f1 = org(d[0], f);
+        a.f2 = org(d[1], f);
+        ST_TRY(step2_dst(&a, T, org(d[2], f), CK_FP32));
+        if (T > 1) ST_TRY(step2_dst(&a, T - 1, org(d[3], f), CK_FP32));
+        a.src.series = L->shot.wavelet.as<float>() + (reverse ? T - 1 : 0);
+        if (!reverse) continue;
+        a.adj = L->shot.adj.view;
+        a.adj.series = L->shot.resid.as<float>() + (size_t)T * L->shot.nrec;
+        a.adj_stride = L->shot.nrec;
+        a.gacc = org(L->gacc, f);
+        for (int i = 0; i < T; ++i) {
+            a.u[i] = org(L->work[0], f);
+            a.ut[i] = U_FP32;
+        }
+    }
+    const std::vector<int> g = step2_groups(lanes, t, nsm);
+    std::vector<int> start;
+    std::vector<BatchLaunch<Step2Args>> bl;
+    DevMem tab, dst;
+    CK_TRY(tab.alloc(sizeof(Step2Args) * NL, false));
+    CK_TRY(dst.alloc(sizeof(int) * 2 * (NL + 1), false));
+    for (size_t k = 0; k + 1 < g.size(); ++k) {
+        const size_t s0 = start.size();
+        start.push_back(0);
+        for (int l = g[k]; l < g[k + 1]; ++l) start.push_back(start.back() + (int)tiles_of(lanes[l]->fg, t));
+        bl.push_back(BatchLaunch<Step2Args>{tab.as<Step2Args>() + g[k], dst.as<int>() + s0, g[k + 1] - g[k], 2, start.back()});
+    }
+    CK_TRY(cudaMemcpy(tab.p, rows.data(), sizeof(Step2Args) * NL, cudaMemcpyHostToDevice));
+    CK_TRY(cudaMemcpy(dst.p, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice));
+    std::vector<float> v;
+    for (int round = 0; round < 5; ++round) {          // the first two bring the clocks up
+        CK_TRY(cudaEventRecord(e0, st));
+        for (const auto& b : bl) CK_TRY(launch_step2_batch(b, t, K, reverse, st));
+        CK_TRY(cudaEventRecord(e1, st));
+        CK_TRY(cudaEventSynchronize(e1));
+        float ms = 0;
+        CK_TRY(cudaEventElapsedTime(&ms, e0, e1));
+        if (round > 1) v.push_back(ms);
+    }
+    std::sort(v.begin(), v.end());
+    *us = 1000.0f * v[1] / (float)T;
+    // (a wait that ran out would have left the tiles at different steps)
+    for (ckfwi_model* L : lanes) {
+        auto& x = L->xch[std::make_tuple(t.bx, t.zlen, reverse ? 1 : 0)];
+        CK_TRY(cudaMemsetAsync(x.buf.p, 0, x.buf.bytes, st));
+        CK_TRY(cudaMemsetAsync(x.epoch.p, 0, x.epoch.bytes, st));
+    }
+    CK_TRY(cudaStreamSynchronize(st));
+    return CKFWI_OK;
+}
+
 // Batch autotuner: a common tile shape and a z-run length per lane, picked
 // by timing batched forward and reverse launches over all lanes.  The
 // candidates split every column into nzc runs, nzc chosen so that the
 // whole batch has 1 to 16 CTAs per SM.
-int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const BatchTiles** out)
+int batch_tune(const std::vector<ckfwi_model*>& lanes, const RunSteps& runs, cudaStream_t st, const BatchTiles** out)
 {
     ckfwi_model* m0 = lanes[0];
-    const std::vector<long long> key = lane_ids(lanes, false);
+    std::vector<long long> key = lane_ids(lanes, false);
+    if (m0->fg.dims == 2) key.insert(key.end(), {runs.s[0], runs.s[1]});
     auto it = m0->btiles.find(key);
     if (it != m0->btiles.end()) {
         *out = &it->second;
@@ -3100,10 +3201,11 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
         }
     }
     // CKFWI_BATCH_VER restricts the timed candidates to one generation
-    // (tests); generation 4 has no batched reverse step, which then takes
-    // the vector-blocked kernels
-    const char* bv = std::getenv("CKFWI_BATCH_VER");
-    const int want = bv ? std::atoi(bv) : 0;
+    // (tests; "f,r": forward, reverse); generation 4 has no batched reverse
+    // step, which then takes the vector-blocked kernels
+    int want[2] = {0, 0};
+    if (const char* bv = std::getenv("CKFWI_BATCH_VER"))
+        if (std::sscanf(bv, "%d,%d", &want[0], &want[1]) < 2) want[1] = want[0];
     for (const Tile& t : shapes) {
         long long cols = 0;
         int nzmax = 1;
@@ -3185,20 +3287,38 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
     CK_TRY(cudaEventCreate(&e0));
     CK_TRY(cudaEventCreate(&e1));
     const bool verbose = std::getenv("CKFWI_VERBOSE") != nullptr;
-    float best[2] = {1e30f, 1e30f};
+    const int reps = 3;
+    float best[2] = {1e30f, 1e30f};       // of `reps` steps
     bool warmed = false;
     BatchTiles bt;
-    // 2D lanes that fit the SMs, in groups or together: as for one model
-    bool many[2] = {false, false};
-    if (!want || want == 9) {
-        many[0] = step2_tile(lanes, false, &bt.tf);
-        many[1] = step2_tile(lanes, true, &bt.ta);
-        if (many[0]) bt.zf.assign(NL, bt.tf.zlen);
-        if (many[1]) bt.za.assign(NL, bt.ta.zlen);
-    }
     int rs = CKFWI_OK;
+    std::vector<std::tuple<ckfwi_model*, std::tuple<int, int, int>, bool>> timed9;   // exchange buffers made here
+    // 2D lanes that fit the SMs, in groups or together: launches of many
+    // steps, as many as the schedule's runs have, timed against one step a
+    // launch: groups run in turn, each with its own exchanges, while one step
+    // of all lanes fills the GPU.  (A reverse step of eight lanes of 600 x
+    // 1200, order 8: 91 us in launches of 16 steps, 60 us by itself; of 281 x
+    // 281, order 4: 7.7 and 11.1.  Taking the former wherever they fit cost
+    // such batches up to 1.3 of their time.)
+    for (int r = 0; r < 2 && rs == CKFWI_OK; ++r) {
+        if (want[r] && want[r] != 9) continue;
+        Tile t;
+        float us = 0;
+        if (!step2_tile(lanes, r == 1, &t)) continue;
+        const auto key9 = std::make_tuple(t.bx, t.zlen, r);
+        for (ckfwi_model* L : lanes)
+            if (!L->xch.count(key9)) timed9.emplace_back(L, key9, r == 1);   // not another run's
+        rs = step2_time(lanes, t, r == 1, std::min(runs.s[r], m0->g.nt), st, e0, e1, &us);
+        if (verbose)
+            std::fprintf(stderr, "ckfwi batch autotune %s lanes %d ver %d tile %dx%d steps %d: %.1f us\n",
+                         r ? "adj" : "fwd", NL, t.ver, t.bx, t.zlen, runs.s[r], us);
+        best[r] = reps * us / 1000.0f;
+        (r ? bt.ta : bt.tf) = t;
+        (r ? bt.za : bt.zf).assign(NL, t.zlen);
+    }
     for (const Cand& c : cands) {
-        if (many[0] && many[1]) break;
+        if (rs != CKFWI_OK) break;
+        if (want[0] == 9 && want[1] == 9) break;
         long long total = 0;
         const std::vector<int> s = lane_starts(lanes, c.t, c.z, &total);
         if (total > 0x7fffffffLL) continue;
@@ -3216,8 +3336,7 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
         }
         for (int pass = 0; pass < 2 && rs == CKFWI_OK; ++pass) {
             if (pass == 1 && c.t.ver == 4) continue;    // generation 4 has no batched reverse step
-            if (many[pass]) continue;
-            if (want && c.t.ver != want && !(want == 4 && pass == 1 && c.t.ver == 3)) continue;
+            if (want[pass] && c.t.ver != want[pass] && !(want[pass] == 4 && pass == 1 && c.t.ver == 3)) continue;
             auto go = [&]() {
                 const BatchLaunch<FwdArgs> bf{ftab, dst.as<int>(), NL, dims, total};
                 const BatchLaunch<AdjArgs> ba{atab, dst.as<int>(), NL, dims, total};
@@ -3234,7 +3353,6 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
                 return pass == 0 ? launch_fwd_batch(bf, c.t, K, CK_NONE, st)
                                  : launch_adj_batch(ba, c.t, K, U_FP32, st);
             };
-            const int reps = 3;
             // the first candidate also brings the clocks up; then the median of three timings
             cudaError_t e = cudaSuccess;
             for (int r = 0; r < (warmed ? 1 : 20) && e == cudaSuccess; ++r) e = go();
@@ -3276,6 +3394,9 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, cudaStream_t st, const Ba
     cudaEventDestroy(e1);
     ST_TRY(rs);
     if (bt.zf.empty() || bt.za.empty()) return CKFWI_EINVAL;
+    // give back the exchange buffers of a form that was timed and not chosen
+    for (const auto& x : timed9)
+        if (std::get<2>(x) ? bt.ta.ver != 9 : bt.tf.ver != 9) std::get<0>(x)->xch.erase(std::get<1>(x));
     // the probes wrote into working buffers; clear them
     for (ckfwi_model* L : lanes) {
         for (DevMem* d : {L->work, L->lam})
@@ -3306,8 +3427,11 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
     for (int l = 0; l < NL; ++l) ST_TRY(set_shot(lanes[l], shots + l));
     const RunCfg rc = run_cfg(m0->g.nt, o);
     for (int l = 0; l < NL; ++l) ST_TRY(prepare_storage(lanes[l], rc, o));
+    std::vector<Action> acts;
+    long long cnt[3] = {rc.N - 1, 0, 0};
+    make_schedule(m0, rc, acts, cnt);
     const BatchTiles* bt = nullptr;
-    ST_TRY(batch_tune(lanes, st, &bt));
+    ST_TRY(batch_tune(lanes, run_steps(rc, acts), st, &bt));
     for (int l = 0; l < NL; ++l) {
         ST_TRY(prepare_states(lanes[l], rc, bt->tf, bt->ta));
         ST_TRY(step2_receivers(lanes[l], bt->tf));
@@ -3317,9 +3441,6 @@ int gradient_batch(const std::vector<ckfwi_model*>& lanes, const ckfwi_shot* sho
                                mem == CKFWI_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
         ST_TRY(reset_flags(L, st));
     }
-    std::vector<Action> acts;
-    long long cnt[3] = {rc.N - 1, 0, 0};
-    make_schedule(m0, rc, acts, cnt);
     Ctx cx{m0, st, 0};
     cx.mode = rc.mode;
     cx.lanes = lanes;
