@@ -267,15 +267,17 @@ struct DevInj {
 struct ShotDev {
     int nrec = 0;
     int nst = 0;
-    DevMem ridx, rwt, rzx, wavelet;
+    DevMem ridx, rwt, wavelet;
     DevInj src, adj;
     DevMem dsim, dobs, resid;
     std::vector<unsigned char> key;    // host description the maps were built from
-    std::vector<int2> first;           // 2D: every receiver's first point (z, x), as rzx holds them
-    // 2D: the receivers by tile of the launches of many steps (Step2Args), by
-    // tile shape; `made` is false once the receivers have changed
+    // 2D: every receiver's first point (z, x) and weights, and the receivers by
+    // tile of the launches of many steps (Step2Args) for each tile shape in
+    // use; `made` is false once the receivers have changed
+    std::vector<int2> first;
+    std::vector<float4> weights;
     struct ByTile {
-        DevMem list, start;
+        DevMem list, wt, start;
         bool made = false;
     };
     std::map<std::pair<int, int>, ByTile> by_tile;
@@ -589,12 +591,13 @@ int set_shot(ckfwi_model* m, const ckfwi_shot* s)
     ST_TRY(d.adj.set(build_inj(es)));
     if (g.dims == 2) {
         d.first.resize(s->nrec);
+        d.weights.resize(s->nrec);
         for (int r = 0; r < s->nrec; ++r) {
             const long long o = ridx[(size_t)r * nst];
+            const float* w = rw.data() + (size_t)r * nst;
             d.first[r] = make_int2((int)(o / f.pxy), (int)(o % f.pxy));
+            d.weights[r] = make_float4(w[0], w[1], w[2], w[3]);
         }
-        CK_TRY(d.rzx.alloc(d.first.size() * sizeof(int2), false));
-        CK_TRY(cudaMemcpy(d.rzx.p, d.first.data(), d.first.size() * sizeof(int2), cudaMemcpyHostToDevice));
         for (auto& t : d.by_tile) t.second.made = false;
     }
     CK_TRY(d.ridx.alloc(ridx.size() * sizeof(long long), false));
@@ -1293,7 +1296,8 @@ int step2_exchange(ckfwi_model* m, const Tile& t, bool reverse, Step2Args* a)
 // The shot's receivers by tile, for launches of many forward steps in tile t.
 // (A tile that sorts them out itself has to look at all of them: with 20000
 // on a line of 464 x 1104, 1500 a tile, in every step: 7.1 ms for 400 steps,
-// 3.4 ms with one step a launch.)
+// 3.4 ms with one step a launch.  Points and weights come in the tile's order
+// too, so that a warp reads them side by side.)
 int step2_receivers(ckfwi_model* m, const Tile& t)
 {
     if (t.ver != 9) return CKFWI_OK;
@@ -1302,14 +1306,22 @@ int step2_receivers(ckfwi_model* m, const Tile& t)
     const std::vector<int2>& at = m->shot.first;
     const int nbx = (m->fg.nx + t.bx - 1) / t.bx;
     auto tile = [&](const int2& p) { return (size_t)(p.x / t.zlen) * nbx + p.y / t.bx; };
-    std::vector<int> start((size_t)tiles_of(m->fg, t) + 1, 0), list(at.size());
+    std::vector<int> start((size_t)tiles_of(m->fg, t) + 1, 0);
     for (const int2& p : at) ++start[tile(p) + 1];
     for (size_t b = 1; b < start.size(); ++b) start[b] += start[b - 1];
     std::vector<int> next(start.begin(), start.end() - 1);
-    for (size_t r = 0; r < at.size(); ++r) list[next[tile(at[r])]++] = (int)r;
-    CK_TRY(bt.list.alloc(list.size() * sizeof(int), false));
+    std::vector<int2> list(at.size());
+    std::vector<float4> wt(at.size());
+    for (size_t r = 0; r < at.size(); ++r) {
+        const int k = next[tile(at[r])]++;
+        list[k] = make_int2(step2_place(m->K, t, at[r].x, at[r].y), (int)r);
+        wt[k] = m->shot.weights[r];
+    }
+    CK_TRY(bt.list.alloc(list.size() * sizeof(int2), false));
+    CK_TRY(bt.wt.alloc(wt.size() * sizeof(float4), false));
     CK_TRY(bt.start.alloc(start.size() * sizeof(int), false));
-    CK_TRY(cudaMemcpy(bt.list.p, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CK_TRY(cudaMemcpy(bt.list.p, list.data(), list.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    CK_TRY(cudaMemcpy(bt.wt.p, wt.data(), wt.size() * sizeof(float4), cudaMemcpyHostToDevice));
     CK_TRY(cudaMemcpy(bt.start.p, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice));
     bt.made = true;
     return CKFWI_OK;
@@ -1414,11 +1426,11 @@ int fwd_steps2(Ctx& cx, const Role& u, const Role& up, int n, int T, bool record
         }
         if (record) {
             a.smp = sample_of(m, n);
-            a.rzx = m->shot.rzx.as<int2>();
             const Tile& t = cx.tile(false);
             const ShotDev::ByTile& bt = m->shot.by_tile[std::make_pair(t.bx, t.zlen)];
             if (!bt.made) return CKFWI_EINVAL;
-            a.rlist = bt.list.as<int>();
+            a.rlist = bt.list.as<int2>();
+            a.rwt = bt.wt.as<float4>();
             a.rstart = bt.start.as<int>();
         }
         ST_TRY(step2_issue(cx, a, false));

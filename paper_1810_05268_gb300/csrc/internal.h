@@ -151,10 +151,10 @@ struct Step2Args {
     unsigned* epoch;      // and each tile's step count
     long long wait_limit; // looks at a neighbour's edge before giving up
     // forward
-    Sample smp;           // receivers: level n + i goes to out + i n
-    const int2* rzx;      // each receiver's first point (z, x)
-    const int* rlist;     // the receivers by tile (the one that holds their first point):
-    const int* rstart;    // tile b's are rlist[rstart[b]] .. rlist[rstart[b + 1] - 1]
+    Sample smp;           // receivers (n, out): level n + i goes to out + i n
+    const int2* rlist;    // the receivers by tile (the one that holds their first point): that point's
+    const float4* rwt;    // place in the staged tile and the receiver's index; and its four weights
+    const int* rstart;    // tile b's are entries rstart[b] .. rstart[b + 1] - 1
     // reverse
     Inj adj;              // step i takes series - i adj_stride
     long long adj_stride;
@@ -242,6 +242,7 @@ cudaError_t launch_adj3_batch(const BatchLaunch<AdjArgs>& b, const Tile& t, int 
 // stencil_2d.cu: many steps a launch (Tile.ver 9)
 bool step2_supported(int dims, int K, const Tile& t, bool reverse);
 size_t step2_exchange_bytes(int K, const Tile& t, long long tiles);
+int step2_place(int K, const Tile& t, int z, int x);   // of a grid point in its tile, as staged
 cudaError_t launch_step2(const Step2Args& a, const Tile& t, int K, bool reverse, cudaStream_t s);
 // the lanes' tiles (b.blocks) must be resident together
 cudaError_t launch_step2_batch(const BatchLaunch<Step2Args>& b, const Tile& t, int K, bool reverse, cudaStream_t s);

@@ -61,7 +61,6 @@ namespace {
 
 constexpr int NT2 = 512;                          // threads
 constexpr int NE2 = 256;                          // of them, the ones that compute edges and exchange them
-constexpr int RL2 = 512;                          // receivers of a tile listed in shared memory; the rest stay in the lane's list
 constexpr int SLOTS2 = 4;                         // exchange buffers in turn
 
 // columns a strip between x neighbours has, and the x margin of a staged
@@ -80,7 +79,7 @@ struct Tile2 {
     __host__ __device__ int own() const { return bx * bz; }
     __host__ size_t smem(bool reverse) const
     {
-        return (size_t)((reverse ? 4 : 2) * plane() + (reverse ? 2 : 1) * own() + bx + (bz + 3) / 4 * 4 + RL2) * 4;
+        return (size_t)((reverse ? 4 : 2) * plane() + (reverse ? 2 : 1) * own() + bx + (bz + 3) / 4 * 4) * 4;
     }
 };
 
@@ -584,31 +583,27 @@ __device__ __forceinline__ void fwd2_body(const Step2Args& a, int b, float* sm)
     float* w = b2 + t.plane();
     float* exs = w + t.own();
     float* ezs = exs + t.bx;
-    int* rl = reinterpret_cast<int*>(ezs + (t.bz + 3) / 4 * 4);
     const unsigned e0 = a.epoch[b];
     Step2Env<K> ev{b1, b2, w, ezs, exs, a.hdt, {}, false, pl.meets(a.src)};
 #pragma unroll
     for (int j = 0; j < K; ++j) ev.c[j] = a.c[j + 1];
     ev.damped = __syncthreads_or(stage_state<K>(ct, b1, b2, w, exs, ezs, a));
-    const int* list = a.smp.n > 0 ? a.rlist + a.rstart[b] : nullptr;
-    const int listed = a.smp.n > 0 ? a.rstart[b + 1] - a.rstart[b] : 0;
-    for (int k = tid; k < min(listed, RL2); k += NT2) rl[k] = list[k];
+    const int r0 = a.smp.n > 0 ? a.rstart[b] : 0, r1 = a.smp.n > 0 ? a.rstart[b + 1] : 0;
     cp_wait();
     __syncthreads();
     const int spos = (tid - NE2 - pl.in.n % NT2 + 2 * NT2) % NT2;    // the threads after those of the interior sample
     for (int i = 0; i < a.T; ++i) {
         // receivers of level n + i
-        auto sample = [&](int r) {
-            const int2 at = a.rzx[r];
-            const float* p = ev.b1 + (at.x - ct.zt + K) * t.pitch + at.y - ct.xt + ct.PX;
-            const float* wt = a.smp.wt + r * 4;
-            float acc = __fmaf_rn(wt[0], p[0], 0.0f);
-            acc = __fmaf_rn(wt[1], p[1], acc);
-            acc = __fmaf_rn(wt[2], p[t.pitch], acc);
-            acc = __fmaf_rn(wt[3], p[t.pitch + 1], acc);
-            a.smp.out[(long long)i * a.smp.n + r] = acc;
-        };
-        for (int k = spos; k < listed; k += NT2) sample(k < RL2 ? rl[k] : list[k]);
+        for (int k = r0 + spos; k < r1; k += NT2) {
+            const int2 at = __ldg(a.rlist + k);
+            const float4 wt = __ldg(a.rwt + k);
+            const float* p = ev.b1 + at.x;
+            float acc = __fmaf_rn(wt.x, p[0], 0.0f);
+            acc = __fmaf_rn(wt.y, p[1], acc);
+            acc = __fmaf_rn(wt.z, p[t.pitch], acc);
+            acc = __fmaf_rn(wt.w, p[t.pitch + 1], acc);
+            a.smp.out[(long long)i * a.smp.n + at.y] = acc;
+        }
         const bool last = i + 1 == a.T;
         const unsigned e = e0 + 1u + i;
         const bool out0 = i == 0 && goes_out(a, 0), out = goes_out(a, i + 1);
@@ -809,6 +804,11 @@ bool step2_supported(int dims, int K, const Tile& t, bool reverse)
     // neighbours hold each other's whole halo, and a row of vectors has a thread each
     if (t.bx < px2(K) || t.bx % 4 || t.by != 1 || t.vec != 4 || t.zlen < K || t.bx / 4 > 4096) return false;
     return Tile2(K, t.bx, t.zlen).smem(reverse) + sizeof(Step2Args) + 64 <= 227 * 1024;
+}
+
+int step2_place(int K, const Tile& t, int z, int x)
+{
+    return (K + z % t.zlen) * Tile2(K, t.bx, t.zlen).pitch + px2(K) + x % t.bx;
 }
 
 // bytes of a lane's exchange buffer for `tiles` tiles
