@@ -1682,9 +1682,8 @@ int autotune(ckfwi_model* m, cudaStream_t st, bool one_step = false)
             add((int)((f.nz + nzc - 1) / nzc));
         }
         // (an order-16 run of a 3D grid reads 16 planes beyond its own: short
-        // ones do not win where runs of 12 give every SM its four CTAs)
-        const bool longer = m->K > 4 && f.dims == 3 && cols * ((f.nz + 11) / 12) >= 4LL * nsm;
-        for (int z = longer ? 12 : 4; z <= 32; ++z) add(z);
+        // ones never win)
+        for (int z = m->K > 4 && f.dims == 3 ? 12 : 4; z <= 32; ++z) add(z);
         // 3D: columns cut into two to eight equal runs (the lean reverse step
         // of order 8 at 208^3, three CTAs an SM: 69.2 us at runs of 42, 71.9
         // at 21, the best below 33).  Rows of a 2D grid are too few columns
