@@ -185,8 +185,9 @@ typedef struct ckfwi_stats {
      * asynchronous copies, 5 / 6 the OT4 kernels (register-queue / vector-
      * blocked), 7 lean asynchronous copies, 8 fed by tensor copies (its
      * reverse step split in two launches), 9 many steps a launch (2D), 10
-     * the OT4 passes fed by tensor copies; and the tile (x points, y rows, x points per thread, z planes per CTA or,
-     * for generation 2, CTAs per SM, for generation 9, z rows) */
+     * the OT4 passes fed by tensor copies; and the tile (x points, y rows,
+     * x points per thread, z planes per CTA or, for generation 2, CTAs per
+     * SM, for generation 9, z rows) */
     int fwd_ver, fwd_bx, fwd_by, fwd_vec, fwd_zlen;
     int adj_ver, adj_bx, adj_by, adj_vec, adj_zlen;
     int fwd_pf, adj_pf;      /* generations 4 and 8: planes of prefetch (4: 0 = the

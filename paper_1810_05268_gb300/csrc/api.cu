@@ -907,12 +907,6 @@ Tile sampling_tile(const ckfwi_model* m, const Tile& t, const Role& u, const Rol
     return t;
 }
 
-int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by, CUtensorMap* out);
-
-// OT4 steps (ot4.cu): forward, the pass computing w lap f, then the update;
-// reverse, w lap of lam^j and u^{j-1}, the update, the gradient pass.  The
-// reverse step j writes w lap u^{j-1} into z4[1 + j % 2] and pairs the one
-// of step j + 1 with lap lam^j.
 // A pass fed by tensor copies: the staged field, then the point fields
 int ot4q_pass(ckfwi_model* m, int op, const Ot4qArgs& a, std::initializer_list<const float*> points, const Tile& t,
               int ck, cudaStream_t st)
@@ -943,6 +937,10 @@ int ot4q_update(ckfwi_model* m, const FwdArgs& a, const Tile& t, int ck, cudaStr
     return ot4q_pass(m, OT4Q_UPDATE, q, {a.u, a.up, a.w}, t, ck, st);
 }
 
+// OT4 steps (ot4.cu): forward, the pass computing w lap f, then the update;
+// reverse, w lap of lam^j and u^{j-1}, the update, the gradient pass.  The
+// reverse step j writes w lap u^{j-1} into z4[1 + j % 2] and pairs the one
+// of step j + 1 with lap lam^j.
 int ot4_fwd_step(ckfwi_model* m, const FwdArgs& a, const Tile& t, int ck, cudaStream_t st)
 {
     const FieldGeom& f = m->fg;
@@ -1041,8 +1039,6 @@ int ot4_adj_step(ckfwi_model* m, const AdjArgs& a, const Tile& t, int utype, int
     return CKFWI_OK;
 }
 
-// One forward step n of every lane: u -> out, optionally sampling d^n and
-// writing a fused takeshot (ck, ck_u, ck_up).
 // The six tensor maps of a split reverse step (launch_adjq): lam^j with the
 // u box, lam^{j+1} and w with point boxes, u^{j-1} with the u box, lam^{j-1}
 // and g with point boxes
@@ -1063,8 +1059,6 @@ int fwd_steps2(Ctx& cx, const Role& u, const Role& up, int n, int T, bool record
                int ck);
 int adj_steps2(Ctx& cx, const Role& l1, const Role& l2, const Role& o0, const Role& o1, const Role* us, const int* uts,
                int j, int T);
-
-int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by, CUtensorMap* out);
 
 // place (1, 2, ..) of a field's map in the context's table, as a row's tm
 // holds it before the upload; staged: with the u box, else a point box
@@ -1101,6 +1095,8 @@ void place_maps(std::vector<A>& rows, const CUtensorMap* base)
             if (p) p = base + (reinterpret_cast<size_t>(p) - 1);
 }
 
+// One forward step n of every lane: u -> out, optionally sampling d^n and
+// writing a fused takeshot (ck, ck_u, ck_up).
 int fwd_step(Ctx& cx, const Role& u, const Role& up, const Role& out, int n, bool record, int ck,
              const Role& ck_u, const Role& ck_up)
 {

@@ -46,8 +46,9 @@ __host__ __device__ inline Geo geo_of(const CodecView& v) { return make_geo(v.di
 // counter of finished compaction CTAs, the payload words of every group of
 // 1024 chunks and of every group of 32 chunks (accumulated by the encoder,
 // read and reset to zero by the compaction), each chunk's word count, the
-// blocks' bit sizes (16 bits each, whole chunks), and each chunk's staging slot of CW = 32 AREA words (first the blocks' own streams,
-// AREA words apart, then the chunk's bits assembled contiguously).
+// blocks' bit sizes (16 bits each, whole chunks), and each chunk's staging
+// slot of CW = 32 AREA words (first the blocks' own streams, AREA words
+// apart, then the chunk's bits assembled contiguously).
 struct ScratchLayout {
     long long g2, g1, counts, sizes, stage, words;
     int cw;

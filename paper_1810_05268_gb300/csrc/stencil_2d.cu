@@ -9,9 +9,9 @@
 // a launch advances up to STEP2_MAX steps.  The grid is cut into at most one
 // tile per SM; a CTA keeps its bz x bx tile of u^n, u^{n-1} and w (and a K
 // wide halo of u^n) in shared memory, and only the tiles' edges travel: each
-// step a CTA computes its edge points first, publishes them, computes the
-// interior while they travel, and takes its neighbours' edges as the next
-// halo.  (Tiles that recompute their halos, several steps deep, so that CTAs
+// step half of a CTA's threads compute its edge points and publish them while
+// the other half start on the interior, all share what is left of it, and the
+// neighbours' edges become the next halo.  (Tiles that recompute their halos, several steps deep, so that CTAs
 // never meet, were built first: 4.7 us a step at 464 x 1104, the redundant
 // points cost more than the exchange.)
 //
@@ -42,8 +42,8 @@
 // step's chain is an edge vector (about 1000 cycles: a lone warp issues an
 // instruction every 6 cycles), the exchange (1350 cycles between two CTAs
 // that do nothing else) and the interior beside it.  Two points a thread (1024
-// threads), edges strictly before the interior and the rare code out of line
-// were each slower.
+// threads), all edges before any interior (a barrier between them) and the rare
+// code out of line were each slower.
 //
 // What leaves a launch: the last two levels as the next state, any level that
 // a checkpoint takes (FP32, BF16 or FP16: u^s of one checkpoint, u^{s-1} of
@@ -524,8 +524,8 @@ __device__ __forceinline__ void step2(const Plan2<K>& pl, const Step2Env<K>& ev,
         if (send) ed.send(ct.slot(e), v, e);
         emit(ed.r, ed.q, win[K], v);
     }
-    // (Beside the interior the edges would share the issue slots with it and
-    // leave twice as late: 1900 cycles against 950 at 464 x 1104.)
+    // the interior: by the threads without edges while the others are at
+    // theirs; where it has more rows than those threads, all share what is left
     Rows2 pr = pl.in;
     if (pr.rp == 1) {
         if (pr.first() < pr.n) {                  // a row each: one round
