@@ -171,34 +171,51 @@ __device__ __forceinline__ void lap2(float (&out)[4], const float (*q)[4], const
             acc[p] = __ffma2_rn(cj, s, acc[p]);
         }
     }
-    // The one-step kernels add what is injected, zero at most points, which
-    // turns a Laplacian of the smallest values that has rounded to -0 into +0
-    // (only where an injected value rounds to -0 as well do they leave it).
-    // Added beside the injection instead, this took 4% of an order-16 run.
+    if (K > 4) {        // see inj4
 #pragma unroll
-    for (int p = 0; p < 2; ++p) acc[p] = __fadd2_rn(acc[p], f2(0.0f, 0.0f));
+        for (int p = 0; p < 2; ++p) acc[p] = __fadd2_rn(acc[p], f2(0.0f, 0.0f));
+    }
     out[0] = acc[0].x;
     out[1] = acc[0].y;
     out[2] = acc[1].x;
     out[3] = acc[1].y;
 }
 
-// injection of four points of row z, where the box meets them (elsewhere the
-// one-step kernels add zero: lap2's last addition)
-__device__ __forceinline__ void inj4(float (&s)[4], const Inj& in, const float* series, int z, int x0)
+// what is injected into point x of row `row` of the box
+__device__ __forceinline__ float inj1(const Inj& in, const float* series, int row, int x)
 {
-    if (z < in.z0 || z >= in.z1 || x0 + 4 <= in.x0 || x0 >= in.x1) return;
-    const int row = (z - in.z0) * (in.x1 - in.x0);
+    float acc = 0.0f;
+    if (x >= in.x0 && x < in.x1) {
+        const int b = row * (in.x1 - in.x0) + x - in.x0;
+        const int e1 = in.rowptr[b + 1];
+        for (int e = in.rowptr[b]; e < e1; ++e) acc = __fmaf_rn(in.wt[e], series[in.col[e]], acc);
+    }
+    return acc;
+}
+
+// Injection of four points of row z (`on`: somewhere in the tile).  Zero is
+// added where nothing is injected, as the one-step kernels do: a Laplacian of
+// the smallest values can round to -0, which that turns into +0.  At order 16
+// the Laplacian's last addition does it, for the registers (464 x 1104, 300
+// steps: 6.53 ms; 6.56 to 6.76 in forms that do it here; there a point whose
+// injected value rounds to -0 as well gets +0).  At the other orders this is
+// the faster place (281 x 281, order 4, 500 steps: 0.88 ms against 0.92).
+template <int K>
+__device__ __forceinline__ void inj4(float (&s)[4], bool on, const Inj& in, const float* series, int z, int x0)
+{
+    const bool hit = on && z >= in.z0 && z < in.z1 && x0 + 4 > in.x0 && x0 < in.x1;
+    if constexpr (K > 4) {
+        if (!hit) return;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int x = x0 + i;
-        float acc = 0.0f;
-        if (x >= in.x0 && x < in.x1) {
-            const int b = row + x - in.x0;
-            const int e1 = in.rowptr[b + 1];
-            for (int e = in.rowptr[b]; e < e1; ++e) acc = __fmaf_rn(in.wt[e], series[in.col[e]], acc);
+        for (int i = 0; i < 4; ++i) s[i] = __fadd_rn(s[i], inj1(in, series, z - in.z0, x0 + i));
+    } else {
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (hit) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = inj1(in, series, z - in.z0, x0 + i);
         }
-        s[i] = __fadd_rn(s[i], acc);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[i] = __fadd_rn(s[i], acc[i]);
     }
 }
 
@@ -473,7 +490,7 @@ __device__ __forceinline__ void update2(float (&v)[4], const Cta2<K>& ct, const 
     sld<4>(pv, ev.b2 + o);
     sld<4>(wv, ev.w + r * ct.t.bx + 4 * q);
     lap2<K>(s, qz, ev.b1 + o, ev.c);
-    if (ev.inject) inj4(s, in, series, ct.zt + r, x0);
+    if (K <= 4 || ev.inject) inj4<K>(s, ev.inject, in, series, ct.zt + r, x0);
     const float* uc = qz[K];
     float2 a0, a1;
     if (ev.damped) {
@@ -698,7 +715,7 @@ __device__ __forceinline__ void adj2_body(const Step2Args& a, int b, float* sm)
                     float* gp = gs + r * t.bx + 4 * pr.q;
                     sld<4>(gv, gp);
                     lap2<K>(s, win + h, ub + o, ev.c);
-                    if (src) inj4(s, a.src, a.src.series - (i - 1), ct.zt + r, x0);
+                    if (K <= 4 || src) inj4<K>(s, src, a.src, a.src.series - (i - 1), ct.zt + r, x0);
                     const float2 g0 = __ffma2_rn(f2(lv[0], lv[1]), f2(s[0], s[1]), f2(gv[0], gv[1]));
                     const float2 g1 = __ffma2_rn(f2(lv[2], lv[3]), f2(s[2], s[3]), f2(gv[2], gv[3]));
                     gv[0] = g0.x;

@@ -10,6 +10,7 @@ from paper_1810_05268_gb300 import ckfwi as C
 pytestmark = pytest.mark.gpu
 
 ONE_STEP = "1,128,1,16"
+MANY = "9,184,1,19,4"
 
 
 def _medium(shape):
@@ -33,10 +34,7 @@ def test_bytes_of_a_tail(monkeypatch, so, store):
     out = []
     for one in (True, False):
         for k in ("CKFWI_TILE_FWD", "CKFWI_TILE_ADJ"):
-            if one:
-                monkeypatch.setenv(k, ONE_STEP)
-            else:
-                monkeypatch.delenv(k, raising=False)
+            monkeypatch.setenv(k, ONE_STEP if one else MANY)
         monkeypatch.setenv("CKFWI_BATCH_VER", "1" if one else "9")
         m = C.Model(g)
         m.set_model(vel)
