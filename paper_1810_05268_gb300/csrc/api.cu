@@ -313,6 +313,10 @@ struct GraphExec {
 
 constexpr size_t MAX_GRAPHS = 8;   // recorded graphs kept per model
 constexpr long long WAIT_LIMIT = 1LL << 22;   // back-off rounds of a bounded wait in the kernels
+// 2D grids of fewer points take launches of many steps without being timed: a
+// step is then bound by latency alone (120 x 900, 130 steps, 4 checkpoints,
+// recorded: 2.13-2.55 ms by order, 2.37-2.70 with one step a launch)
+constexpr long long STEP2_SURE = 1LL << 18;
 
 // Tile shape and per-lane z-run lengths of a batch of lanes.
 struct BatchTiles {
@@ -379,6 +383,14 @@ struct ckfwi_model {
     Tile tf{}, ta{};
     Tile t1[2];                     // 2D: forward / reverse tile of one step a launch, beside launches of many (ver 9)
     bool tuned1 = false;
+    // 2D, in a recorded graph [us]: a launch of one step; a launch of many is
+    // `launch` + its steps x `step` (forward, reverse)
+    struct StepTimes {
+        float one = 0, launch = 0, step = 0;
+        bool fixed = true;          // many steps a launch without asking (a forced tile, a small grid)
+    };
+    StepTimes t2[2];
+    bool timed2 = false;
     Tile t4[5];                     // OT4 fed by tensor copies: the tile of each pass (ver 10 when tuned)
     bool tuned = false;
     int nparts = 128;
@@ -759,6 +771,7 @@ struct Ctx {
     Prof prof;
     long long count[PC_N] = {0, 0, 0, 0, 0};
     int mode = CKFWI_STORE_FP32;    // storage mode R_SLOT roles resolve for
+    bool one[2] = {false, false};   // forward / reverse steps by launches of one, where the model's are of many
     bool stage = false;             // FP32 host slots go through the device staging pairs
     bool pend[3] = {false, false, false};  // a copy from staging pair k to a host slot is in flight
     int sk = 0;                     // the staging pair the next host checkpoint takes
@@ -796,7 +809,10 @@ struct Ctx {
     Tile bf{}, ba{};                // batch tile shapes; z-run length per lane in zf / za
     std::vector<int> zf, za;
     // the tile of the forward / reverse steps; launches of several 2D steps take ver 9
-    const Tile& tile(bool reverse) const { return batch ? (reverse ? ba : bf) : (reverse ? m->ta : m->tf); }
+    const Tile& tile(bool reverse) const
+    {
+        return batch ? (reverse ? ba : bf) : one[reverse] ? m->t1[reverse] : (reverse ? m->ta : m->tf);
+    }
     bool several(bool reverse) const { return tile(reverse).ver == 9; }
     // the tile of a launch of one step
     const Tile& step_tile(bool reverse) const { return stage && several(reverse) ? m->t1[reverse] : tile(reverse); }
@@ -1238,8 +1254,9 @@ std::vector<int> step2_groups(const std::vector<ckfwi_model*>& lanes, const Tile
 // lanes costs a step of its own.  False when no tile fits: the grid is too
 // large for the SMs' shared memory, and the kernels of one step a launch are
 // the better ones there anyway (the step is then bound by its points, not by
-// its launch).
-bool step2_tile(const std::vector<ckfwi_model*>& lanes, bool reverse, Tile* out)
+// its launch).  near: tiles of other widths whose estimate is close to the
+// least one, at most ten, spread over the widths.
+bool step2_tile(const std::vector<ckfwi_model*>& lanes, bool reverse, Tile* out, std::vector<Tile>* near = nullptr)
 {
     const ckfwi_model* m = lanes[0];
     if (m->fg.dims != 2 || m->ot != 2) return false;
@@ -1253,6 +1270,7 @@ bool step2_tile(const std::vector<ckfwi_model*>& lanes, bool reverse, Tile* out)
     }
     const double per = 1.5 * (2 + m->K) / 6.0;   // cycles a vector
     double best = 1e30;
+    std::map<int, std::pair<double, Tile>> by_width;
     // the smallest tile of every number of columns and rows of the widest grid
     for (int cols = 1; cols <= nsm; ++cols)
         for (int rows = 1; rows * cols <= nsm; ++rows) {
@@ -1273,7 +1291,17 @@ bool step2_tile(const std::vector<ckfwi_model*>& lanes, bool reverse, Tile* out)
                 best = cost;
                 *out = t;
             }
+            auto& w = by_width.emplace(t.bx, std::make_pair(1e30, t)).first->second;
+            if (cost < w.first) w = std::make_pair(cost, t);
         }
+    if (near) {
+        std::vector<Tile> v;
+        for (const auto& w : by_width)
+            if (w.second.first <= 1.06 * best) v.push_back(w.second.second);
+        const size_t n = std::min<size_t>(v.size(), 10);
+        near->clear();
+        for (size_t i = 0; i < n; ++i) near->push_back(v[n > 1 ? i * (v.size() - 1) / (n - 1) : 0]);
+    }
     return best < 1e30;
 }
 
@@ -1647,6 +1675,75 @@ int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by
     return CKFWI_OK;
 }
 
+// the working fields, after runs that were only timed
+int clear_work(ckfwi_model* m, cudaStream_t st)
+{
+    for (DevMem* d : {m->work, m->lam})
+        for (int i = 0; i < 4 && d[i].p; ++i) CK_TRY(cudaMemsetAsync(d[i].p, 0, d[i].bytes, st));
+    CK_TRY(cudaMemsetAsync(m->gacc.p, 0, m->gacc.bytes, st));
+    return CKFWI_OK;
+}
+
+// One launch of T forward or reverse steps on the model's working fields, for
+// timing: T = 0 is a launch of one step in the tile of those (t1)
+int step2_probe(ckfwi_model* m, bool reverse, int T, cudaStream_t st)
+{
+    Ctx cx{m, st, 0};
+    cx.one[reverse] = T == 0;
+    if (T == 0 && !reverse) return fwd_step(cx, work_r(0), work_r(1), work_r(2), 0, false, CK_NONE, NONE_R, NONE_R);
+    if (T == 0) return adj_step(cx, lam_r(0), lam_r(1), lam_r(2), work_r(0), U_FP32, 1);
+    if (reverse) {
+        const std::vector<Role> us(T, work_r(0));
+        const std::vector<int> ut(T, U_FP32);
+        return adj_steps2(cx, lam_r(0), lam_r(1), lam_r(2), T > 1 ? lam_r(3) : NONE_R, us.data(), ut.data(), T, T);
+    }
+    Emits out{{T, work_r(2)}};
+    if (T > 1) out.emplace_back(T - 1, work_r(3));
+    return fwd_steps2(cx, work_r(0), work_r(1), 0, T, false, out, Emits(), CK_NONE);
+}
+
+// The tile of launches of many steps among those of nearly equal estimates.
+// The estimate does not see how a tile's edges spread over the threads and
+// the banks; on large tiles that decides: 800 x 1600, order 16, forward 13.8
+// us a step in tiles of 32 x 267, 8.3 in 124 x 73 (13.1 by one-step launches);
+// 700 x 1100, order 8, reverse 10.8 in 44 x 117, 7.6 in 184 x 28.
+int step2_tune(ckfwi_model* m, bool reverse, const std::vector<Tile>& tiles, cudaStream_t st, cudaEvent_t e0,
+               cudaEvent_t e1, bool verbose)
+{
+    Tile& own = reverse ? m->ta : m->tf;
+    const int T = std::min(16, m->g.nt);
+    Tile pick = own;
+    float best = 1e30f;
+    CK_TRY(cudaStreamSynchronize(st));
+    for (size_t i = 0; i < tiles.size(); ++i) {
+        own = tiles[i];
+        Step2Args x;
+        ST_TRY(step2_exchange(m, own, reverse, &x));        // allocated outside the timing
+        std::vector<float> v;
+        for (int round = i == 0 ? -8 : -1; round < 3; ++round) {    // the first runs bring the clocks up
+            CK_TRY(cudaEventRecord(e0, st));
+            ST_TRY(step2_probe(m, reverse, T, st));
+            CK_TRY(cudaEventRecord(e1, st));
+            CK_TRY(cudaEventSynchronize(e1));
+            float ms = 0;
+            CK_TRY(cudaEventElapsedTime(&ms, e0, e1));
+            if (round >= 0) v.push_back(ms);
+        }
+        std::sort(v.begin(), v.end());
+        if (verbose)
+            std::fprintf(stderr, "ckfwi 2D autotune %s tile %dx%d: %.2f us a step\n", reverse ? "adj" : "fwd", own.bx,
+                         own.zlen, 1000.0f * v[1] / (float)T);
+        if (v[1] < best) {
+            best = v[1];
+            pick = own;
+        }
+    }
+    for (const Tile& t : tiles)
+        if (t.bx != pick.bx || t.zlen != pick.zlen) m->xch.erase(std::make_tuple(t.bx, t.zlen, reverse ? 1 : 0));
+    own = pick;
+    return CKFWI_OK;
+}
+
 // --------------------------------------------------------------- autotune
 // (one_step: the tiles of one step a launch where the model's are of many)
 int autotune(ckfwi_model* m, cudaStream_t st, bool one_step = false)
@@ -1849,13 +1946,18 @@ int autotune(ckfwi_model* m, cudaStream_t st, bool one_step = false)
     bool ff = one_step ? m->tf.ver != 9 : forced("CKFWI_TILE_FWD", &tf, false);
     bool fa = one_step ? m->ta.ver != 9 : forced("CKFWI_TILE_ADJ", &ta, true);
     forced("CKFWI_TILE_OT4_LAP", &m->t4[OT4Q_LAP], false);   // pass 1 of an OT4 step, as tuning leaves it
-    // a 2D grid that fits the SMs takes the kernels of many steps a launch:
-    // nothing to time (281 x 281 and 464 x 1104: 1.5 and 3.1 us a forward
+    // a 2D grid that fits the SMs takes the kernels of many steps a launch; in
+    // a small one there is nothing to time (281 x 281 and 464 x 1104: 1.5 and 3.1 us a forward
     // step, against 3.3 and 5.1 us of kernel time for one step a launch, and
     // 6.3 us when the host launches it)
-    ff = ff || (!one_step && step2_tile({m}, false, &tf));
-    fa = fa || (!one_step && step2_tile({m}, true, &ta));
     const bool verbose = std::getenv("CKFWI_VERBOSE") != nullptr;
+    for (bool reverse : {false, true}) {
+        std::vector<Tile> near;
+        bool& found = reverse ? fa : ff;
+        if (found || one_step || !step2_tile({m}, reverse, reverse ? &ta : &tf, &near)) continue;
+        found = true;
+        if (f.npts >= STEP2_SURE && near.size() > 1) ST_TRY(step2_tune(m, reverse, near, st, e0, e1, verbose));
+    }
     // time one candidate: the median of `rounds` timings of `reps` launches
     auto time_of = [&](const Tile& t, int pass, int rounds, float* out) -> int {
         std::vector<float> v;
@@ -1958,10 +2060,7 @@ int autotune(ckfwi_model* m, cudaStream_t st, bool one_step = false)
     Step2Args x2;
     if (tf.ver == 9) ST_TRY(step2_exchange(m, tf, false, &x2));
     if (ta.ver == 9) ST_TRY(step2_exchange(m, ta, true, &x2));
-    // the probe runs wrote into working buffers; clear them
-    for (DevMem* d : {m->work, m->lam})
-        for (int i = 0; i < 4 && d[i].p; ++i) CK_TRY(cudaMemsetAsync(d[i].p, 0, d[i].bytes, st));
-    CK_TRY(cudaMemsetAsync(m->gacc.p, 0, m->gacc.bytes, st));
+    ST_TRY(clear_work(m, st));
     for (int i = 0; i < 3; ++i)
         if (m->z4[i].p) CK_TRY(cudaMemsetAsync(m->z4[i].p, 0, m->z4[i].bytes, st));
     CK_TRY(cudaStreamSynchronize(st));
@@ -2845,7 +2944,7 @@ void fill_stats(ckfwi_stats* stats, Ctx& cx, const RunCfg& rc, const long long* 
                 const FieldGeom& f)
 {
     std::memset(stats, 0, sizeof(*stats));
-    const Tile tf = cx.batch ? cx.bf : cx.m->tf, ta = cx.batch ? cx.ba : cx.m->ta;
+    const Tile tf = cx.tile(false), ta = cx.tile(true);
     stats->fwd_ver = tf.ver;
     stats->fwd_bx = tf.bx;
     stats->fwd_by = tf.by;
@@ -2922,6 +3021,132 @@ void make_schedule(const ckfwi_model* m, const RunCfg& rc, std::vector<Action>& 
         revolve_schedule(rc.N, rc.M, acts, cnt);
 }
 
+// What a schedule asks of launches of many 2D steps, forward and reverse: its
+// steps, the launches its runs take (forward steps past checkpoints, reverse
+// steps of states that need no recomputation), and the steps of an average
+// launch as a power of two from below
+struct RunSteps {
+    long long steps[2], launches[2];
+    int s[2];
+};
+RunSteps run_steps(const RunCfg& rc, const std::vector<Action>& acts)
+{
+    RunSteps rs{{0, 0}, {0, 0}, {1, 1}};
+    const int most[2] = {STEP2_MAX, rc.codec ? CODEC_NF : STEP2_MAX};
+    auto run = [&](int r, long long len) {
+        rs.steps[r] += len;
+        rs.launches[r] += (len + most[r] - 1) / most[r];
+    };
+    if (rc.store_all) run(0, rc.N), run(1, rc.N);
+    for (size_t i = 0; i < acts.size(); ++i) {
+        long long len = 0;
+        if (acts[i].op == ACT_ADVANCE) {
+            for (; i < acts.size() && (acts[i].op == ACT_ADVANCE || acts[i].op == ACT_TAKESHOT); ++i)
+                if (acts[i].op == ACT_ADVANCE) len += acts[i].b;
+            --i;
+            run(0, len);
+        } else if (acts[i].op == ACT_YOUTURN) {
+            for (len = 1; i + 2 < acts.size() && acts[i + 1].op == ACT_RESTORE && acts[i + 2].op == ACT_YOUTURN; i += 2) ++len;
+            run(1, len);
+        }
+    }
+    for (int r = 0; r < 2; ++r)
+        while (rs.launches[r] > 0 && 2LL * rs.s[r] * rs.launches[r] <= rs.steps[r]) rs.s[r] *= 2;
+    return rs;
+}
+
+// Time [us] of one of `reps` launches in a recorded graph
+template <class F>
+int graph_time(ckfwi_model* m, int reps, F&& launch, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, float* us)
+{
+    if (!m->cap) CK_TRY(cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
+    cudaGraph_t gr = nullptr;
+    cudaGraphExec_t ex = nullptr;
+    CK_TRY(cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeRelaxed));
+    int rs = CKFWI_OK;
+    for (int k = 0; k < reps && rs == CKFWI_OK; ++k) rs = launch();
+    cudaError_t e = cudaStreamEndCapture(m->cap, &gr);
+    if (rs == CKFWI_OK) rs = cuda_status_or_ok(e);
+    if (rs == CKFWI_OK) rs = cuda_status_or_ok(cudaGraphInstantiate(&ex, gr, 0));
+    if (gr) cudaGraphDestroy(gr);
+    std::vector<float> v;
+    for (int round = 0; round < 4 && rs == CKFWI_OK; ++round) {      // the first is not counted
+        float ms = 0;
+        e = cudaEventRecord(e0, st);
+        if (e == cudaSuccess) e = cudaGraphLaunch(ex, st);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        rs = cuda_status_or_ok(e);
+        if (round > 0) v.push_back(ms);
+    }
+    if (ex) cudaGraphExecDestroy(ex);
+    ST_TRY(rs);
+    std::sort(v.begin(), v.end());
+    *us = 1000.0f * v[1] / (float)reps;
+    return CKFWI_OK;
+}
+
+// The times behind step2_choose, of zero steps on the model's working fields
+int step2_times(ckfwi_model* m, cudaStream_t st)
+{
+    if (m->timed2) return CKFWI_OK;
+    const bool many[2] = {m->tf.ver == 9, m->ta.ver == 9};
+    const char* const force[2] = {"CKFWI_TILE_FWD", "CKFWI_TILE_ADJ"};
+    for (int r = 0; r < 2; ++r) m->t2[r].fixed = !many[r] || m->fg.npts < STEP2_SURE || std::getenv(force[r]);
+    if (!m->t2[0].fixed || !m->t2[1].fixed) {
+        ST_TRY(autotune(m, st, true));
+        cudaEvent_t e0, e1;
+        CK_TRY(cudaEventCreate(&e0));
+        CK_TRY(cudaEventCreate(&e1));
+        int rs = cuda_status_or_ok(cudaStreamSynchronize(st));
+        for (int r = 0; r < 2 && rs == CKFWI_OK; ++r) {
+            if (m->t2[r].fixed) continue;
+            const int T = std::min(16, m->g.nt);
+            float one = 0, t1 = 0, tT = 0;
+            rs = graph_time(m, 32, [&] { return step2_probe(m, r == 1, 0, m->cap); }, st, e0, e1, &one);
+            if (rs == CKFWI_OK) rs = graph_time(m, 32, [&] { return step2_probe(m, r == 1, 1, m->cap); }, st, e0, e1, &t1);
+            if (rs == CKFWI_OK) rs = graph_time(m, 8, [&] { return step2_probe(m, r == 1, T, m->cap); }, st, e0, e1, &tT);
+            m->t2[r].one = one;
+            m->t2[r].step = T > 1 ? std::max(0.0f, tT - t1) / (float)(T - 1) : t1;
+            m->t2[r].launch = t1 - m->t2[r].step;
+            if (std::getenv("CKFWI_VERBOSE"))
+                std::fprintf(stderr, "ckfwi 2D %s steps: one a launch %.2f us; many: %.2f us a launch, %.2f a step\n",
+                             r ? "adj" : "fwd", one, m->t2[r].launch, m->t2[r].step);
+        }
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        ST_TRY(rs);
+        ST_TRY(clear_work(m, st));
+        CK_TRY(cudaStreamSynchronize(st));
+    }
+    m->timed2 = true;
+    return CKFWI_OK;
+}
+
+// Forward and reverse steps of a recorded 2D gradient: launches of many where
+// they fit, unless the schedule's steps take less time one a launch.  A
+// launch of many moves the state into the tiles and out of them, so runs of a
+// few steps (few checkpoints) can be the one-step kernels', whose launches
+// cost little in a graph: 464 x 1104, order 4, 130 steps, 4 checkpoints: 3.27
+// ms by launches of many, 2.92 by launches of one, 2.44 with the reverse steps
+// by launches of one.  (Launched from the host one at a time these cost more
+// than their time, and many a launch was the faster form at every size:
+// nothing is timed there.)  Compressed and 16-bit states are decoded together,
+// or read where they lie, by launches of many, and one by one, in launches of
+// their own, for the others: reverse steps of those stay launches of many
+// (codec, 464 x 1104, order 4, 20 checkpoints: 3.89 ms; 4.42).
+int step2_choose(ckfwi_model* m, const RunCfg& rc, const RunSteps& rs, cudaStream_t st, bool one[2])
+{
+    ST_TRY(step2_times(m, st));
+    for (int r = 0; r < 2; ++r) {
+        const ckfwi_model::StepTimes& t = m->t2[r];
+        if (r == 1 && rc.mode != CKFWI_STORE_FP32) continue;
+        one[r] = !t.fixed && t.one * (double)rs.steps[r] < t.launch * (double)rs.launches[r] + t.step * (double)rs.steps[r];
+    }
+    return CKFWI_OK;
+}
+
 int gradient_one(ckfwi_model* m, const ckfwi_shot* s, const float* d_obs, int mem,
                  const ckfwi_grad_opts* o, double* misfit, ckfwi_stats* stats, cudaStream_t st)
 {
@@ -2933,27 +3158,28 @@ int gradient_one(ckfwi_model* m, const ckfwi_shot* s, const float* d_obs, int me
     const FieldGeom& f = m->fg;
     const RunCfg rc = run_cfg(m->g.nt, o);
     ST_TRY(prepare_storage(m, rc, o));
-    ST_TRY(prepare_states(m, rc, m->tf, m->ta));
-    ST_TRY(step2_receivers(m, m->tf));
+    std::vector<Action> acts;
+    long long cnt[3] = {rc.N - 1, 0, 0};
+    make_schedule(m, rc, acts, cnt);
     // staged host slots: a step that makes a checkpoint and every reverse step
     // is a launch of its own, and a launch of one step is better the one-step
     // kernels' (the many-step ones move the state in and out of the tiles for
     // it: 464 x 1104, 300 steps, half of 20 slots on the host: 7.9 ms with
     // them alone, 5.2 with one-step launches alone, 4.9 with both)
     const bool stage = rc.mode == CKFWI_STORE_FP32 && !rc.codec && !rc.store_all && m->host_slots > 0 && m->side;
+    const bool graph = o->use_graph != 0 && !o->profile;
+    Ctx cx{m, st, 0};
+    cx.mode = rc.mode;
+    cx.stage = stage;
     if (stage && (m->tf.ver == 9 || m->ta.ver == 9)) ST_TRY(autotune(m, st, true));
+    else if (graph && (m->tf.ver == 9 || m->ta.ver == 9)) ST_TRY(step2_choose(m, rc, run_steps(rc, acts), st, cx.one));
+    ST_TRY(prepare_states(m, rc, cx.tile(false), cx.tile(true)));
+    ST_TRY(step2_receivers(m, cx.tile(false)));
     const size_t nd = (size_t)(rc.N + 1) * m->shot.nrec;
     CK_TRY(cudaMemcpyAsync(m->shot.dobs.p, d_obs, nd * sizeof(float),
                            mem == CKFWI_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
     ST_TRY(reset_flags(m, st));
-    std::vector<Action> acts;
-    long long cnt[3] = {rc.N - 1, 0, 0};
-    make_schedule(m, rc, acts, cnt);
-    Ctx cx{m, st, 0};
-    cx.mode = rc.mode;
-    cx.stage = stage;
     long long counters[2] = {0, 0};
-    const bool graph = o->use_graph != 0 && !o->profile;
     if (o->profile) {
         cx.prof.on = true;
         cx.prof.pool = &m->evpool;
@@ -3057,39 +3283,6 @@ std::vector<long long> lane_ids(const std::vector<ckfwi_model*>& lanes, bool wit
         if (with_gen) v.push_back(L->gen);
     }
     return v;
-}
-
-// Steps of an average launch of many 2D steps, forward and reverse, in a
-// schedule: its steps over its runs (forward steps past checkpoints, reverse
-// steps of states that need no recomputation), as a power of two from below
-struct RunSteps {
-    int s[2];
-};
-RunSteps run_steps(const RunCfg& rc, const std::vector<Action>& acts)
-{
-    long long steps[2] = {0, 0}, launches[2] = {0, 0};
-    const int most[2] = {STEP2_MAX, rc.codec ? CODEC_NF : STEP2_MAX};
-    auto run = [&](int r, long long len) {
-        steps[r] += len;
-        launches[r] += (len + most[r] - 1) / most[r];
-    };
-    if (rc.store_all) run(0, rc.N), run(1, rc.N);
-    for (size_t i = 0; i < acts.size(); ++i) {
-        long long len = 0;
-        if (acts[i].op == ACT_ADVANCE) {
-            for (; i < acts.size() && (acts[i].op == ACT_ADVANCE || acts[i].op == ACT_TAKESHOT); ++i)
-                if (acts[i].op == ACT_ADVANCE) len += acts[i].b;
-            --i;
-            run(0, len);
-        } else if (acts[i].op == ACT_YOUTURN) {
-            for (len = 1; i + 2 < acts.size() && acts[i + 1].op == ACT_RESTORE && acts[i + 2].op == ACT_YOUTURN; i += 2) ++len;
-            run(1, len);
-        }
-    }
-    RunSteps rs{{1, 1}};
-    for (int r = 0; r < 2; ++r)
-        while (launches[r] > 0 && 2LL * rs.s[r] * launches[r] <= steps[r]) rs.s[r] *= 2;
-    return rs;
 }
 
 // Time of one step [us] of every lane in launches of T 2D steps, on the lanes'
@@ -3407,12 +3600,7 @@ int batch_tune(const std::vector<ckfwi_model*>& lanes, const RunSteps& runs, cud
     // give back the exchange buffers of a form that was timed and not chosen
     for (const auto& x : timed9)
         if (std::get<2>(x) ? bt.ta.ver != 9 : bt.tf.ver != 9) std::get<0>(x)->xch.erase(std::get<1>(x));
-    // the probes wrote into working buffers; clear them
-    for (ckfwi_model* L : lanes) {
-        for (DevMem* d : {L->work, L->lam})
-            for (int i = 0; i < 4 && d[i].p; ++i) CK_TRY(cudaMemsetAsync(d[i].p, 0, d[i].bytes, st));
-        CK_TRY(cudaMemsetAsync(L->gacc.p, 0, L->gacc.bytes, st));
-    }
+    for (ckfwi_model* L : lanes) ST_TRY(clear_work(L, st));
     CK_TRY(cudaStreamSynchronize(st));
     auto ins = m0->btiles.emplace(key, std::move(bt)).first;
     *out = &ins->second;
