@@ -409,7 +409,8 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const __
     __shared__ uint32_t xtra[ENC_THREADS / 32][4];
     int fld;
     const CodecLane& A = item_of(call, fld);
-    const Geo G = geo_of(A.v);
+    const CodecView v = A.v;
+    const Geo G = geo_of(v);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const long long b = (long long)blockIdx.x * ENC_THREADS + threadIdx.x;
     const long long c = b / CHUNK;
@@ -419,7 +420,7 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const __
     uint32_t* stage = scratch + L.stage + c * L.cw;
     uint32_t* gs = stage + (b % CHUNK) * MW;
     int nbits = 0;
-    if (b < G.nblocks) nbits = encode_block<DIMS>(A.f[call.src[fld]], A.v, G, call.tol_f, b, colw + threadIdx.x, gs, A.err);
+    if (b < G.nblocks) nbits = encode_block<DIMS>(A.f[call.src[fld]], v, G, call.tol_f, b, colw + threadIdx.x, gs, A.err);
     reinterpret_cast<uint16_t*>(scratch + L.sizes)[b] = (uint16_t)nbits;    // 0 past the last block
     __syncwarp();
     int incl = nbits;
@@ -438,14 +439,24 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const __
     for (int k = lane; k < words; k += 32) *bufw(k) = 0u;
     __syncwarp();
     const int sw = (nbits + 31) / 32;
-    for (int k = 0; k < sw; ++k) {
-        uint32_t val = gs[k];
-        const int rem = nbits - 32 * k;
-        if (rem < 32) val &= (1u << rem) - 1u;
-        const int pos = off + 32 * k;
-        const int sh = pos & 31, idx = pos >> 5;
-        atomicOr(bufw(idx), val << sh);
-        if (sh) atomicOr(bufw(idx + 1), val >> (32 - sh));
+    // (four loads before the atomics that take them: the compiler keeps a load
+    // behind an atomic that could be to the same memory)
+    for (int k0 = 0; k0 < sw; k0 += 4) {
+        uint32_t t[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = k0 + i < sw ? gs[k0 + i] : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = k0 + i;
+            if (k >= sw) break;
+            uint32_t val = t[i];
+            const int rem = nbits - 32 * k;
+            if (rem < 32) val &= (1u << rem) - 1u;
+            const int pos = off + 32 * k;
+            const int sh = pos & 31, idx = pos >> 5;
+            atomicOr(bufw(idx), val << sh);
+            if (sh) atomicOr(bufw(idx + 1), val >> (32 - sh));
+        }
     }
     // every block's stream has been read: the slot takes the assembled chunk
     __syncwarp();
@@ -468,13 +479,16 @@ __global__ void __launch_bounds__(ENC_THREADS, ENC_MIN_CTAS) enc_kernel(const __
 // counter, no waiting) sets them back to zero for the next compression.
 // Small CTAs spread the copy over every SM; eight chunks are what the threads
 // copy the sizes of at once (four chunks: an inversion iteration over 2D
-// fields took 484 ms, now 473).
+// fields took 484 ms, now 473).  Twelve CTAs an SM (40 registers; 72 without
+// the bound).  What bounds it is the latency of its copies: a rough field of
+// 300 x 400 x 400 at ratio 1.9 takes 53 us, 63 at 72 registers, 118 with one
+// load in flight a thread; a smooth one at ratio 9 takes 22, 25 and 35.
 constexpr int CMP_THREADS = 128;
 constexpr int CPB = 8;
 static_assert(CPB * CHUNK / 2 <= CMP_THREADS, "a thread copies one word of sizes");
 
 template <int DIMS>
-__global__ void __launch_bounds__(CMP_THREADS) compact_kernel(const __grid_constant__ CodecCall call)
+__global__ void __launch_bounds__(CMP_THREADS, 12) compact_kernel(const __grid_constant__ CodecCall call)
 {
     constexpr int NW = CMP_THREADS / 32;
     __shared__ long long red[3][NW];
@@ -585,16 +599,26 @@ __global__ void __launch_bounds__(CMP_THREADS) compact_kernel(const __grid_const
         if (threadIdx.x < CPB * CHUNK / 2 && w < (G.nblocks + 1) / 2) hdr[HDR + G.nchunks + w] = scratch[L.sizes + w];
     }
     // the CTA's chunks are contiguous in the payload: every thread copies
-    // words of them (all loads independent, so their latencies overlap)
+    // words of them, four loads before their stores (the compiler has to
+    // assume that payload and staging overlap and would keep each load behind
+    // the store before it)
     const uint32_t gw = offs[CPB];
     uint32_t* payload = hdr + G.table_words + prefix;
     const uint32_t* stage = scratch + L.stage + c0 * L.cw;
-    for (uint32_t w = threadIdx.x; w < gw; w += CMP_THREADS) {
-        int lo = 0;
+    for (uint32_t w0 = threadIdx.x; w0 < gw; w0 += 4 * CMP_THREADS) {
+        uint32_t v[4];
 #pragma unroll
-        for (int k = 1; k < CPB; ++k)
-            if (offs[k] <= w) lo = k;
-        payload[w] = stage[(long long)lo * L.cw + (w - offs[lo])];
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t w = w0 + i * CMP_THREADS;
+            int lo = 0;
+#pragma unroll
+            for (int k = 1; k < CPB; ++k)
+                if (offs[k] <= w) lo = k;
+            v[i] = w < gw ? stage[(long long)lo * L.cw + (w - offs[lo])] : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (w0 + i * CMP_THREADS < gw) payload[w0 + i * CMP_THREADS] = v[i];
     }
 }
 
