@@ -37,13 +37,14 @@
 // overwrites u^{n-1} point by point.
 //
 // Measured, from set_model to the data on one GB300: 281 x 281, 500 steps
-// 3.21 -> 0.97 ms (1.5 us a step, a reverse step 2.7); 464 x 1104, 2000 steps
-// 12.5 -> 6.4 ms (3.1 and 6.5).  What bounds it: a
-// step's chain is an edge vector (about 1000 cycles: a lone warp issues an
-// instruction every 6 cycles), the exchange (1350 cycles between two CTAs
-// that do nothing else) and the interior beside it.  Two points a thread (1024
-// threads), all edges before any interior (a barrier between them) and the rare
-// code out of line were each slower.
+// 3.22 -> 0.95 ms (1.5 us a step, a reverse step 2.7); 464 x 1104, 2000 steps
+// 12.5 -> 5.9 ms (2.9 and 4.8; lanes of a batch, whose tile is the least
+// estimate's, 3.1 and 6.5).  What bounds it: a step's chain is an edge vector
+// (about 1000 cycles: a lone warp issues an instruction every 6 cycles), the
+// exchange (1350 cycles between two CTAs that do nothing else) and the
+// interior beside it.  Two points a thread (1024 threads), all edges before
+// any interior (a barrier between them) and the rare code out of line were
+// each slower.
 //
 // What leaves a launch: the last two levels as the next state, any level that
 // a checkpoint takes (FP32, BF16 or FP16: u^s of one checkpoint, u^{s-1} of
