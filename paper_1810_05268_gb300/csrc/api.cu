@@ -1675,6 +1675,17 @@ int tensor_map(ckfwi_model* m, const void* origin_ptr, int utype, int bx, int by
     return CKFWI_OK;
 }
 
+// the exchange buffers and step counts of 2D launches: a launch that gave up
+// leaves its tiles at different steps
+int clear_exchange(ckfwi_model* m, cudaStream_t st)
+{
+    for (auto& x : m->xch) {
+        CK_TRY(cudaMemsetAsync(x.second.buf.p, 0, x.second.buf.bytes, st));
+        CK_TRY(cudaMemsetAsync(x.second.epoch.p, 0, x.second.epoch.bytes, st));
+    }
+    return CKFWI_OK;
+}
+
 // the working fields, after runs that were only timed
 int clear_work(ckfwi_model* m, cudaStream_t st)
 {
@@ -1741,7 +1752,7 @@ int step2_tune(ckfwi_model* m, bool reverse, const std::vector<Tile>& tiles, cud
     for (const Tile& t : tiles)
         if (t.bx != pick.bx || t.zlen != pick.zlen) m->xch.erase(std::make_tuple(t.bx, t.zlen, reverse ? 1 : 0));
     own = pick;
-    return CKFWI_OK;
+    return clear_exchange(m, st);     // should a wait have run out
 }
 
 // --------------------------------------------------------------- autotune
@@ -2099,13 +2110,9 @@ int read_flags(ckfwi_model* m, cudaStream_t st, int* fl)
     else if (h[1] & 4) *fl = CKFWI_CORRUPT;
     else if (h[0] & 8) *fl = CKFWI_TIMEOUT;
     else if ((h[0] & 1) || (h[1] & 1)) *fl = CKFWI_NONFINITE;
-    // a launch of many steps that gave up leaves its tiles at different steps
     // (waited for: the next call may come on any stream)
     if (h[0] & 8) {
-        for (auto& x : m->xch) {
-            CK_TRY(cudaMemsetAsync(x.second.buf.p, 0, x.second.buf.bytes, st));
-            CK_TRY(cudaMemsetAsync(x.second.epoch.p, 0, x.second.epoch.bytes, st));
-        }
+        ST_TRY(clear_exchange(m, st));
         CK_TRY(cudaStreamSynchronize(st));
     }
     return CKFWI_OK;
@@ -3118,6 +3125,7 @@ int step2_times(ckfwi_model* m, cudaStream_t st)
         cudaEventDestroy(e1);
         ST_TRY(rs);
         ST_TRY(clear_work(m, st));
+        ST_TRY(clear_exchange(m, st));
         CK_TRY(cudaStreamSynchronize(st));
     }
     m->timed2 = true;
